@@ -68,7 +68,10 @@ k_step_batch(const BatchCavity<R>* __restrict__ cav, const BatchItem* __restrict
         S* d = dst + off;
         if (w.kind == 0) {
             const int x = w.a + tx, y = w.b + ty;
-            if (x < ks.nx && y < ks.ny && !is_wall(ks, x, y)) interior_update(ks, s, d, x, y, step);
+            if (x < ks.nx && y < ks.ny && !is_wall(ks, x, y)) {
+                if (ks.omf == R(0) && ks.omT == R(0)) interior_update<R, S, false, true>(ks, s, d, x, y, step);
+                else interior_update<R, S, false, false>(ks, s, d, x, y, step);
+            }
         } else if ((int)threadIdx.x < w.b) {
             int x, y;
             perimeter_node(ks, w.a + (int)threadIdx.x, x, y);

@@ -63,6 +63,22 @@ __host__ __device__ constexpr R w_of(int i) {
 enum : int { BC_PERIODIC = 0, BC_DIRICHLET = 1, BC_ADIABATIC = 2 };
 enum : int { SW = 0, SE = 1, SS = 2, SN = 3 };
 
+// Porosity-dependent constants of the node update (lbm_core.cuh): e the
+// porosity, itf, itT = 1/tau, a = 1.5 itf rho0 A invD the share of S in Q.
+template <class V>
+struct Cell {
+    V eps, ie;         // e, 1/e
+    V eg, eax, heax;   // e g beta, e a_x, e a_x / 2
+    V c0, c0sq, c1;    // quadratic solve (Sec. 3.1)
+    V ih, il, ci;      // 1/(2 c0) and its rounding error, -c1/(2 c0)
+    V nnuK, nFK;       // - e nu/K, - e F_e/sqrt(K)
+    V e2, e3;          // e p = e1 sum f + e2 u.F + e3 |u|^2
+    V re;              // rho0 / e
+    V qu, qF;          // of u u and u F in Q, S folded in: cu2 - a re, cuF + a re
+    V cu2, cuF;        // the same with S apart: 4.5 itf rho0/e, 9 rho0 (1 - 1/2tau_f)/e
+    V b, nb, ug, kc;   // (1/e - 1/sigma)/2, -b, 6 (1 - 1/2tau_T) b, 4.5 itT/e
+};
+
 // Constants of one run in the compute type R (filled on the host).
 template <class R>
 struct KConst {
@@ -96,11 +112,14 @@ struct KConst {
     R p_pref_eps;          // c_s^2 / (1 - w_0)
     int da_inf, forch;
     const R* ay_row;       // extra external acceleration a_y per row, or nullptr
-    // constants of the interior fast path (see interior_update)
-    R inv_rho0, half_eps_ax, half_eps, p_uF, p_uu;
-    R fA_ep, fA_uu, fA_tr, fA_uF, f_cu2, f_ScS, f_cucF, f_cu, f_cF;
-    R h_sig, h_uu, h_pT, h_kQ, h_cu2, h_u3, h_ug, h_uQ, h_g, h_W;
-    R h0_sig, h0_uu, h0_pT, h0_kQ;
+    // constants of the node update (lbm_core.cuh): those of the uniform
+    // porosity, and the factors that give a porosity field's
+    Cell<R> cell;
+    R inv_rho0, hq_sigma, half_Q, eay, half_ax;      // 1/rho0, Q/(2 sigma), Q/2, eps a_y, a_x/2
+    R nnuK_q2, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie;
+    R a_ep, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF, gain;
+    R h_sig, h_kQ, h_pT, h0_pT, h_u3, h_uQ, h_g, h_W, h_Wr;
+    R u_abs[4];            // |u_bc| per side
     // nodes at the end of a staged step's sweep whose stores ask L2 to keep
     // them (evict-last hint): the next step reads those rows first (0: none)
     long long l2_hot;
@@ -573,173 +592,8 @@ __device__ __forceinline__ void node_update_generic(const KConst<R>& k, const Wa
     eq_accumulate(k, cb, b, R(1), R(1), R(1), R(1), out);
 }
 
-// Fast-path constants of a node with its own porosity (porosity field).
-template <class R>
-__device__ __forceinline__ void apply_eps(KConst<R>& k, R eps) {
-    const CellC<R> c = cell_consts(k, eps);
-    const R itf = R(1) - k.omf, itT = R(1) - k.omT;
-    k.eps = eps;
-    k.inv_eps = c.inv_eps;
-    k.e_nuK = c.e_nuK;
-    k.e_FK = c.e_FK;
-    k.c0 = c.c0;
-    k.c0sq = c.c0sq;
-    k.c1 = c.c1;
-    k.p_pref = c.p_pref;
-    k.bcoef = c.bcoef;
-    k.half_eps = R(0.5) * eps;
-    k.half_eps_ax = R(0.5) * eps * k.ax;
-    k.p_uF = c.p_pref * (R(4) / R(3)) * k.rho0 * k.kf * k.tau_f * c.inv_eps;
-    k.p_uu = c.p_pref * (R(2) / R(3)) * k.rho0 * c.inv_eps;
-    k.fA_uu = R(1.5) * itf * k.rho0 * c.inv_eps;
-    k.fA_uF = R(3) * k.rho0 * k.kf * c.inv_eps;
-    k.f_cu2 = R(4.5) * itf * k.rho0 * c.inv_eps;
-    k.f_cucF = R(9) * k.rho0 * k.kf * c.inv_eps;
-    k.h_uu = itT * R(1.5) * c.inv_eps;
-    k.h_cu2 = itT * R(4.5) * c.inv_eps;
-    k.h_ug = R(6) * k.kT * c.bcoef;
-    k.h0_uu = itT * (R(4) / R(9)) * R(1.5) * c.inv_eps;
-}
-
-// Macroscopic state of a node in the fast path: the moments the step
-// computes after streaming (Sec. 3.1-3.3) plus the derived quantities the
-// collision uses.
-template <class R>
-struct FastState {
-    R th, T, ux, uy, uu, Fx, Fy, uF, p, ep, Sxx, Syy, Sxy, gx, gy;
-};
-
 // Planes of the moment state (tau = 1 storage): p, u, S, T - T0, grad T.
 enum MomentPlane { MP = 0, MUX, MUY, MSXX, MSYY, MSXY, MTH, MGX, MGY };
 constexpr int kMPlanes = 9;
-
-// Moments of an interior node from its pulled populations (f[1..8], h[0..8]),
-// in the fast path's arrangement of node_moments.
-template <class R>
-__device__ __forceinline__ FastState<R> fast_moments(const KConst<R>& k, const R* f, const R* h, int y) {
-    FastState<R> s;
-    const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + (h[6] + h[7])) + h[8];
-    s.th = (sh + R(0.5) * k.Q) * k.inv_sigma;
-    s.T = k.T0 + s.th;
-    const R a13 = f[1] + f[3], a24 = f[2] + f[4], d58 = (f[5] + f[7]) + (f[6] + f[8]);
-    const R sf = a13 + a24 + d58;
-    const R mx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
-    const R my = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-    const R Pxx = a13 + d58, Pyy = a24 + d58;
-    const R Pxy = (f[5] + f[7]) - (f[6] + f[8]);
-    const R Gy = k.gbeta * s.th + row_ay(k, y);
-    const R vx = mx * k.inv_rho0 + k.half_eps_ax;
-    const R vy = my * k.inv_rho0 + k.half_eps * Gy;
-    const R vmag = sqrt(vx * vx + vy * vy);
-    const R iden = R(1) / (k.c0 + sqrt(k.c0sq + k.c1 * vmag));
-    s.ux = vx * iden;
-    s.uy = vy * iden;
-    if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
-    s.uu = s.ux * s.ux + s.uy * s.uy;
-    // |u| = |v| / (c0 + sqrt(c0^2 + c1 |v|)): no second square root
-    const R drag = k.e_nuK + k.e_FK * (vmag * iden);
-    s.Fx = k.eps * k.ax - drag * s.ux;
-    s.Fy = k.eps * Gy - drag * s.uy;
-    s.uF = s.ux * s.Fx + s.uy * s.Fy;
-    const R p = k.p_pref * sf - k.p_uF * s.uF - k.p_uu * s.uu;
-    s.p = p;
-    s.ep = k.eps * p;
-    const R re = k.rho0 * k.inv_eps;
-    s.Sxx = (Pxx - s.ep + re * s.ux * (s.Fx - s.ux)) * k.invD;
-    s.Syy = (Pyy - s.ep + re * s.uy * (s.Fy - s.uy)) * k.invD;
-    s.Sxy = (Pxy + re * (R(0.5) * (s.ux * s.Fy + s.Fx * s.uy) - s.ux * s.uy)) * k.invD;
-    const R hx = (h[1] - h[3]) + (h[5] - h[7]) + (h[8] - h[6]);
-    const R hy = (h[2] - h[4]) + (h[5] - h[7]) + (h[6] - h[8]);
-    const R qs = R(0.5) * k.Q * k.inv_sigma;
-    const R Nx = hx + s.T * (R(0.5) * s.Fx - s.ux) + qs * s.ux;
-    const R Ny = hy + s.T * (R(0.5) * s.Fy - s.uy) + qs * s.uy;
-    const R a = k.a_const - R(0.5) * s.ep * k.inv_rho0;
-    const R d = a - k.bcoef * s.uu;
-    // one reciprocal for 1/a = d r and 1/d = a r, r = 1/(a d)
-    const R r = R(1) / (a * d);
-    const R t = k.bcoef * (s.ux * Nx + s.uy * Ny) * (a * r);
-    const R ia = d * r;
-    s.gx = (Nx + t * s.ux) * ia;
-    s.gy = (Ny + t * s.uy) * ia;
-    return s;
-}
-
-// Collision of one node from its state: h_i* = (1 - 1/tau) h_i +
-// [h_i^eq/tau + source_i], the bracket split into the parts even and odd
-// under c_i -> -c_i so that each pair of opposite directions shares one
-// evaluation.  TAU1: tau_f = tau_T = 1, where the first term vanishes and
-// f, h are not read.  SOURCES = false drops the force and heat-source terms
-// (F_i, P_i, Q_i) and keeps the equilibria alone.  wscale (TAU1 only)
-// multiplies every output: the FP16 storage scale folded into the weights.
-template <class R, bool TAU1, bool SOURCES = true>
-__device__ __forceinline__ void fast_collide(const KConst<R>& k, const FastState<R>& s, const R* f,
-                                             const R* h, R* fo, R* ho, R wscale = R(1)) {
-    const R uF = SOURCES ? s.uF : R(0);
-    const R Fx = SOURCES ? s.Fx : R(0), Fy = SOURCES ? s.Fy : R(0);
-    const R kQ = SOURCES ? k.h_kQ : R(0), uQ = SOURCES ? k.h_uQ : R(0), k0Q = SOURCES ? k.h0_kQ : R(0);
-    const R T = s.T, ep = s.ep, uu = s.uu, ux = s.ux, uy = s.uy, gx = s.gx, gy = s.gy;
-    const R EF0 = k.fA_ep * ep - k.fA_uu * uu - k.fA_tr * (s.Sxx + s.Syy) - k.fA_uF * uF;
-    const R EH0 = k.h_sig * s.th - k.h_uu * T * uu + k.h_pT * T * ep + kQ;
-    const R Kc = k.h_cu2 * T;
-    const R Ku = k.h_u3 * T + (SOURCES ? k.h_ug * (ux * gx + uy * gy) : R(0)) + uQ;
-    const R epr = ep * k.inv_rho0;
-    const R Wx = SOURCES ? T * Fx + epr * gx : R(0), Wy = SOURCES ? T * Fy + epr * gy : R(0);
-    auto pair = [&](int i, int j, R w, R cu, R cF, R ScS, R cg, R cW) {
-        const R evF = EF0 + k.f_cu2 * cu * cu + k.f_ScS * ScS + k.f_cucF * cu * cF;
-        const R odF = k.f_cu * cu + k.f_cF * cF;
-        const R evH = EH0 + Kc * cu * cu;
-        const R odH = Ku * cu + k.h_g * cg + k.h_W * cW;
-        if (TAU1) {
-            fo[i] = w * (evF + odF);
-            fo[j] = w * (evF - odF);
-            ho[i] = w * (evH + odH);
-            ho[j] = w * (evH - odH);
-        } else {
-            fo[i] = k.omf * f[i] + w * (evF + odF);
-            fo[j] = k.omf * f[j] + w * (evF - odF);
-            ho[i] = k.omT * h[i] + w * (evH + odH);
-            ho[j] = k.omT * h[j] + w * (evH - odH);
-        }
-    };
-    const R w1 = wscale * (R(1) / R(9)), w5 = wscale * w_diag<R>();
-    pair(1, 3, w1, ux, Fx, s.Sxx, gx, Wx);
-    pair(2, 4, w1, uy, Fy, s.Syy, gy, Wy);
-    pair(5, 7, w5, ux + uy, Fx + Fy, s.Sxx + s.Syy + R(2) * s.Sxy, gx + gy, Wx + Wy);
-    pair(6, 8, w5, uy - ux, Fy - Fx, s.Sxx + s.Syy - R(2) * s.Sxy, gy - gx, Wy - Wx);
-    const R c0 = k.h0_sig * s.th - k.h0_uu * T * uu - k.h0_pT * T * ep + k0Q;
-    ho[0] = TAU1 ? wscale * c0 : k.omT * h[0] + c0;
-}
-
-// Interior node of one step, fast path.  Same arithmetic as node_moments +
-// eq_terms + BGK collision, rearranged for the GPU: the nine pull sources are
-// 32-bit offsets from the node (periodic wrap by per-thread deltas), plane
-// strides are uniform across the launch; then fast_moments and fast_collide.
-// TAU1: tau_f = tau_T = 1 (no (1 - 1/tau) terms; FP16 storage then takes its
-// scale in the collision weights).
-template <class R, class S, bool TAU1 = false>
-__device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __restrict__ src,
-                                                S* __restrict__ dst, int x, int y, uint32_t step) {
-    const int dxm = x == 0 ? k.nx - 1 : -1;
-    const int dxp = x == k.nx - 1 ? 1 - k.nx : 1;
-    const int dym = y == 0 ? (k.ny - 1) * k.pitch : -k.pitch;
-    const int dyp = y == k.ny - 1 ? (1 - k.ny) * k.pitch : k.pitch;
-    const int o[9] = {0, dxm, dym, dxp, dyp, dxm + dym, dxp + dym, dxp + dyp, dxm + dyp};
-    const int pl = k.plane32;
-    const int at = y * k.pitch + x;
-    const S* __restrict__ c = src + at;
-    const float sc = k.scale;
-    R f[9], h[9];
-#pragma unroll
-    for (int i = 1; i < 9; ++i) f[i] = load_pop<S, R>(c + ((i - 1) * pl + o[i]), sc);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) h[i] = load_pop<S, R>(c + ((8 + i) * pl + o[i]), sc);
-    const FastState<R> s = fast_moments(k, f, h, y);
-    R fo[9], ho[9];
-    constexpr bool prescale = TAU1 && std::is_same<S, __half>::value;
-    if constexpr (TAU1) fast_collide<R, true>(k, s, f, h, fo, ho, prescale ? R(k.inv_scale) : R(1));
-    else fast_collide<R, false>(k, s, f, h, fo, ho);
-    Dither dither((uint32_t)at, step);
-    store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
-}
 
 }  // namespace lbm

@@ -2,6 +2,7 @@
 // batched step's Nusselt kernel (internal).
 #pragma once
 
+#include "lbm_core.cuh"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -26,8 +27,8 @@ __device__ __forceinline__ State<R> node_state_at(const KConst<R>& k, const S* _
     return wall_state(k, cb, w, s, thff, thb);
 }
 
-// (u_x, u_y, T - T0) of node (x, y) after streaming: the step's fast path
-// for interior nodes (same moments as node_state_at up to rounding order),
+// (u_x, u_y, T - T0) of node (x, y) after streaming: the step's own
+// arithmetic for interior nodes (same moments as node_state_at up to rounding order),
 // node_state_at for wall nodes.
 template <class R, class S>
 __device__ __forceinline__ void node_u_th(const KConst<R>& k, const S* __restrict__ src, int x, int y, R* ux,
@@ -41,14 +42,9 @@ __device__ __forceinline__ void node_u_th(const KConst<R>& k, const S* __restric
     }
     Pops<R> P;
     pull(k, src, x, y, P);
-    FastState<R> s;
-    if (k.eps_field) {
-        KConst<R> kc = k;
-        apply_eps(kc, node_eps(k, x, y));
-        s = fast_moments(kc, P.f, P.h, y);
-    } else {
-        s = fast_moments(k, P.f, P.h, y);
-    }
+    const Cell<R> c = node_cell(k, x, y);
+    const CoreState<R> s = core_moments(k, c, eps_ay(k, c, y), P.f, P.h);
+    if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
     *ux = s.ux;
     *uy = s.uy;
     *th = s.th;

@@ -182,8 +182,10 @@ inline lbm::KConst<R> make_kconst(const lbm_params* p, const Derived& d, const L
     k.inv_eps = R(1.0 / eps);
     k.sigma = R(p->sigma);
     k.inv_sigma = R(1.0 / p->sigma);
-    k.omf = R(1.0 - 1.0 / p->tau_f);
-    k.omT = R(1.0 - 1.0 / p->tau_T);
+    // 1 - 1/tau, complementary to 1/tau as rounded to R (h_sig below): their
+    // sum multiplies the temperature in each step
+    k.omf = R(1) - R(1.0 / p->tau_f);
+    k.omT = R(1) - R(1.0 / p->tau_T);
     k.tau_f = R(p->tau_f);
     k.kf = R(1.0 - 0.5 / p->tau_f);
     k.kT = R(1.0 - 0.5 / p->tau_T);
@@ -213,39 +215,106 @@ inline lbm::KConst<R> make_kconst(const lbm_params* p, const Derived& d, const L
     k.inv_scale = 1.0f / k.scale;
     k.flag = flag;
     k.plane32 = (int)L.plane_elems;
-    // interior fast path: h* = (1 - 1/tau) h + [h^eq / tau + source], split
-    // into parts even and odd in c_i (lbm_device.cuh, interior_update)
+    // the node update (lbm_core.cuh)
     const double rho0 = p->rho0, ie = 1.0 / eps, itf = 1.0 / p->tau_f, itT = 1.0 / p->tau_T;
     const double kf = 1.0 - 0.5 / p->tau_f, kT = 1.0 - 0.5 / p->tau_T;
-    const double bc = 0.5 * (1.0 / eps - 1.0 / p->sigma);
+    const double invD = 1.0 / (kCs2 * rho0 * (d.A - p->tau_f));
+    // eps p = e1 sum f, e1 = c_s^2/(1 - w_0) = 3/5.  Each step multiplies the
+    // pressure by 1 - 1/tau + e1 (3/tau) (4 w_1 + 4 w_5) = 1, so e1 is fitted
+    // to the other factors as R holds them and its own rounding kept apart
+    // (e1_lo): an error of one unit in the last place would build up.
+    const R fA = R(3.0 * itf);
+    const double wsum = 4.0 * (double(R(1) / R(9)) + double(R(1) / R(36)));
+    const double e1 = sizeof(R) == 4 ? (1.0 - double(k.omf)) / (double(fA) * wsum) : kCs2 / (1.0 - kW0);
+    const double aS = 1.5 * itf * rho0 * d.A * invD;
+    const double b0 = -0.5 / p->sigma, bc = 0.5 * ie + b0;
     k.inv_rho0 = R(1.0 / rho0);
-    k.half_eps_ax = R(0.5 * eps * p->ax);
-    k.half_eps = R(0.5 * eps);
-    k.p_uF = R(kCs2 / (eps * (1.0 - kW0)) * (4.0 / 3.0) * rho0 * kf * p->tau_f * ie);
-    k.p_uu = R(kCs2 / (eps * (1.0 - kW0)) * (2.0 / 3.0) * rho0 * ie);
-    k.fA_ep = R(3.0 * itf);
-    k.fA_uu = R(1.5 * itf * rho0 * ie);
-    k.fA_tr = R(0.5 * itf * rho0 * d.A);
-    k.fA_uF = R(3.0 * rho0 * kf * ie);
-    k.f_cu2 = R(4.5 * itf * rho0 * ie);
-    k.f_ScS = R(1.5 * itf * rho0 * d.A);
-    k.f_cucF = R(9.0 * rho0 * kf * ie);
+    k.hq_sigma = R(0.5 * d.Q / p->sigma);
+    k.half_Q = R(0.5 * d.Q);
+    k.eay = R(eps * p->ay);
+    k.half_ax = R(0.5 * p->ax);
+    k.e1 = R(e1);
+    k.e1_lo = R(e1 - double(k.e1));
+    k.aS = R(aS);
+    k.qu_ie = R(rho0 * (4.5 * itf - aS));
+    k.qF_ie = R(rho0 * (9.0 * kf + aS));
     k.f_cu = R(3.0 * rho0 * itf);
+    // Each step multiplies the momentum by 1 - 1/tau + (f_cu/rho0) (2 w_1 +
+    // 4 w_5) = 1: what the factors as R holds them miss (8e-9 in FP32 at
+    // tau = 1) goes into u = v/(2 c0), whose constant has a low part.
+    k.gain = sizeof(R) == 4 ? R((1.0 - double(k.omf)) * rho0 /
+                                    ((2.0 * double(R(1) / R(9)) + 4.0 * double(R(1) / R(36))) * double(k.f_cu)) - 1.0)
+                            : R(0);
+    // The sum of the collided f_1..f_8 is fA wsum (eps p) + tsum tr Q, and the
+    // u u and u F parts of the two cancel (e2 = -(4/5) rho0 kf tau/eps, e3 =
+    // -(2/5) rho0/eps): fitted to the factors as R holds them, since the rest
+    // is a source of mass in each step.
+    const double tsum = sizeof(R) == 4 ? 2.0 * double(R(1) / R(9)) + 4.0 * double(R(1) / R(36)) + double(R(-1) / R(3)) * wsum : 4.0 / 27.0;
+    const double c3 = sizeof(R) == 4 ? -tsum / (double(fA) * wsum) : -(4.0 / 27.0) / (3.0 * itf * (1.0 - kW0));
+    k.e2_ie = R(c3 * (double(k.qF_ie) - double(k.aS) * rho0));
+    k.e3_ie = R(c3 * (double(k.qu_ie) + double(k.aS) * rho0));
+    k.cu2_ie = R(4.5 * itf * rho0);
+    k.cuF_ie = R(9.0 * rho0 * kf);
+    k.b_0 = R(b0);
+    k.ug_b = R(6.0 * kT);
+    k.kc_ie = R(4.5 * itT);
+    k.a_ep = R(-0.5 / rho0);
+    k.aS2 = R(2.0 * aS);
+    k.f_ScS = R(1.5 * itf * rho0 * d.A);
+    k.f_ScS2 = R(3.0 * itf * rho0 * d.A);
+    k.fA_ep = fA;
     k.f_cF = R(3.0 * rho0 * kf);
     k.h_sig = R(itT * p->sigma);
-    k.h_uu = R(itT * 1.5 * ie);
-    k.h_pT = R(itT * 3.0 / rho0);
     k.h_kQ = R(kT * d.Q);
-    k.h_cu2 = R(itT * 4.5 * ie);
+    k.h_pT = R(itT * 3.0 / rho0);
+    k.h0_pT = R(-itT * (5.0 / 3.0) / rho0);
     k.h_u3 = R(3.0 * itT);
-    k.h_ug = R(6.0 * kT * bc);
     k.h_uQ = R(3.0 * kT * d.Q / p->sigma);
     k.h_g = R(itT * p->sigma * d.B);
     k.h_W = R(3.0 * kT);
-    k.h0_sig = R(itT * kW0 * p->sigma);
-    k.h0_uu = R(itT * kW0 * 1.5 * ie);
-    k.h0_pT = R(itT * (5.0 / 3.0) / rho0);
-    k.h0_kQ = R(kW0 * kT * d.Q);
+    k.h_Wr = R(3.0 * kT / rho0);
+    for (int s = 0; s < 4; ++s) k.u_abs[s] = R(sqrt(p->u_bc[s][0] * p->u_bc[s][0] + p->u_bc[s][1] * p->u_bc[s][1]));
+    lbm::Cell<R>& c = k.cell;
+    c.eps = R(eps);
+    c.ie = R(ie);
+    c.eg = R(eps * d.gbeta);
+    c.eax = R(eps * p->ax);
+    c.heax = R(0.5 * eps * p->ax);
+    c.c0 = R(c0);
+    c.c0sq = R(c0 * c0);
+    c.c1 = R(c1);
+    c.nnuK = R(-eps * nuK);
+    c.nFK = R(-eps * FK);
+    c.ih = R(0.5 / c0);
+    c.il = R(0.5 / c0 * (1.0 + double(k.gain)) - double(c.ih));
+    c.ci = R(-c1 * 0.5 / c0);
+    c.re = R(rho0 * ie);
+    c.qu = R(rho0 * (4.5 * itf - aS) * ie);
+    c.qF = R(rho0 * (9.0 * kf + aS) * ie);
+    c.e2 = R(c3 * (double(c.qF) - double(k.aS) * rho0 * ie));
+    // e3's own rounding is the larger rest: of the neighbours of q_u within
+    // three units in the last place (5e-7 of the u u term, no source of mass)
+    // the one whose e3 is nearest to a value of R
+    if (sizeof(R) == 4) {
+        float q = float(c.qu), best = q;
+        double least = 1e30;
+        for (int j = 0; j < 3; ++j) q = nextafterf(q, -1e30f);
+        for (int j = 0; j < 7; ++j, q = nextafterf(q, 1e30f)) {
+            const double want = c3 * (double(q) + double(k.aS) * rho0 * ie), miss = fabs(want - double(float(want)));
+            if (miss < least) {
+                least = miss;
+                best = q;
+            }
+        }
+        c.qu = R(best);
+    }
+    c.e3 = R(c3 * (double(c.qu) + double(k.aS) * rho0 * ie));
+    c.cu2 = R(4.5 * itf * rho0 * ie);
+    c.cuF = R(9.0 * rho0 * kf * ie);
+    c.b = R(bc);
+    c.nb = R(-bc);
+    c.ug = R(6.0 * kT * bc);
+    c.kc = R(4.5 * itT * ie);
     // porosity field support (the field pointer is set by lbm_set_fields)
     k.eps_field = nullptr;
     k.kc_inv_ref = R(eps < 1.0 ? (1.0 - eps) * (1.0 - eps) / (eps * eps * eps) : 0.0);
@@ -253,6 +322,12 @@ inline lbm::KConst<R> make_kconst(const lbm_params* p, const Derived& d, const L
     k.inv_sqrt_Kref = R(isinf(d.K) ? 0.0 : 1.0 / sqrt(d.K));
     k.p_pref_eps = R(kCs2 / (1.0 - kW0));
     k.da_inf = p->da_infinite ? 1 : 0;
+    // with q = (1 - e)/e: eps nu/K(e) = nu/K_ref q^2 / kc, eps F_eps/sqrt(K(e))
+    // = 1.75/sqrt(150 kc K_ref) q/e, kc = (1 - eps)^2/eps^3 at the reference
+    const double kc = eps < 1.0 ? (1.0 - eps) * (1.0 - eps) / (eps * eps * eps) : 0.0;
+    const bool drag = !p->da_infinite && kc > 0.0 && !isinf(d.K);
+    k.nnuK_q2 = R(drag ? -nuK / kc : 0.0);
+    k.nFK_q = R(drag && p->forchheimer ? -1.75 / sqrt(150.0 * kc * d.K) : 0.0);
     k.forch = p->forchheimer ? 1 : 0;
     k.ay_row = nullptr;
     return k;

@@ -34,13 +34,7 @@ k_step(const __grid_constant__ KConst<R> k, const S* __restrict__ src, S* __rest
         wall_update(k, src, dst, x, y, step);
         return;
     }
-    if constexpr (EPS_FIELD) {
-        KConst<R> kc = k;
-        apply_eps(kc, node_eps(k, x, y));
-        interior_update<R, S, TAU1>(kc, src, dst, x, y, step);
-    } else {
-        interior_update<R, S, TAU1>(k, src, dst, x, y, step);
-    }
+    interior_update<R, S, EPS_FIELD, TAU1>(k, src, dst, x, y, step);
 }
 
 template <class R, class S>

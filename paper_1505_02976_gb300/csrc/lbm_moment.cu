@@ -13,7 +13,7 @@
 //   1. expands the moments of every node (and a one-node halo) into its
 //      17 post-collision populations,
 //   2. pulls the 17 populations of each node from its neighbours,
-//   3. computes the new moments (fast_moments), and the boundary state of the
+//   3. computes the new moments (core_moments), and the boundary state of the
 //      wall nodes from their x_f, x_ff neighbours, and stores them.
 // Each warp owns a strip of up to 30 columns (32 lanes: the strip and one
 // halo column on each side) and a segment of rows, and marches up the
@@ -32,6 +32,7 @@
 
 #include <algorithm>
 
+#include "lbm_core.cuh"
 #include "lbm_internal.h"
 
 #ifndef LBM_MOMENT_WAVES
@@ -48,45 +49,41 @@ constexpr int kMStrip = 30;      // output columns of a strip, at most (32 lanes
 template <class R> struct MomentOccupancy { static constexpr int blocks = LBM_MOMENT_BLOCKS; };
 template <> struct MomentOccupancy<double> { static constexpr int blocks = 2; };
 
-// State of a node from its stored moments; F is recomputed from (u, T) as in
-// fast_moments (and, for a wall node, as in wall_state).
-template <class R>
-__device__ __forceinline__ FastState<R> state_from_moments(const KConst<R>& k, const R* m, int y) {
-    FastState<R> s;
-    s.p = m[MP];
+// Populations of a node from its stored moments; F is recomputed from (u, T)
+// as in core_moments (and, for a wall node, as in core_boundary).
+template <class R, bool SOURCES>
+__device__ __forceinline__ void expand_moments(const KConst<R>& k, const Cell<R>& c, R eay, const R* m, R* fo, R* ho) {
+    CoreState<R> s;
     s.ux = m[MUX];
     s.uy = m[MUY];
-    s.Sxx = m[MSXX];
-    s.Syy = m[MSYY];
-    s.Sxy = m[MSXY];
     s.th = m[MTH];
     s.gx = m[MGX];
     s.gy = m[MGY];
-    s.T = k.T0 + s.th;
-    s.uu = s.ux * s.ux + s.uy * s.uy;
-    const R drag = k.e_nuK + k.e_FK * sqrt(s.uu);
-    const R Gy = k.gbeta * s.th + row_ay(k, y);
-    s.Fx = k.eps * k.ax - drag * s.ux;
-    s.Fy = k.eps * Gy - drag * s.uy;
-    s.uF = s.ux * s.Fx + s.uy * s.Fy;
-    s.ep = k.eps * s.p;
-    return s;
+    s.T = ladd(k.T0, s.th);
+    const R uu = lfma(s.ux, s.ux, lmul(s.uy, s.uy));
+    const R nd = lfma(c.nFK, lsqrt(uu), c.nnuK);
+    s.Fx = lfma(nd, s.ux, c.eax);
+    s.Fy = lfma(nd, s.uy, lfma(c.eg, s.th, eay));
+    s.ep = lmul(c.eps, m[MP]);
+    const Shear<R> S = {m[MSXX], m[MSYY], m[MSXY]};
+    R Qxx, Qyy, Q2;
+    shear_form<SOURCES>(k, c, s.ux, s.uy, s.Fx, s.Fy, S, Qxx, Qyy, Q2);
+    core_emit<true, SOURCES>(k, c, s, Qxx, Qyy, Q2, (const R*)nullptr, (const R*)nullptr, fo, ho, R(1));
+}
+
+// Constants of node (x, y), the porosity field known at compile time.
+template <class R, bool EPS_FIELD>
+__device__ __forceinline__ Cell<R> moment_cell(const KConst<R>& k, int x, int y) {
+    if constexpr (EPS_FIELD) return field_cell<R>(k, node_eps(k, x, y));
+    else return uniform_cell<R>(k);
 }
 
 // Plane strides are 32-bit (9 planes of ny * pitch < 2^31 elements).
 template <class R>
-__device__ __forceinline__ void store_moments(const KConst<R>& k, R* dst, long long at, const FastState<R>& s) {
+__device__ __forceinline__ void store_moments(const KConst<R>& k, R* dst, long long at, const R* m) {
     R* d = dst + at;
-    const int pl = k.plane32;
-    d[MP * pl] = s.p;
-    d[MUX * pl] = s.ux;
-    d[MUY * pl] = s.uy;
-    d[MSXX * pl] = s.Sxx;
-    d[MSYY * pl] = s.Syy;
-    d[MSXY * pl] = s.Sxy;
-    d[MTH * pl] = s.th;
-    d[MGX * pl] = s.gx;
-    d[MGY * pl] = s.gy;
+#pragma unroll
+    for (int q = 0; q < kMPlanes; ++q) d[q * k.plane32] = m[q];
 }
 
 // Boundary state of wall node (x, y) from m, the new moments of its x_f node,
@@ -148,13 +145,8 @@ __device__ __forceinline__ Expanded<R> expand_node(const KConst<R>& k, const R* 
     Expanded<R> e;
     if (!ok) return e;
     R fo[9], ho[9];
-    if constexpr (EPS_FIELD) {
-        KConst<R> kc = k;
-        apply_eps(kc, node_eps(k, xe, r));
-        fast_collide<R, true, SOURCES>(kc, state_from_moments(kc, m, r), nullptr, nullptr, fo, ho);
-    } else {
-        fast_collide<R, true, SOURCES>(k, state_from_moments(k, m, r), nullptr, nullptr, fo, ho);
-    }
+    const Cell<R> c = moment_cell<R, EPS_FIELD>(k, xe, r);
+    expand_moments<R, SOURCES>(k, c, eps_ay(k, c, r), m, fo, ho);
     e.up[0] = fo[2]; e.up[1] = fo[5]; e.up[2] = fo[6];
     e.up[3] = ho[2]; e.up[4] = ho[5]; e.up[5] = ho[6];
     e.hz[0] = fo[1]; e.hz[1] = fo[3]; e.hz[2] = ho[0]; e.hz[3] = ho[1]; e.hz[4] = ho[3];
@@ -242,17 +234,22 @@ k_step_m(const __grid_constant__ KConst<R> k, const R* __restrict__ src, R* dst,
         h[8] = __shfl_up_sync(0xffffffffu, ep.dn[5], 1);
         const bool wall_row = (wallS && y == 0) || (wallN && y == k.ny - 1);
         if (!wall_row) {
-            FastState<R> s = {};
+            R mo[kMPlanes] = {};
             if (out_col && !wall_col) {
-                const long long at = (long long)y * k.pitch + x;
-                if constexpr (EPS_FIELD) {
-                    KConst<R> kc = k;
-                    apply_eps(kc, node_eps(k, x, y));
-                    s = fast_moments(kc, f, h, y);
-                } else {
-                    s = fast_moments(k, f, h, y);
-                }
-                store_moments(k, dst, at, s);
+                const Cell<R> c = moment_cell<R, EPS_FIELD>(k, x, y);
+                const CoreState<R> s = core_moments(k, c, eps_ay(k, c, y), f, h);
+                const Shear<R> S = core_shear(k, c, s);
+                if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
+                mo[MP] = lmul(s.ep, c.ie);
+                mo[MUX] = s.ux;
+                mo[MUY] = s.uy;
+                mo[MSXX] = S.xx;
+                mo[MSYY] = S.yy;
+                mo[MSXY] = S.xy;
+                mo[MTH] = s.th;
+                mo[MGX] = s.gx;
+                mo[MGY] = s.gy;
+                store_moments(k, dst, (long long)y * k.pitch + x, mo);
             }
             if (wallWE) {
                 // x_f and x_ff of a W or E wall node are the nodes one and two
@@ -262,16 +259,9 @@ k_step_m(const __grid_constant__ KConst<R> k, const R* __restrict__ src, R* dst,
                 const int in = x == 0 ? 1 : -1;
                 const int lf = wall_col ? lane + in : lane, lff = wall_col ? lane + 2 * in : lane;
                 R mf[kMPlanes];
-                mf[MP] = __shfl_sync(0xffffffffu, s.p, lf);
-                mf[MUX] = __shfl_sync(0xffffffffu, s.ux, lf);
-                mf[MUY] = __shfl_sync(0xffffffffu, s.uy, lf);
-                mf[MSXX] = __shfl_sync(0xffffffffu, s.Sxx, lf);
-                mf[MSYY] = __shfl_sync(0xffffffffu, s.Syy, lf);
-                mf[MSXY] = __shfl_sync(0xffffffffu, s.Sxy, lf);
-                mf[MTH] = __shfl_sync(0xffffffffu, s.th, lf);
-                mf[MGX] = __shfl_sync(0xffffffffu, s.gx, lf);
-                mf[MGY] = __shfl_sync(0xffffffffu, s.gy, lf);
-                const R thff = __shfl_sync(0xffffffffu, s.th, lff);
+#pragma unroll
+                for (int q = 0; q < kMPlanes; ++q) mf[q] = __shfl_sync(0xffffffffu, mo[q], lf);
+                const R thff = __shfl_sync(0xffffffffu, mo[MTH], lff);
                 if (wall_col) wall_store(k, dst, x, y, mf, thff);
             }
         } else if (y == k.ny - 1) {
@@ -298,10 +288,9 @@ __global__ void k_expand_m(const __grid_constant__ KConst<R> k, const R* __restr
     R m[kMPlanes];
 #pragma unroll
     for (int q = 0; q < kMPlanes; ++q) m[q] = src[q * k.plane + at];
-    KConst<R> kc = k;
-    if (k.eps_field) apply_eps(kc, node_eps(k, x, y));
+    const Cell<R> c = node_cell(k, x, y);
     R fo[9], ho[9];
-    fast_collide<R, true, SOURCES>(kc, state_from_moments(kc, m, y), nullptr, nullptr, fo, ho);
+    expand_moments<R, SOURCES>(k, c, eps_ay(k, c, y), m, fo, ho);
 #pragma unroll
     for (int i = 1; i < 9; ++i) dst[(i - 1) * k.plane + at] = fo[i];
 #pragma unroll

@@ -23,34 +23,123 @@ __device__ __forceinline__ void store_node(const KConst<R>& k, S* __restrict__ d
     store_planes<S, R>(dst + at, k.plane, fo, ho, k.inv_scale, dither);
 }
 
-// Wall node of one step: the generic update of its x_f neighbour's pulled
-// populations (NEES rebuild and boundary collision, see
-// node_update_generic).  Kept out of line: only the 4(N - 1) wall threads
-// take it.
+// Interior node of one step: the nine pull sources are 32-bit offsets from
+// the node (periodic wrap by per-thread deltas), plane strides are uniform
+// across the launch.  TAU1: tau_f = tau_T = 1 (FP16 storage then takes its
+// scale in the collision weights).
+template <class R, class S, bool EPS_FIELD, bool TAU1>
+__device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __restrict__ src,
+                                                S* __restrict__ dst, int x, int y, uint32_t step) {
+    const int dxm = x == 0 ? k.nx - 1 : -1;
+    const int dxp = x == k.nx - 1 ? 1 - k.nx : 1;
+    const int dym = y == 0 ? (k.ny - 1) * k.pitch : -k.pitch;
+    const int dyp = y == k.ny - 1 ? (1 - k.ny) * k.pitch : k.pitch;
+    const int o[9] = {0, dxm, dym, dxp, dyp, dxm + dym, dxp + dym, dxp + dyp, dxm + dyp};
+    const int pl = k.plane32;
+    const int at = y * k.pitch + x;
+    const S* __restrict__ c = src + at;
+    const float sc = k.scale;
+    R f[9], h[9];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) f[i] = load_pop<S, R>(c + ((i - 1) * pl + o[i]), sc);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) h[i] = load_pop<S, R>(c + ((8 + i) * pl + o[i]), sc);
+    Cell<R> cell;
+    if constexpr (EPS_FIELD) cell = field_cell<R>(k, k.eps_field[(long long)y * k.nx + x]);
+    else cell = uniform_cell<R>(k);
+    R fo[9], ho[9];
+    constexpr bool prescale = TAU1 && std::is_same<S, __half>::value;
+    core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo, ho, prescale ? R(k.inv_scale) : R(1));
+    Dither dither((uint32_t)at, step);
+    store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
+}
+
+// Where a wall node's update takes its pulled values from: the population
+// buffer src in global memory.
 template <class R, class S>
-__device__ __noinline__ void wall_update(const KConst<R>& k, const S* __restrict__ src,
-                                         S* __restrict__ dst, int x, int y, uint32_t step) {
+struct GlobalSource {
+    const S* src;
+    __device__ __forceinline__ void operator()(const KConst<R>& k, int x, int y, Pops<R>& P) const { pull(k, src, x, y, P); }
+};
+
+// Wall node (x, y) of one step.  At tau_f = tau_T = 1 the extrapolated
+// non-equilibrium part vanishes and the node is the collision of its boundary
+// state (core_boundary): one moment evaluation at x_f and one collision.
+template <class R, class Source>
+__device__ __forceinline__ void wall_node_tau1(const KConst<R>& k, const Source& source, int x, int y, R* fo, R* ho) {
     const WallInfo w = classify(k, x, y);
     Pops<R> P;
-    pull(k, src, w.xs, w.ys, P);
+    source(k, w.xs, w.ys, P);
+    R thff = R(0);
+    if (w.tside < 0) {
+        Pops<R> Q;
+        source(k, w.xff, w.yff, Q);  // only h is used
+        thff = core_theta(k, core_hsum(Q.h));
+    }
+    const Cell<R> cs = node_cell(k, w.xs, w.ys), cb = node_cell(k, x, y);
+    CoreState<R> s = core_moments(k, cs, eps_ay(k, cs, w.ys), P.f, P.h);
+    const Shear<R> S_ = core_shear(k, cs, s);
+    const R thb = w.tside >= 0 ? k.T_bc[w.tside] - k.T0 : R(0);
+    core_boundary(k, cs, cb, eps_ay(k, cb, y), k.u_bc[w.uside][0], k.u_bc[w.uside][1], k.u_abs[w.uside], w.tside >= 0,
+                  w.fixgx != 0, w.fixgy != 0, thb, thff, s);
+    R Qxx, Qyy, Q2;
+    shear_form<true>(k, cb, s.ux, s.uy, s.Fx, s.Fy, S_, Qxx, Qyy, Q2);
+    core_emit<true, true>(k, cb, s, Qxx, Qyy, Q2, P.f, P.h, fo, ho, R(1));
+    if (!lfinite(ho[0])) atomicOr(k.flag, 1);
+}
+
+// The same at other relaxation times: the generic update of its x_f
+// neighbour's pulled populations (NEES rebuild and boundary collision, see
+// node_update_generic).
+template <class R, class Source>
+__device__ __forceinline__ void wall_node_generic(const KConst<R>& k, const Source& source, int x, int y, R* fo, R* ho) {
+    const WallInfo w = classify(k, x, y);
+    Pops<R> P;
+    source(k, w.xs, w.ys, P);
     R in[17], out[17];
 #pragma unroll
     for (int i = 1; i < 9; ++i) in[i - 1] = P.f[i];
 #pragma unroll
     for (int i = 0; i < 9; ++i) in[8 + i] = P.h[i];
     R thff = R(0);
-    if (w.tside < 0) thff = (pull_hsum<R, R, S>(k, src, w.xff, w.yff) + R(0.5) * k.Q) * k.inv_sigma;
+    if (w.tside < 0) {
+        Pops<R> Q;
+        source(k, w.xff, w.yff, Q);
+        thff = (Q.h[0] + Q.h[1] + Q.h[2] + Q.h[3] + Q.h[4] + Q.h[5] + Q.h[6] + Q.h[7] + Q.h[8] + R(0.5) * k.Q) * k.inv_sigma;
+    }
     const R thb = w.tside >= 0 ? k.T_bc[w.tside] - k.T0 : R(0);
     node_update_generic(k, w, in, node_eps(k, w.xs, w.ys), node_eps(k, x, y), thff, thb, row_ay(k, w.ys),
                         row_ay(k, y), out);
     if (!isfinite(out[0] + out[8])) atomicOr(k.flag, 1);
-    R fo[9], ho[9];
 #pragma unroll
     for (int i = 1; i < 9; ++i) fo[i] = out[i - 1];
 #pragma unroll
     for (int i = 0; i < 9; ++i) ho[i] = out[8 + i];
+}
+
+// Both out of line: only the 4(N - 1) wall threads take them.
+template <class R, class S>
+__device__ __noinline__ void wall_update_tau1(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst,
+                                              int x, int y, uint32_t step) {
+    R fo[9], ho[9];
+    wall_node_tau1(k, GlobalSource<R, S>{src}, x, y, fo, ho);
     Dither dither((uint32_t)(y * k.pitch + x), step);
     store_node(k, dst, (long long)y * k.pitch + x, fo, ho, &dither);
+}
+template <class R, class S>
+__device__ __noinline__ void wall_update_generic(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst,
+                                                 int x, int y, uint32_t step) {
+    R fo[9], ho[9];
+    wall_node_generic(k, GlobalSource<R, S>{src}, x, y, fo, ho);
+    Dither dither((uint32_t)(y * k.pitch + x), step);
+    store_node(k, dst, (long long)y * k.pitch + x, fo, ho, &dither);
+}
+
+template <class R, class S>
+__device__ __forceinline__ void wall_update(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst, int x,
+                                            int y, uint32_t step) {
+    if (k.omf == R(0) && k.omT == R(0)) wall_update_tau1(k, src, dst, x, y, step);
+    else wall_update_generic(k, src, dst, x, y, step);
 }
 
 }  // namespace lbm

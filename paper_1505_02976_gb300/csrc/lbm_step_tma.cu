@@ -1,8 +1,8 @@
 // lbm_step_tma.cu -- the FP32 / FP16-storage step with its loads staged by
 // the tensor memory accelerator (TMA).
 //
-// Same per-node arithmetic as k_step (fast_moments and fast_collide for
-// interior nodes, the out-of-line NEES path for wall nodes), but the 17
+// Same per-node arithmetic as k_step (core_interior for interior nodes, the
+// out-of-line NEES path for wall nodes), but the 17
 // pulled values of every interior node reach the block through shared
 // memory.  Pull streaming reads plane i of output row y from global row
 // y - c_iy, so each plane of each global row is used by exactly one output
@@ -33,7 +33,6 @@
 #include <type_traits>
 
 #include "lbm_internal.h"
-#include "lbm_pair.cuh"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -256,18 +255,10 @@ __device__ __forceinline__ bool staged_rows(const KConst<float>& k, const S* __r
 #pragma unroll
             for (int i = 0; i < 9; ++i) h[i] = load_pop<S, float>(sl + ((8 + i) * L::plane + plane_dx(8 + i)), k.scale);
             float fo[9], ho[9];
-            auto collide = [&](const KConst<float>& kk) {
-                const FastState<float> st = fast_moments(kk, f, h, y);
-                if constexpr (TAU1) fast_collide<float, true>(kk, st, f, h, fo, ho, prescale ? kk.inv_scale : 1.0f);
-                else fast_collide<float, false>(kk, st, f, h, fo, ho);
-            };
-            if constexpr (EPS_FIELD) {
-                KConst<float> kc = k;
-                apply_eps(kc, node_eps(k, x, y));
-                collide(kc);
-            } else {
-                collide(k);
-            }
+            Cell<float> cell;
+            if constexpr (EPS_FIELD) cell = field_cell<float>(k, node_eps(k, x, y));
+            else cell = uniform_cell<float>(k);
+            core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo, ho, prescale ? k.inv_scale : 1.0f);
             const int at = y * k.pitch + x;
             Dither dither((uint32_t)at, step);
             store_planes<S, float>(dst + at, k.plane32, fo, ho, prescale ? 1.0f : k.inv_scale, &dither, hot);
@@ -344,20 +335,16 @@ __device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const _
         const int at = y * k.pitch + xa;
         if constexpr (TAU1 && !EPS_FIELD) {
             if (act0 && act1) {
-                // both nodes interior: the lane form on the pair, node a in
-                // .x and node b in .y of every packed value (the compiler
-                // may fuse some of its multiplies into the following adds,
-                // so the pair's values can differ from those of the
-                // one-node path by FP32 rounding; the stored FP16 values
-                // then differ by at most one rounding step)
+                // both nodes interior: the packed form of the node update,
+                // node a in .x and node b in .y of every packed value
                 float2 f2[9], h2[9], fo2[9], ho2[9];
                 const float2 sc = make_float2(k.scale, k.scale);
 #pragma unroll
                 for (int i = 1; i < 9; ++i) f2[i] = lmul(__half22float2(pk[i - 1]), sc);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) h2[i] = lmul(__half22float2(pk[8 + i]), sc);
-                const LaneState<float2> st = lane_moments<float2>(k, f2, h2, y);
-                lane_collide<float2>(k, st, fo2, ho2, k.inv_scale);
+                const Cell<float2> cell = uniform_cell<float2>(k);
+                core_interior<true>(k, cell, eps_ay(k, cell, y), f2, h2, fo2, ho2, k.inv_scale);
                 const Dither dither((uint32_t)at, step);
                 uint32_t* wd = reinterpret_cast<uint32_t*>(dst + at);
                 const int pw = k.plane32 >> 1;
@@ -390,18 +377,10 @@ __device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const _
             for (int i = 1; i < 9; ++i) f[i] = (n == 0 ? __low2float(pk[i - 1]) : __high2float(pk[i - 1])) * k.scale;
 #pragma unroll
             for (int i = 0; i < 9; ++i) h[i] = (n == 0 ? __low2float(pk[8 + i]) : __high2float(pk[8 + i])) * k.scale;
-            auto collide = [&](const KConst<float>& kk) {
-                const FastState<float> st = fast_moments(kk, f, h, y);
-                if constexpr (TAU1) fast_collide<float, true>(kk, st, f, h, fo[n], ho[n], kk.inv_scale);
-                else fast_collide<float, false>(kk, st, f, h, fo[n], ho[n]);
-            };
-            if constexpr (EPS_FIELD) {
-                KConst<float> kc = k;
-                apply_eps(kc, node_eps(k, xa + n, y));
-                collide(kc);
-            } else {
-                collide(k);
-            }
+            Cell<float> cell;
+            if constexpr (EPS_FIELD) cell = field_cell<float>(k, node_eps(k, xa + n, y));
+            else cell = uniform_cell<float>(k);
+            core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo[n], ho[n], TAU1 ? k.inv_scale : 1.0f);
         }
         if (act0 && act1) {
             const Dither dither((uint32_t)at, step);
