@@ -6,23 +6,15 @@
 // node x of s_{n+1} depends on the 17 populations it pulls from its source
 // node (x itself, or x_f for a wall node), on T(x_ff) for adiabatic walls,
 // on the porosity at the source and at x, and on the Dirichlet T_b.  The
-// adjoint runs the steps backwards:
-//   k_adj_pass,   per node, the transposed Jacobian of its update applied to
-//   k_adj_combine: lambda_{n+1}(x), from directional derivatives of the very
-//                 same per-node code (node_update_generic) evaluated in dual
-//                 numbers, giving the adjoints of the pulled values and the
-//                 porosity / wall-temperature contributions.  The update
-//                 depends on its 17 pulled values only through the BGK term
-//                 (1 - 1/tau) in and through nine linear moment sums M in
-//                 (Sec. 3.1-3.3: sum g, c g, sum f, c f, c c f), so
-//                 J = diag(1 - 1/tau) + D M and J^T l = diag(1 - 1/tau) l +
-//                 M^T D^T l: nine derivatives along directions d_k with
-//                 M d_k = e_k give D^T l (plus up to two for the porosity
-//                 and wall temperature), one thread per (node, pass);
-//   k_adj_gather: the transpose of pull streaming: each stored value
-//                 collects the adjoints of every node that pulled it (its
-//                 downstream neighbour, the wall nodes whose x_f or x_ff it
-//                 feeds), deterministically, without atomics.
+// adjoint runs the steps backwards, one launch a step (k_adj_step): the thread
+// of interior node s pulls its 17 values of the state again, and takes the
+// adjoint of everything computed from them -- its own collision and, beside a
+// wall, the collisions of the up to three wall nodes whose x_f it is -- back
+// through the moments to the 17 pulled values (reverse mode, by hand: about
+// three times the operations of the step).  The transpose of pull streaming
+// is then a store of each adjoint at the place it was pulled from: every
+// place is pulled by at most one interior node, so no two threads write the
+// same word and the result does not depend on their order.
 // States are recomputed from checkpoints kept every ceil(sqrt(n)) steps.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -32,6 +24,7 @@
 #include <string>
 #include <vector>
 
+#include "lbm_core.cuh"
 #include "lbm_handle.h"
 #include "lbm_host.h"
 #include "lbm_internal.h"
@@ -43,181 +36,413 @@ constexpr int kAdjBlock = 128;
 template <class R>
 __device__ __forceinline__ long long at_of(const KConst<R>& k, int x, int y) { return (long long)y * k.pitch + x; }
 
-// Directions d_k in the space of the 17 pulled values (f_1..f_8, h_0..h_8)
-// with M d_k = e_k for the moment sums k = 0 sum h, 1 sum_x c_x h,
-// 2 sum c_y h, 3 sum f, 4 sum c_x f, 5 sum c_y f, 6 sum c_x^2 f,
-// 7 sum c_y^2 f, 8 sum c_x c_y f (M: row k holds the weights of sum k).
-__device__ __forceinline__ float moment_dir(int k, int q) {
-    if (q >= 8) {
-        const int i = q - 8;
-        if (k == 0) return i == 0 ? 1.f : 0.f;
-        if (k == 1) return i == 1 ? 0.5f : (i == 3 ? -0.5f : 0.f);
-        if (k == 2) return i == 2 ? 0.5f : (i == 4 ? -0.5f : 0.f);
-        return 0.f;
+// Adjoint of the state a collision is computed from, T and p folded into th
+// and ep.
+template <class R>
+struct StateBar {
+    R th, ux, uy, Fx, Fy, ep, Sxx, Syy, Sxy, gx, gy;
+};
+// Adjoint of a node's porosity constants: e itself, 1/e, and the drag
+// coefficients a1 = e nu/K, a2 = e F_e/sqrt(K).
+template <class R>
+struct CellBar {
+    R e, ie, a1, a2;
+};
+
+// What the backward pass needs of a node's moments (node_moments' names).
+template <class R>
+struct AdjState {
+    R e, ie, a1, a2, c0, c1;           // porosity and its constants
+    R th, T, Gy, vx, vy, vm, rs, iden; // rs: sqrt(c0^2 + c1 |v|)
+    R ux, uy, um, drag, Fx, Fy, uu, ep;
+    R Sxx, Syy, Sxy, Px, Py, Nx, Ny, ia, id, t, gx, gy;
+};
+
+// Collision adjoint: adds to B and C what the outputs' adjoints lf (flow) and
+// lh (thermal) give for f^eq, g^eq of the state, scaled by sF, sT, and, with
+// SOURCES, for F_i, P_i + Q_i (lbm_core.cuh: core_emit with S explicit).
+template <bool SOURCES, class R>
+__device__ __forceinline__ void emit_adjoint(const KConst<R>& k, R ie, R sF, R sT, R ux, R uy, R Fx, R Fy, R ep, R T,
+                                             R gx, R gy, const R* lf, const R* lh, StateBar<R>& B, CellBar<R>& C) {
+    const R w1 = R(1) / R(9), w5 = w_diag<R>(), w0 = R(4) / R(9);
+    const R third = R(1) / R(3);
+    {
+        const R a1 = w1 * lf[1], a2 = w1 * lf[2], a3 = w1 * lf[3], a4 = w1 * lf[4];
+        const R a5 = w5 * lf[5], a6 = w5 * lf[6], a7 = w5 * lf[7], a8 = w5 * lf[8];
+        const R d = (a5 + a7) + (a6 + a8), x13 = a1 + a3, y24 = a2 + a4;
+        const R LE = x13 + y24 + d;
+        const R Qx = x13 + d - third * LE, Qy = y24 + d - third * LE, Q2 = (a5 + a7) - (a6 + a8);
+        const R Dx = (a1 - a3) + (a5 - a7) + (a8 - a6), Dy = (a2 - a4) + (a5 - a7) + (a6 - a8);
+        B.ep += R(3) * sF * LE;
+        const R fS = R(1.5) * k.rho0 * k.A * sF;
+        B.Sxx += fS * Qx;
+        B.Syy += fS * Qy;
+        B.Sxy += R(2) * fS * Q2;
+        const R c2 = R(4.5) * k.rho0 * sF, cF = SOURCES ? R(9) * k.rho0 * k.kf : R(0);
+        const R tx = ie * (R(2) * c2 * ux + cF * Fx), ty = ie * (R(2) * c2 * uy + cF * Fy);
+        const R fu = R(3) * k.rho0 * sF;
+        B.ux += Qx * tx + Q2 * ty + fu * Dx;
+        B.uy += Qy * ty + Q2 * tx + fu * Dy;
+        C.ie += c2 * (ux * ux * Qx + uy * uy * Qy + R(2) * ux * uy * Q2);
+        if constexpr (SOURCES) {
+            const R fF = R(3) * k.rho0 * k.kf;
+            B.Fx += cF * ie * (ux * Qx + uy * Q2) + fF * Dx;
+            B.Fy += cF * ie * (uy * Qy + ux * Q2) + fF * Dy;
+            C.ie += cF * (ux * Fx * Qx + uy * Fy * Qy + (ux * Fy + uy * Fx) * Q2);
+        }
     }
-    const int i = q + 1;
-    const bool axis13 = i == 1 || i == 3, axis24 = i == 2 || i == 4, diag = i >= 5;
-    switch (k) {
-    case 3: return axis13 || axis24 ? 0.5f : -0.25f;            // sum f
-    case 4: return i == 1 ? 0.5f : (i == 3 ? -0.5f : 0.f);      // sum c_x f
-    case 5: return i == 2 ? 0.5f : (i == 4 ? -0.5f : 0.f);      // sum c_y f
-    case 6: return axis24 ? -0.5f : (diag ? 0.25f : 0.f);       // sum c_x^2 f
-    case 7: return axis13 ? -0.5f : (diag ? 0.25f : 0.f);       // sum c_y^2 f
-    case 8: return diag ? ((i == 5 || i == 7) ? 0.25f : -0.25f) : 0.f;  // sum c_x c_y f
-    default: return 0.f;
+    {
+        const R a1 = w1 * lh[1], a2 = w1 * lh[2], a3 = w1 * lh[3], a4 = w1 * lh[4];
+        const R a5 = w5 * lh[5], a6 = w5 * lh[6], a7 = w5 * lh[7], a8 = w5 * lh[8];
+        const R d = (a5 + a7) + (a6 + a8), x13 = a1 + a3, y24 = a2 + a4;
+        const R M1 = x13 + y24 + d, M0 = M1 + w0 * lh[0];
+        const R Bx = x13 + d, By = y24 + d, B2 = (a5 + a7) - (a6 + a8);
+        const R Vx = (a1 - a3) + (a5 - a7) + (a8 - a6), Vy = (a2 - a4) + (a5 - a7) + (a6 - a8);
+        const R uu = ux * ux + uy * uy;
+        R Tb = R(0);  // adjoint of T
+        B.th += k.sigma * sT * M0;
+        const R kc = R(4.5) * sT;
+        const R q = ux * ux * Bx + uy * uy * By + R(2) * ux * uy * B2 - third * uu * M0;
+        Tb += kc * ie * q;
+        C.ie += kc * T * q;
+        const R kT2 = R(2) * kc * ie * T;
+        B.ux += kT2 * (ux * Bx + uy * B2 - third * ux * M0);
+        B.uy += kT2 * (uy * By + ux * B2 - third * uy * M0);
+        const R Teb = sT * k.inv_rho0 * (R(3) * M1 - (R(5) / R(3)) * lh[0]);  // adjoint of T eps p
+        Tb += ep * Teb;
+        B.ep += T * Teb;
+        const R Kb = ux * Vx + uy * Vy;
+        R K = R(3) * sT * T, hg = k.sigma * k.B * sT;
+        Tb += R(3) * sT * Kb;
+        if constexpr (SOURCES) {
+            const R W = R(3) * k.kT, b6 = R(6) * k.kT, ug = b6 * R(0.5) * (ie - k.inv_sigma), gu = ux * gx + uy * gy;
+            K += ug * gu + W * k.Q * k.inv_sigma;
+            hg += W * k.inv_rho0 * ep;
+            B.ep += W * k.inv_rho0 * (gx * Vx + gy * Vy);
+            B.Fx += W * T * Vx;
+            B.Fy += W * T * Vy;
+            Tb += W * (Fx * Vx + Fy * Vy);
+            const R uk = ug * Kb;
+            B.ux += uk * gx;
+            B.uy += uk * gy;
+            B.gx += uk * ux;
+            B.gy += uk * uy;
+            C.ie += R(0.5) * b6 * gu * Kb;
+        }
+        B.ux += K * Vx;
+        B.uy += K * Vy;
+        B.gx += hg * Vx;
+        B.gy += hg * Vy;
+        B.th += Tb;
     }
 }
 
-// Weight of pulled value q in moment sum k (row k of M).
-__device__ __forceinline__ float moment_weight(int k, int q) {
-    if (q >= 8) {
-        const int i = q - 8;
-        return k == 0 ? 1.f : (k == 1 ? float(cx_of(i)) : (k == 2 ? float(cy_of(i)) : 0.f));
-    }
-    const int i = q + 1;
-    const float cx = float(cx_of(i)), cy = float(cy_of(i));
-    switch (k) {
-    case 3: return 1.f;
-    case 4: return cx;
-    case 5: return cy;
-    case 6: return cx * cx;
-    case 7: return cy * cy;
-    case 8: return cx * cy;
-    default: return 0.f;
+// Moments of an interior node (node_moments), every intermediate kept.
+template <class R>
+__device__ __forceinline__ AdjState<R> adjoint_state(const KConst<R>& k, R e, R ay, const R* f, const R* h) {
+    AdjState<R> s;
+    const Cell<R> c = k.eps_field ? field_cell<R>(k, e) : uniform_cell<R>(k);
+    s.e = c.eps;
+    s.ie = c.ie;
+    s.a1 = -c.nnuK;
+    s.a2 = -c.nFK;
+    s.c0 = c.c0;
+    s.c1 = c.c1;
+    s.th = (((h[1] + h[3]) + (h[2] + h[4])) + ((h[5] + h[7]) + (h[6] + h[8])) + h[0]) * k.inv_sigma + k.hq_sigma;
+    s.T = k.T0 + s.th;
+    const R s13 = f[1] + f[3], s24 = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
+    const R d57 = f[5] - f[7], d86 = f[8] - f[6], d58 = s57 + s68;
+    const R mx = (f[1] - f[3]) + (d57 + d86), my = (f[2] - f[4]) + (d57 - d86);
+    s.Gy = k.gbeta * s.th + ay;
+    s.vx = mx * k.inv_rho0 + R(0.5) * s.e * k.ax;
+    s.vy = my * k.inv_rho0 + R(0.5) * s.e * s.Gy;
+    s.vm = lsqrt(s.vx * s.vx + s.vy * s.vy);
+    s.rs = lsqrt(c.c0sq + s.c1 * s.vm);
+    s.iden = lrcp(s.c0 + s.rs);
+    s.ux = s.vx * s.iden;
+    s.uy = s.vy * s.iden;
+    s.um = s.vm * s.iden;
+    s.drag = s.a1 + s.a2 * s.um;
+    s.Fx = s.e * k.ax - s.drag * s.ux;
+    s.Fy = s.e * s.Gy - s.drag * s.uy;
+    s.uu = s.ux * s.ux + s.uy * s.uy;
+    const R uF = s.ux * s.Fx + s.uy * s.Fy;
+    s.ep = k.e1 * (s13 + s24 + d58) + (c.e2 * uF + c.e3 * s.uu);
+    s.Px = s13 + d58 - s.ep;
+    s.Py = s24 + d58 - s.ep;
+    const R Pxy = s57 - s68;
+    const R dx = s.Fx - s.ux, dy = s.Fy - s.uy;
+    s.Sxx = k.invD * (s.Px + c.re * s.ux * dx);
+    s.Syy = k.invD * (s.Py + c.re * s.uy * dy);
+    s.Sxy = k.invD * (Pxy + R(0.5) * c.re * (s.ux * dy + s.uy * dx));
+    const R h57 = h[5] - h[7], h86 = h[8] - h[6];
+    const R hx = (h[1] - h[3]) + (h57 + h86), hy = (h[2] - h[4]) + (h57 - h86);
+    const R qT = k.hq_sigma - s.T;
+    s.Nx = hx + s.ux * qT + R(0.5) * s.T * s.Fx;
+    s.Ny = hy + s.uy * qT + R(0.5) * s.T * s.Fy;
+    const R a = k.a_const + k.a_ep * s.ep, d = a - c.b * s.uu, r = lrcp(a * d);
+    s.ia = d * r;
+    s.id = a * r;
+    s.t = c.b * (s.ux * s.Nx + s.uy * s.Ny) * r;
+    s.gx = s.Nx * s.ia + s.t * s.ux;
+    s.gy = s.Ny * s.ia + s.t * s.uy;
+    return s;
+}
+
+// Adjoint of the moments: from B (adjoint of the state) to the adjoints of the
+// moment sums M = (sum h, c h, sum f, c f, c c f), adding the porosity's to C.
+template <class R>
+struct SumsBar {
+    R h0, hx, hy, f0, fx, fy, fxx, fyy, fxy;
+};
+template <class R>
+__device__ __forceinline__ SumsBar<R> moments_adjoint(const KConst<R>& k, const AdjState<R>& s, StateBar<R> B,
+                                                      CellBar<R>& C) {
+    SumsBar<R> m;
+    const R ux = s.ux, uy = s.uy, Fx = s.Fx, Fy = s.Fy;
+    const R re = k.rho0 * s.ie, b = R(0.5) * (s.ie - k.inv_sigma);
+    // S = [P + re (u F + F u)/2 - re u u]/D
+    const R qxx = k.invD * B.Sxx, qyy = k.invD * B.Syy, qxy = k.invD * B.Sxy;
+    const R dx = Fx - ux, dy = Fy - uy;
+    m.fxy = qxy;
+    C.ie += k.rho0 * (qxx * ux * dx + qyy * uy * dy + R(0.5) * qxy * (ux * dy + uy * dx));
+    const R rx = re * qxx, ry = re * qyy, rxy = re * qxy;
+    B.ux += rx * (Fx - R(2) * ux) + rxy * (R(0.5) * Fy - uy);
+    B.uy += ry * (Fy - R(2) * uy) + rxy * (R(0.5) * Fx - ux);
+    B.Fx += rx * ux + R(0.5) * rxy * uy;
+    B.Fy += ry * uy + R(0.5) * rxy * ux;
+    // grad T = N/a + t u, t = b u.N/(a d), d = a - b |u|^2, a = a_const + a_ep ep
+    const R tb = ux * B.gx + uy * B.gy, ng = s.Nx * B.gx + s.Ny * B.gy;
+    const R uN = ux * s.Nx + uy * s.Ny, iad = s.ia * s.id;
+    const R nb = b * iad * tb;             // adjoint of u.N
+    const R db = -s.t * s.id * tb;         // of d
+    const R ab = -s.ia * s.ia * ng - s.t * s.ia * tb + db;  // of a
+    const R bb = uN * iad * tb - s.uu * db;                 // of b
+    C.ie += R(0.5) * bb;
+    R uub = -b * db;                       // of |u|^2
+    R epb = B.ep + k.a_ep * ab - (qxx + qyy);
+    const R Nxb = s.ia * B.gx + nb * ux, Nyb = s.ia * B.gy + nb * uy;
+    B.ux += s.t * B.gx + nb * s.Nx;
+    B.uy += s.t * B.gy + nb * s.Ny;
+    m.hx = Nxb;
+    m.hy = Nyb;
+    // N = c h + u (Q/2 sigma - T) + T F/2
+    const R qT = k.hq_sigma - s.T, hT = R(0.5) * s.T;
+    B.ux += qT * Nxb;
+    B.uy += qT * Nyb;
+    B.Fx += hT * Nxb;
+    B.Fy += hT * Nyb;
+    R thb = B.th + R(0.5) * (Fx * Nxb + Fy * Nyb) - (ux * Nxb + uy * Nyb);
+    // ep = e1 sum f + e2 u.F + e3 |u|^2
+    const R e2 = k.e2_ie * s.ie, e3 = k.e3_ie * s.ie;
+    m.f0 = k.e1 * epb;
+    m.fxx = qxx;
+    m.fyy = qyy;
+    const R uFb = e2 * epb;
+    uub += e3 * epb;
+    C.ie += epb * (k.e2_ie * (ux * Fx + uy * Fy) + k.e3_ie * s.uu);
+    B.ux += uFb * Fx + R(2) * uub * ux;
+    B.uy += uFb * Fy + R(2) * uub * uy;
+    B.Fx += uFb * ux;
+    B.Fy += uFb * uy;
+    // F = e a - (a1 + a2 |u|) u
+    const R dragb = -(B.Fx * ux + B.Fy * uy);
+    B.ux -= s.drag * B.Fx;
+    B.uy -= s.drag * B.Fy;
+    C.e += k.ax * B.Fx + s.Gy * B.Fy;
+    R Gyb = s.e * B.Fy;
+    C.a1 += dragb;
+    C.a2 += s.um * dragb;
+    const R umb = s.a2 * dragb;
+    // u = v/den, |u| = |v|/den, den = c0 + sqrt(c0^2 + c1 |v|), c0 = (1 + a1/2)/2, c1 = a2/2
+    const R denb = -s.iden * (ux * B.ux + uy * B.uy + s.um * umb);
+    const R rb = R(0.5) * denb * lrcp(s.rs);
+    C.a1 += R(0.25) * (denb + R(2) * s.c0 * rb);
+    C.a2 += R(0.5) * s.vm * rb;
+    const R vmb = s.iden * umb + s.c1 * rb;
+    // |v| is not differentiable at 0, but there it only enters times v: 0
+    const R vs = s.vm > R(0) ? vmb * lrcp(s.vm) : R(0);
+    const R vxb = s.iden * B.ux + vs * s.vx, vyb = s.iden * B.uy + vs * s.vy;
+    m.fx = k.inv_rho0 * vxb;
+    m.fy = k.inv_rho0 * vyb;
+    C.e += R(0.5) * (k.ax * vxb + s.Gy * vyb);
+    Gyb += R(0.5) * s.e * vyb;
+    thb += k.gbeta * Gyb;
+    m.h0 = k.inv_sigma * thb;
+    return m;
+}
+
+// d e-total of a node's porosity from its constants' adjoints: 1/e, and with
+// q = 1/e - 1, a1 = A1 q^2, a2 = A2 q/e (field_cell).
+template <class R>
+__device__ __forceinline__ R porosity_adjoint(const KConst<R>& k, R ie, const CellBar<R>& C) {
+    const R q = ie - R(1), ie2 = ie * ie;
+    return C.e - ie2 * (C.ie - R(2) * k.nnuK_q2 * q * C.a1 - k.nFK_q * (q + ie) * C.a2);
+}
+
+// T(x_ff) adjoints waiting at node (x, y): its thermal value along c_i is
+// pulled by s = (x, y) + c_i, and the adiabatic wall nodes whose x_ff is s left
+// theirs in Vff.
+template <class R>
+__device__ __forceinline__ R pending_ff(const KConst<R>& k, const R* __restrict__ Vff, int sx, int sy) {
+    const bool wW = k.bc[SW] != BC_PERIODIC, wE = k.bc[SE] != BC_PERIODIC, wS = k.bc[SS] != BC_PERIODIC,
+               wN = k.bc[SN] != BC_PERIODIC;
+    if (!wW) sx = sx < 0 ? sx + k.nx : (sx >= k.nx ? sx - k.nx : sx);
+    if (!wS) sy = sy < 0 ? sy + k.ny : (sy >= k.ny ? sy - k.ny : sy);
+    const bool inx = wW ? sx >= 1 && sx <= k.nx - 2 : true, iny = wS ? sy >= 1 && sy <= k.ny - 2 : true;
+    if (!inx || !iny) return R(0);
+    R v = R(0);
+    const bool W2 = wW && sx == 2, E2 = wE && sx == k.nx - 3, S2 = wS && sy == 2, N2 = wN && sy == k.ny - 3;
+    if (W2) v += Vff[at_of(k, 0, sy)];
+    if (E2) v += Vff[at_of(k, k.nx - 1, sy)];
+    if (S2) v += Vff[at_of(k, sx, 0)];
+    if (N2) v += Vff[at_of(k, sx, k.ny - 1)];
+    if (W2 && S2) v += Vff[at_of(k, 0, 0)];
+    if (E2 && S2) v += Vff[at_of(k, k.nx - 1, 0)];
+    if (W2 && N2) v += Vff[at_of(k, 0, k.ny - 1)];
+    if (E2 && N2) v += Vff[at_of(k, k.nx - 1, k.ny - 1)];
+    return v * k.inv_sigma;
+}
+
+// Adjoints of node (x, y)'s 17 post-collision values.
+template <class R>
+__device__ __forceinline__ void load_lambda(const KConst<R>& k, const R* __restrict__ lam, const R* __restrict__ Vff,
+                                            bool ff, int x, int y, R* lf, R* lh) {
+    const R* l = lam + at_of(k, x, y);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) lf[i] = l[(long long)(i - 1) * k.plane];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) lh[i] = l[(long long)(8 + i) * k.plane];
+    lf[0] = R(0);
+    // x_ff lies two nodes inside a wall: only nodes within three of one collect
+    if (ff && (x <= 3 || y <= 3 || x >= k.nx - 4 || y >= k.ny - 4)) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) lh[i] += pending_ff(k, Vff, x + cx_of(i), y + cy_of(i));
     }
 }
 
-// Passes of the local transposed Jacobian: 0..8 the moment directions d_k,
-// 9 porosity at the source node, 10 porosity at the node (wall nodes only),
-// 11 T(x_ff) (adiabatic walls), 12 the Dirichlet T_b.
-constexpr int kAdjPasses = 13;
+// One adjoint step.  state: s_n; lam, Vff: adjoints of s_{n+1}; lam_prev,
+// Vff_prev: those of s_n (places no interior node pulls are never written and
+// stay 0).  Threads run over the interior nodes, x fastest.  ff: some wall is
+// adiabatic.  early: the state was complete before the previous launch began,
+// so it may be read before the grid dependency is resolved.
+// Bound: 256^2 FP32 fits L2 and one wave of warps; the step takes about the
+// latency of its chain (loads, ~700 dependent operations, stores).  Blocks of
+// 64 threads (32 in FP64, whose pipe serves two lanes a cycle and SM) spread
+// small lattices over more SMs.  Before, 9 to 11 forward-mode passes a node in
+// a thread each, then a combining and a gathering launch: whole calls with 256
+// steps at 256^2 FP32 took 38.0 ms against 8.8 ms, with 100 steps at 65 x 49
+// FP64 45.7 against 10.8 ms (forward and recomputed steps included).
+template <class R> struct AdjLaunch { static constexpr int block = 64, blocks = 8; };
+template <> struct AdjLaunch<double> { static constexpr int block = 32, blocks = 8; };
 
-// One pass per thread (blockIdx.z = pass j): the directional derivative of
-// node (x, y)'s update along its direction, dotted with lambda_{n+1}(x).
-// D[j][x]: for j < 9 (D^T l)_j = l . J d_j - l . (diag(1 - 1/tau) d_j);
-// otherwise l . (dout / d input j), 0 where the input does not exist.
-template <class R, class S>
-__global__ void __launch_bounds__(kAdjBlock)
-k_adj_pass(const __grid_constant__ KConst<R> k, const S* __restrict__ state, const R* __restrict__ lam,
-           R* __restrict__ D) {
-    const int x = blockIdx.x * kAdjBlock + threadIdx.x;
-    const int y = blockIdx.y;
-    const int j = blockIdx.z;
-    if (x >= k.nx) return;
-    const long long a = at_of(k, x, y);
-    const WallInfo w = classify(k, x, y);
-    const bool field = k.eps_field != nullptr;
-    const bool used = j < 9 || (j == 9 && field) || (j == 10 && field && w.wall) ||
-                      (j == 11 && w.wall && w.tside < 0) || (j == 12 && w.wall && w.tside >= 0);
-    if (!used) {
-        D[j * k.plane + a] = R(0);
-        return;
-    }
-    const int xs = w.wall ? w.xs : x, ys = w.wall ? w.ys : y;
+template <class R, class S, bool TAU1>
+__global__ void __launch_bounds__(AdjLaunch<R>::block, AdjLaunch<R>::blocks)
+k_adj_step(const __grid_constant__ KConst<R> k, const S* __restrict__ state, const R* __restrict__ lam,
+           const R* __restrict__ Vff, R* __restrict__ lam_prev, R* __restrict__ Vff_prev, double* __restrict__ g_eps,
+           double* __restrict__ g_tb, bool ff, bool early) {
+    if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool wx = k.bc[SW] != BC_PERIODIC, wy = k.bc[SS] != BC_PERIODIC;
+    const int x0 = wx ? 1 : 0, y0 = wy ? 1 : 0, nxi = k.nx - 2 * x0, nyi = k.ny - 2 * y0;
+    const long long n = (long long)blockIdx.x * AdjLaunch<R>::block + threadIdx.x;
+    const bool live = n < (long long)nxi * nyi;
+    const int yi = live ? (int)(n / nxi) : 0;
+    const int x = x0 + (live ? (int)(n - (long long)yi * nxi) : 0), y = y0 + yi;
     Pops<R> P;
-    pull(k, state, xs, ys, P);
-    R thff = R(0);
-    if (w.wall && w.tside < 0) thff = (pull_hsum<R, R, S>(k, state, w.xff, w.yff) + R(0.5) * k.Q) * k.inv_sigma;
-    const R thb = (w.wall && w.tside >= 0) ? k.T_bc[w.tside] - k.T0 : R(0);
-    const R eps_s = node_eps(k, xs, ys), eps_x = node_eps(k, x, y);
-    Dual<R> din[17], dout[17];
+    pull(k, state, x, y, P);
+    const AdjState<R> s = adjoint_state(k, node_eps(k, x, y), row_ay(k, y), P.f, P.h);
+    if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // only now may the next step's blocks start: their early reads then come
+    // after the launch before this one
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!live) return;
+    StateBar<R> B = {};
+    CellBar<R> C = {};
+    R lf[9], lh[9], vf[9], vh[9];
+    load_lambda(k, lam, Vff, ff, x, y, lf, lh);
+    emit_adjoint<true>(k, s.ie, R(1) - k.omf, R(1) - k.omT, s.ux, s.uy, s.Fx, s.Fy, s.ep, s.T, s.gx, s.gy, lf, lh, B, C);
 #pragma unroll
-    for (int i = 1; i < 9; ++i) din[i - 1] = Dual<R>(P.f[i], j < 9 ? R(moment_dir(j, i - 1)) : R(0));
-#pragma unroll
-    for (int i = 0; i < 9; ++i) din[8 + i] = Dual<R>(P.h[i], j < 9 ? R(moment_dir(j, 8 + i)) : R(0));
-    const Dual<R> des(eps_s, j == 9 ? R(1) : R(0));
-    // an interior node's own porosity is its source porosity
-    const Dual<R> dex = w.wall ? Dual<R>(eps_x, j == 10 ? R(1) : R(0)) : des;
-    const Dual<R> dff(thff, j == 11 ? R(1) : R(0));
-    const Dual<R> dtb(thb, j == 12 ? R(1) : R(0));
-    node_update_generic(k, w, din, des, dex, dff, dtb, row_ay(k, ys), row_ay(k, y), dout);
-    R acc = R(0);
-#pragma unroll
-    for (int q = 0; q < 17; ++q) {
-        const R l = lam[q * k.plane + a];
-        acc += dout[q].d * l;
-        if (j < 9) acc -= (q < 8 ? k.omf : k.omT) * l * R(moment_dir(j, q));
+    for (int i = 0; i < 9; ++i) {
+        vf[i] = TAU1 ? R(0) : k.omf * lf[i];
+        vh[i] = TAU1 ? R(0) : k.omT * lh[i];
     }
-    D[j * k.plane + a] = acc;
-}
-
-// V = J^T l = diag(1 - 1/tau) l + M^T D^T l per node, the x_ff adjoint, and
-// the porosity / wall-temperature gradient contributions.
-template <class R>
-__global__ void __launch_bounds__(kAdjBlock)
-k_adj_combine(const __grid_constant__ KConst<R> k, const R* __restrict__ lam, const R* __restrict__ D,
-              R* __restrict__ V, R* __restrict__ Vff, double* __restrict__ g_eps, double* __restrict__ g_epsf,
-              double* __restrict__ g_tb) {
-    const int x = blockIdx.x * kAdjBlock + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= k.nx) return;
-    const long long a = at_of(k, x, y);
-    R dtl[9];
-#pragma unroll
-    for (int m = 0; m < 9; ++m) dtl[m] = D[m * k.plane + a];
-#pragma unroll
-    for (int q = 0; q < 17; ++q) {
-        R v = (q < 8 ? k.omf : k.omT) * lam[q * k.plane + a];
-#pragma unroll
-        for (int m = 0; m < 9; ++m) v += R(moment_weight(m, q)) * dtl[m];
-        V[q * k.plane + a] = v;
-    }
-    Vff[a] = D[11 * k.plane + a];
-    const long long c = (long long)y * k.nx + x;
-    const R v_es = D[9 * k.plane + a];
-    if (!classify(k, x, y).wall) {
-        g_eps[c] += double(v_es);
-    } else {
-        g_eps[c] += double(D[10 * k.plane + a]);
-        g_epsf[c] += double(v_es);
-        g_tb[c] += double(D[12 * k.plane + a]);
-    }
-}
-
-// Does some wall node b satisfy (x_f or x_ff of b) == s?  Checked only near
-// the walls (sources of both lie at most two nodes inside).
-template <class R>
-__device__ __forceinline__ bool near_wall(const KConst<R>& k, int sx, int sy) {
-    return (k.bc[SW] != BC_PERIODIC && (sx <= 2 || sx >= k.nx - 3)) ||
-           (k.bc[SS] != BC_PERIODIC && (sy <= 2 || sy >= k.ny - 3));
-}
-
-// Transpose of pull streaming: lambda_n(y, q) = sum of V_q over the nodes that
-// pulled value (y, q) during step n -> n+1.
-template <class R>
-__global__ void __launch_bounds__(kAdjBlock)
-k_adj_gather(const __grid_constant__ KConst<R> k, const R* __restrict__ V, const R* __restrict__ Vff,
-             R* __restrict__ lam_prev) {
-    const int x = blockIdx.x * kAdjBlock + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= k.nx) return;
-    const bool px = k.bc[SW] == BC_PERIODIC, py = k.bc[SS] == BC_PERIODIC;
+    // wall nodes whose x_f this node is
+    const int bx = wx && x == 1 ? 0 : (wx && x == k.nx - 2 ? k.nx - 1 : -1);
+    const int by = wy && y == 1 ? 0 : (wy && y == k.ny - 2 ? k.ny - 1 : -1);
+    if (bx >= 0 || by >= 0) {
 #pragma unroll 1
-    for (int q = 0; q < 17; ++q) {
-        const int i = q < 8 ? q + 1 : q - 8;
-        int sx = x + cx_of(i), sy = y + cy_of(i);  // the node that pulls (x, y) along c_i
-        R acc = R(0);
-        if (px) sx = (sx + k.nx) % k.nx;
-        if (py) sy = (sy + k.ny) % k.ny;
-        if (sx >= 0 && sx < k.nx && sy >= 0 && sy < k.ny) {
-            const WallInfo ws = classify(k, sx, sy);
-            if (!ws.wall) acc += V[q * k.plane + at_of(k, sx, sy)];
-            if (near_wall(k, sx, sy)) {
-                for (int d = 1; d < 9; ++d) {
-                    for (int m = 1; m <= 2; ++m) {
-                        if (m == 2 && q < 8) continue;  // x_ff feeds only T
-                        const int bx = sx - m * cx_of(d), by = sy - m * cy_of(d);
-                        if (bx < 0 || bx >= k.nx || by < 0 || by >= k.ny) continue;
-                        const WallInfo wb = classify(k, bx, by);
-                        if (!wb.wall) continue;
-                        if (m == 1 && wb.xs == sx && wb.ys == sy) acc += V[q * k.plane + at_of(k, bx, by)];
-                        if (m == 2 && wb.tside < 0 && wb.xff == sx && wb.yff == sy)
-                            acc += Vff[at_of(k, bx, by)] * k.inv_sigma;
-                    }
+        for (int m = 0; m < 3; ++m) {
+            const int X = m == 1 ? x : bx, Y = m == 0 ? y : by;  // W/E side, S/N side, corner
+            if (X < 0 || Y < 0) continue;
+            const WallInfo w = classify(k, X, Y);
+            load_lambda(k, lam, Vff, ff, X, Y, lf, lh);
+            const R eb = k.eps_field ? k.eps_field[(long long)Y * k.nx + X] : k.eps;
+            const Cell<R> cb = k.eps_field ? field_cell<R>(k, eb) : uniform_cell<R>(k);
+            R thb = R(0), thff = R(0);
+            if (w.tside >= 0) {
+                thb = k.T_bc[w.tside] - k.T0;
+            } else {
+                thff = (pull_hsum<R, R, S>(k, state, w.xff, w.yff) + R(0.5) * k.Q) * k.inv_sigma;
+                thb = (R(4) * s.th - thff) * (R(1) / R(3));
+            }
+            const bool cutx = w.tside < 0 && w.fixgx, cuty = w.tside < 0 && w.fixgy;
+            const R gx = cutx ? R(0) : s.gx, gy = cuty ? R(0) : s.gy;
+            const R ux = k.u_bc[w.uside][0], uy = k.u_bc[w.uside][1], um = k.u_abs[w.uside];
+            const R Gy = k.gbeta * thb + row_ay(k, Y), drag = -cb.nnuK - cb.nFK * um;
+            const R Fx = cb.eps * k.ax - drag * ux, Fy = cb.eps * Gy - drag * uy;
+            const R p = s.ep * s.ie, ep = k.eps_field ? p * cb.eps : s.ep;
+            StateBar<R> D = {};
+            CellBar<R> E = {};
+            emit_adjoint<true>(k, cb.ie, R(1), R(1), ux, uy, Fx, Fy, ep, k.T0 + thb, gx, gy, lf, lh, D, E);
+            // F = e a - (a1 + a2 |u_b|) u_b with u_b given
+            const R dragb = -(D.Fx * ux + D.Fy * uy);
+            E.a1 += dragb;
+            E.a2 += um * dragb;
+            E.e += k.ax * D.Fx + Gy * D.Fy;
+            const R thbb = D.th + cb.eps * k.gbeta * D.Fy;
+            if (w.tside >= 0) {
+                g_tb[(long long)Y * k.nx + X] += double(thbb);
+            } else {
+                B.th += (R(4) / R(3)) * thbb;
+                Vff_prev[at_of(k, X, Y)] = -(R(1) / R(3)) * thbb;
+            }
+            if (k.eps_field) {
+                B.ep += D.ep * s.ie * cb.eps;
+                C.ie += D.ep * s.ep * cb.eps;
+                E.e += D.ep * p;
+                g_eps[(long long)Y * k.nx + X] += double(porosity_adjoint(k, cb.ie, E));
+            } else {
+                B.ep += D.ep;
+            }
+            B.Sxx += D.Sxx;
+            B.Syy += D.Syy;
+            B.Sxy += D.Sxy;
+            if (!cutx) B.gx += D.gx;
+            if (!cuty) B.gy += D.gy;
+            if constexpr (!TAU1) {
+                // (1 - 1/tau)[f(x_f) - f^eq(x_f)]
+                emit_adjoint<false>(k, s.ie, -k.omf, -k.omT, s.ux, s.uy, s.Fx, s.Fy, s.ep, s.T, s.gx, s.gy, lf, lh, B, C);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    vf[i] += k.omf * lf[i];
+                    vh[i] += k.omT * lh[i];
                 }
             }
         }
-        lam_prev[q * k.plane + at_of(k, x, y)] = acc;
+    }
+    const SumsBar<R> m = moments_adjoint(k, s, B, C);
+    if (k.eps_field) g_eps[(long long)y * k.nx + x] += double(porosity_adjoint(k, s.ie, C));
+    // pulled value i of this node came from (x, y) - c_i
+    const int xm = x == 0 ? k.nx - 1 : x - 1, xp = x == k.nx - 1 ? 0 : x + 1;
+    const int ym = y == 0 ? k.ny - 1 : y - 1, yp = y == k.ny - 1 ? 0 : y + 1;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int cx = cx_of(i), cy = cy_of(i);
+        R* o = lam_prev + at_of(k, cx > 0 ? xm : (cx < 0 ? xp : x), cy > 0 ? ym : (cy < 0 ? yp : y));
+        const R rx = R(cx), ry = R(cy);
+        if (i > 0)
+            o[(long long)(i - 1) * k.plane] = vf[i] + m.f0 + rx * m.fx + ry * m.fy + rx * rx * m.fxx + ry * ry * m.fyy + rx * ry * m.fxy;
+        o[(long long)(8 + i) * k.plane] = vh[i] + m.h0 + rx * m.hx + ry * m.hy;
     }
 }
 
@@ -243,23 +468,25 @@ __global__ void k_adj_seed(const __grid_constant__ KConst<R> k, const double* __
     }
 }
 
-// D: scratch of kAdjPasses planes.
 template <class R, class S>
-cudaError_t launch_adj_local(const KConst<R>& k, const S* state, const R* lam, R* D, R* V, R* Vff, double* g_eps,
-                             double* g_epsf, double* g_tb, cudaStream_t st) {
-    const unsigned bx = (unsigned)((k.nx + kAdjBlock - 1) / kAdjBlock);
-    k_adj_pass<R, S><<<dim3(bx, (unsigned)k.ny, kAdjPasses), kAdjBlock, 0, st>>>(k, state, lam, D);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_adj_combine<R><<<dim3(bx, (unsigned)k.ny), kAdjBlock, 0, st>>>(k, lam, D, V, Vff, g_eps, g_epsf, g_tb);
-    return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t launch_adj_gather(const KConst<R>& k, const R* V, const R* Vff, R* lam_prev, cudaStream_t st) {
-    const dim3 grid((unsigned)((k.nx + kAdjBlock - 1) / kAdjBlock), (unsigned)k.ny);
-    k_adj_gather<R><<<grid, kAdjBlock, 0, st>>>(k, V, Vff, lam_prev);
-    return cudaGetLastError();
+cudaError_t launch_adj_step(const KConst<R>& k, const S* state, const R* lam, const R* Vff, R* lam_prev, R* Vff_prev,
+                            double* g_eps, double* g_tb, bool early, cudaStream_t st) {
+    const int wx = k.bc[SW] != BC_PERIODIC ? 1 : 0, wy = k.bc[SS] != BC_PERIODIC ? 1 : 0;
+    const long long n = (long long)(k.nx - 2 * wx) * (k.ny - 2 * wy);
+    bool ff = false;
+    for (int s = 0; s < 4; ++s) ff = ff || k.bc[s] == BC_ADIABATIC;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + AdjLaunch<R>::block - 1) / AdjLaunch<R>::block));
+    cfg.blockDim = dim3(AdjLaunch<R>::block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (k.omf == R(0) && k.omT == R(0))
+        return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, true>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ff, early);
+    return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, false>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ff, early);
 }
 
 template <class R>
@@ -330,14 +557,17 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
     char* segs = (char*)alloc(sb * (size_t)K);
     R* lam0 = (R*)alloc(lam_bytes);
     R* lam1 = (R*)alloc(lam_bytes);
-    R* V = (R*)alloc(lam_bytes);
-    R* Vff = (R*)alloc((size_t)k.plane * sizeof(R));
-    R* Dp = (R*)alloc((size_t)lbm::kAdjPasses * k.plane * sizeof(R));  // per-pass products
-    double* g = (double*)alloc(4 * N * sizeof(double));  // g_eps, g_epsf, g_tb, dL/dT
-    if (!ckpt || !segs || !lam0 || !lam1 || !V || !Vff || !Dp || !g)
+    const size_t ff_bytes = (size_t)k.plane * sizeof(R);
+    R* ff0 = (R*)alloc(2 * ff_bytes);  // T(x_ff) adjoints left at the wall nodes, two buffers
+    double* g = (double*)alloc(3 * N * sizeof(double));  // g_eps, g_tb, dL/dT
+    if (!ckpt || !segs || !lam0 || !lam1 || !ff0 || !g)
         return fail_free(LBM_ERR_OOM, "adjoint buffers (checkpoints grow as sqrt(n))");
-    double *g_eps = g, *g_epsf = g + N, *g_tb = g + 2 * N, *dLdT = g + 3 * N;
-    if (cudaMemsetAsync(g, 0, 3 * N * sizeof(double), st) != cudaSuccess) return fail_free(LBM_ERR_CUDA, "memset");
+    R* ff1 = ff0 + k.plane;
+    double *g_eps = g, *g_tb = g + N, *dLdT = g + 2 * N;
+    // lam1 holds 0 where no node ever writes (lam0 is written whole by the seed)
+    if (cudaMemsetAsync(g, 0, 2 * N * sizeof(double), st) != cudaSuccess ||
+        cudaMemsetAsync(lam1, 0, lam_bytes, st) != cudaSuccess || cudaMemsetAsync(ff0, 0, 2 * ff_bytes, st) != cudaSuccess)
+        return fail_free(LBM_ERR_CUDA, "memset");
 
     // forward, keeping a checkpoint at the start of every segment
     const int64_t step0 = h->steps;
@@ -400,27 +630,24 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
             if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, "recompute step");
         }
         for (int64_t t = len - 1; t >= 0; --t) {
-            e = lbm::launch_adj_local(k, (const S*)(segs + sb * (size_t)t), lc, Dp, V, Vff, g_eps, g_epsf, g_tb, st);
-            if (e == cudaSuccess) e = lbm::launch_adj_gather(k, V, Vff, ln, st);
-            if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, std::string("adjoint kernels: ") + cudaGetErrorString(e));
+            // the first launch after the recomputation waits before it reads the state
+            e = lbm::launch_adj_step(k, (const S*)(segs + sb * (size_t)t), lc, ff0, ln, ff1, g_eps, g_tb, t < len - 1, st);
+            if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, std::string("adjoint kernel: ") + cudaGetErrorString(e));
             std::swap(lc, ln);
+            std::swap(ff0, ff1);
         }
     }
     // gradients
-    std::vector<double> hg(3 * N);
-    if (cudaMemcpyAsync(hg.data(), g, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    std::vector<double> hg(N);
+    if ((dloss_deps && cudaMemcpyAsync(dloss_deps, g_eps, N * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
+        cudaMemcpyAsync(hg.data(), g_tb, N * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return fail_free(LBM_ERR_CUDA, "gradient copy");
-    std::vector<double> ge(hg.begin(), hg.begin() + N);
     for (int y = 0; y < p.ny; ++y)
-        for (int x = 0; x < p.nx; ++x) {
+        for (int x = 0; x < p.nx; x += (y == 0 || y == p.ny - 1 || p.nx < 2) ? 1 : p.nx - 1) {
             const HostWall w = host_classify(p, x, y);
-            if (!w.wall) continue;
-            const size_t c = (size_t)y * p.nx + x;
-            ge[(size_t)w.ys * p.nx + w.xs] += hg[N + c];
-            if (w.tside >= 0) dTbc[w.tside] += hg[2 * N + c];
+            if (w.wall && w.tside >= 0) dTbc[w.tside] += hg[(size_t)y * p.nx + x];
         }
-    if (dloss_deps) memcpy(dloss_deps, ge.data(), N * sizeof(double));
     if (dloss_dTbc) memcpy(dloss_dTbc, dTbc, sizeof(dTbc));
     for (void* a : allocs) cudaFreeAsync(a, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) return lbm_handle_fail(h, LBM_ERR_CUDA, "adjoint cleanup");
