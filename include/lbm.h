@@ -132,11 +132,14 @@ typedef struct {
 lbm_status lbm_set_moment_segments(lbm_handle* h, int32_t segments);
 
 /* Step kernel of a population handle (no counterpart in the paper; a
- * launch choice).  FP32 and FP16 lattices walled on all four sides default
+ * launch choice).  FP32 lattices of at least 8 x 8 nodes (any sides) take
+ * their steps in pairs by default, two per launch, each node computed as in
+ * the one-step kernels; the last of an odd number of steps, and smaller
+ * lattices, take a one-step kernel.  FP32 and FP16 lattices walled on all four sides default
  * to staged rows: each block loads the 17 planes its rows pull from into
  * shared memory with tensor copies and waits on them with bounded waits.
  * staged = 0 selects the kernel in which every thread loads its own 17
- * values from global memory; staged = 1 restores the staged kernel
+ * values from global memory, one step per launch; staged = 1 restores the default
  * (LBM_ERR_ARG where it is unavailable: FP64, a periodic side, the moment
  * state, a lattice under 4 x 4, or a CUDA driver without tensor-map encoding).
  * Both kernels run the same per-node arithmetic (results agree to rounding;
@@ -213,7 +216,7 @@ lbm_status lbm_stream_function(lbm_handle* h, double* psi, int on_device, double
 lbm_status lbm_set_force_profile(lbm_handle* h, const double* ay);
 
 /* Advance n >= 0 time steps (stream, rebuild walls, collide; one kernel
- * launch per step).  Asynchronous on the handle's stream.  Returns
+ * launch per step, or per two steps of an FP32 lattice).  Asynchronous on the handle's stream.  Returns
  * LBM_ERR_NONFINITE or LBM_ERR_TIMEOUT if an earlier synchronising call saw
  * the corresponding flag.  FP32 lattices walled on all four sides stage the
  * pulled rows in shared memory with tensor copies and bounded waits. */

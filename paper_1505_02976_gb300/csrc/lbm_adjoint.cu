@@ -141,7 +141,7 @@ __device__ __forceinline__ void emit_adjoint(const KConst<R>& k, R ie, R sF, R s
 template <class R>
 __device__ __forceinline__ AdjState<R> adjoint_state(const KConst<R>& k, R e, R ay, const R* f, const R* h) {
     AdjState<R> s;
-    const Cell<R> c = k.eps_field ? field_cell<R>(k, e) : uniform_cell<R>(k);
+    const Cell<R> c = k.eps_field ? field_cell<R>(k, e) : k.cell;
     s.e = c.eps;
     s.ie = c.ie;
     s.a1 = -c.nnuK;
@@ -377,7 +377,7 @@ k_adj_step(const __grid_constant__ KConst<R> k, const S* __restrict__ state, con
             const WallInfo w = classify(k, X, Y);
             load_lambda(k, lam, Vff, ff, X, Y, lf, lh);
             const R eb = k.eps_field ? k.eps_field[(long long)Y * k.nx + X] : k.eps;
-            const Cell<R> cb = k.eps_field ? field_cell<R>(k, eb) : uniform_cell<R>(k);
+            const Cell<R> cb = k.eps_field ? field_cell<R>(k, eb) : k.cell;
             R thb = R(0), thff = R(0);
             if (w.tside >= 0) {
                 thb = k.T_bc[w.tside] - k.T0;

@@ -233,6 +233,12 @@ lbm_status lbm_create(const lbm_params* p, void* stream, void* workspace, size_t
         h->tma = h->tma_ready;
         h->tma_rows = lbm::tma_rows_default(h->k32);
     }
+    h->sms = 1;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        (void)cudaGetLastError();
+    h->two_steps = p->precision == LBM_F32 && !p->moment_state && lbm::two_steps_supported(h->k32);
     h->msegments = 1;
     if (p->moment_state)
         h->msegments = p->precision == LBM_F64 ? lbm::moment_segments_default(h->k64)
@@ -369,6 +375,16 @@ lbm_status lbm_step(lbm_handle* h, int64_t n) {
     }
     for (int64_t i = 0; i < n; ++i) {
         const int src = h->cur, dst = 1 - h->cur;
+        if (h->two_steps && n - i >= 2) {
+            const cudaError_t e = lbm::launch_two_steps(h->k32, (const float*)h->buf(src), (float*)h->buf(dst),
+                                                        (uint32_t)h->launches, h->sms, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "two-step kernel");
+            h->cur = dst;
+            h->steps += 2;
+            ++i;
+            ++h->launches;
+            continue;
+        }
         if (h->tma) {
             const uint32_t step = (uint32_t)h->steps;
             cudaError_t e = h->prm.precision == LBM_F32
@@ -399,6 +415,7 @@ lbm_status lbm_set_step_staging(lbm_handle* h, int32_t staged) {
     if (staged && !h->tma_ready)
         return fail(h, LBM_ERR_ARG, "staged rows need FP32 or FP16 populations on a lattice walled on all sides");
     h->tma = staged != 0;
+    h->two_steps = staged != 0 && h->prm.precision == LBM_F32 && lbm::two_steps_supported(h->k32);
     return LBM_OK;
 }
 

@@ -88,87 +88,189 @@ __device__ __forceinline__ bool lfinite(float a) { return isfinite(a); }
 __device__ __forceinline__ bool lfinite(double a) { return isfinite(a); }
 __device__ __forceinline__ bool lfinite(float2 a) { return isfinite(a.x) && isfinite(a.y); }
 
-// ------------------------------------------------------------ node constants
+// ------------------------------------------------------------ run constants
+// The packed form takes every constant as a pair of equal values, laid out so
+// in the kernel's parameters: a packed instruction reads its operands as
+// aligned 64-bit pairs, and a pair made from one 32-bit constant costs two
+// moves at each use (ALU instructions a row of pairs of the two-step kernel:
+// 104 with the moves, 70 without; 59.9 -> 58.3 us a step at 2048^2, the FP16
+// step unchanged within 1 %).
+struct PairConst {
+    float2 inv_rho0, hq_sigma, half_Q, eay, half_ax, nnuK_q2, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie, a_ep, a_const, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF, gain, h_sig, h_kQ, h_pT, h_u3, h_uQ, h_g, h_W, h_Wr, inv_sigma, T0, invD, rho0, gbeta, ax, omf, omT;
+    float2 half, nhalf, nthird, nquarter, one, two;  // literals
+    float2 w1, w5f, w5h, w0, pT, n1, n5f;            // weights (core_weights)
+    Cell<float2> cell;
+};
 
-// The run's own constants (uniform porosity), one copy per lane.
-template <class L, class R>
-__device__ __forceinline__ Cell<L> uniform_cell(const KConst<R>& k) {
-    Cell<L> c;
-    c.eps = lset<L>(k.cell.eps);
-    c.ie = lset<L>(k.cell.ie);
-    c.eg = lset<L>(k.cell.eg);
-    c.eax = lset<L>(k.cell.eax);
-    c.heax = lset<L>(k.cell.heax);
-    c.c0 = lset<L>(k.cell.c0);
-    c.c0sq = lset<L>(k.cell.c0sq);
-    c.c1 = lset<L>(k.cell.c1);
-    c.ih = lset<L>(k.cell.ih);
-    c.il = lset<L>(k.cell.il);
-    c.ci = lset<L>(k.cell.ci);
-    c.nnuK = lset<L>(k.cell.nnuK);
-    c.nFK = lset<L>(k.cell.nFK);
-    c.e2 = lset<L>(k.cell.e2);
-    c.e3 = lset<L>(k.cell.e3);
-    c.re = lset<L>(k.cell.re);
-    c.qu = lset<L>(k.cell.qu);
-    c.qF = lset<L>(k.cell.qF);
-    c.cu2 = lset<L>(k.cell.cu2);
-    c.cuF = lset<L>(k.cell.cuF);
-    c.b = lset<L>(k.cell.b);
-    c.nb = lset<L>(k.cell.nb);
-    c.ug = lset<L>(k.cell.ug);
-    c.kc = lset<L>(k.cell.kc);
-    return c;
+// Weights of the outputs: axis, diagonal (flow, thermal), rest, and the rest
+// direction's T p term; all times the storage scale.
+template <class L>
+struct CoreWeights {
+    L w1, w5f, w5h, w0, pT, n1, n5f;  // n1, n5f: -w1, -w5f
+};
+template <class R>
+__host__ __device__ __forceinline__ CoreWeights<R> core_weights(const KConst<R>& k, R scale) {
+    // the flow's own diagonal weight, rounded to nearest: 2 w_1 + 4 w_5 is
+    // then within 7.5e-9 of 1/3, which scales the momentum in each step
+    // (w_diag, fitted to the sum of all nine, is 1.5e-8 off)
+    return {scale * (R(1) / R(9)), scale * (R(1) / R(36)), scale * w_diag<R>(), scale * (R(4) / R(9)), scale * k.h0_pT,
+            -(scale * (R(1) / R(9))), -(scale * (R(1) / R(36)))};
+}
+__device__ __forceinline__ CoreWeights<float2> core_weights(const PairConst& q, float) {
+    return {q.w1, q.w5f, q.w5h, q.w0, q.pT, q.n1, q.n5f};
 }
 
-// Constants at porosity e of a porosity field.  With q = (1 - e)/e the
-// Kozeny-Carman and Ergun relations (Sec. 2) collapse to eps nu/K = a q^2 and
-// eps F_eps/sqrt(K) = b q/e: one reciprocal, no square root.
-template <class L, class R>
-__device__ __forceinline__ Cell<L> field_cell(const KConst<R>& k, L e) {
+// The pairs of a run's constants; scale: the storage scale of the outputs.
+inline PairConst make_pair_const(const KConst<float>& k, float scale) {
+    PairConst q;
+    auto two = [](float v) { return make_float2(v, v); };
+    q.inv_rho0 = two(k.inv_rho0);
+    q.hq_sigma = two(k.hq_sigma);
+    q.half_Q = two(k.half_Q);
+    q.eay = two(k.eay);
+    q.half_ax = two(k.half_ax);
+    q.nnuK_q2 = two(k.nnuK_q2);
+    q.nFK_q = two(k.nFK_q);
+    q.e1 = two(k.e1);
+    q.e1_lo = two(k.e1_lo);
+    q.e2_ie = two(k.e2_ie);
+    q.e3_ie = two(k.e3_ie);
+    q.qu_ie = two(k.qu_ie);
+    q.qF_ie = two(k.qF_ie);
+    q.cu2_ie = two(k.cu2_ie);
+    q.cuF_ie = two(k.cuF_ie);
+    q.b_0 = two(k.b_0);
+    q.ug_b = two(k.ug_b);
+    q.kc_ie = two(k.kc_ie);
+    q.a_ep = two(k.a_ep);
+    q.a_const = two(k.a_const);
+    q.aS = two(k.aS);
+    q.aS2 = two(k.aS2);
+    q.f_ScS = two(k.f_ScS);
+    q.f_ScS2 = two(k.f_ScS2);
+    q.fA_ep = two(k.fA_ep);
+    q.f_cu = two(k.f_cu);
+    q.f_cF = two(k.f_cF);
+    q.gain = two(k.gain);
+    q.h_sig = two(k.h_sig);
+    q.h_kQ = two(k.h_kQ);
+    q.h_pT = two(k.h_pT);
+    q.h_u3 = two(k.h_u3);
+    q.h_uQ = two(k.h_uQ);
+    q.h_g = two(k.h_g);
+    q.h_W = two(k.h_W);
+    q.h_Wr = two(k.h_Wr);
+    q.inv_sigma = two(k.inv_sigma);
+    q.T0 = two(k.T0);
+    q.invD = two(k.invD);
+    q.rho0 = two(k.rho0);
+    q.gbeta = two(k.gbeta);
+    q.ax = two(k.ax);
+    q.omf = two(k.omf);
+    q.omT = two(k.omT);
+    q.half = two(0.5f);
+    q.nhalf = two(-0.5f);
+    q.nthird = two(-1.0f / 3.0f);
+    q.nquarter = two(-0.25f);
+    q.one = two(1.0f);
+    q.two = two(2.0f);
+    const CoreWeights<float> w = core_weights(k, scale);
+    q.w1 = two(w.w1);
+    q.w5f = two(w.w5f);
+    q.w5h = two(w.w5h);
+    q.w0 = two(w.w0);
+    q.pT = two(w.pT);
+    q.n1 = two(w.n1);
+    q.n5f = two(w.n5f);
+    q.cell.eps = two(k.cell.eps);
+    q.cell.ie = two(k.cell.ie);
+    q.cell.eg = two(k.cell.eg);
+    q.cell.eax = two(k.cell.eax);
+    q.cell.heax = two(k.cell.heax);
+    q.cell.c0 = two(k.cell.c0);
+    q.cell.c0sq = two(k.cell.c0sq);
+    q.cell.c1 = two(k.cell.c1);
+    q.cell.ih = two(k.cell.ih);
+    q.cell.il = two(k.cell.il);
+    q.cell.ci = two(k.cell.ci);
+    q.cell.nnuK = two(k.cell.nnuK);
+    q.cell.nFK = two(k.cell.nFK);
+    q.cell.e2 = two(k.cell.e2);
+    q.cell.e3 = two(k.cell.e3);
+    q.cell.re = two(k.cell.re);
+    q.cell.qu = two(k.cell.qu);
+    q.cell.qF = two(k.cell.qF);
+    q.cell.cu2 = two(k.cell.cu2);
+    q.cell.cuF = two(k.cell.cuF);
+    q.cell.b = two(k.cell.b);
+    q.cell.nb = two(k.cell.nb);
+    q.cell.ug = two(k.cell.ug);
+    q.cell.kc = two(k.cell.kc);
+    return q;
+}
+
+template <class R> __device__ __forceinline__ R q_half(const KConst<R>&) { return R(0.5); }
+template <class R> __device__ __forceinline__ R q_nhalf(const KConst<R>&) { return R(-0.5); }
+template <class R> __device__ __forceinline__ R q_nthird(const KConst<R>&) { return R(-1) / R(3); }
+template <class R> __device__ __forceinline__ R q_nquarter(const KConst<R>&) { return R(-0.25); }
+template <class R> __device__ __forceinline__ R q_one(const KConst<R>&) { return R(1); }
+template <class R> __device__ __forceinline__ R q_two(const KConst<R>&) { return R(2); }
+__device__ __forceinline__ float2 q_half(const PairConst& q) { return q.half; }
+__device__ __forceinline__ float2 q_nhalf(const PairConst& q) { return q.nhalf; }
+__device__ __forceinline__ float2 q_nthird(const PairConst& q) { return q.nthird; }
+__device__ __forceinline__ float2 q_nquarter(const PairConst& q) { return q.nquarter; }
+__device__ __forceinline__ float2 q_one(const PairConst& q) { return q.one; }
+__device__ __forceinline__ float2 q_two(const PairConst& q) { return q.two; }
+
+// Constants at porosity e of a porosity field.  With r = (1 - e)/e the
+// Kozeny-Carman and Ergun relations (Sec. 2) collapse to eps nu/K = a r^2 and
+// eps F_eps/sqrt(K) = b r/e: one reciprocal, no square root.
+template <class L, class Q>
+__device__ __forceinline__ Cell<L> field_cell(const Q& q, L e) {
+    using R = typename LaneReal<L>::type;
     Cell<L> c;
     const L ie = lrcp(e);
-    const L q = lmul(lsub(lset<L>(R(1)), e), ie);
+    const L r = lmul(lsub(q_one(q), e), ie);
     c.eps = e;
     c.ie = ie;
-    c.eg = lmul(e, lset<L>(k.gbeta));
-    c.eax = lmul(e, lset<L>(k.ax));
-    c.heax = lmul(e, lset<L>(k.half_ax));
-    c.nnuK = lmul(lmul(q, q), lset<L>(k.nnuK_q2));
-    c.nFK = lmul(lmul(q, ie), lset<L>(k.nFK_q));
-    c.c0 = lfma(lset<L>(R(-0.25)), c.nnuK, lset<L>(R(0.5)));
+    c.eg = lmul(e, q.gbeta);
+    c.eax = lmul(e, q.ax);
+    c.heax = lmul(e, q.half_ax);
+    c.nnuK = lmul(lmul(r, r), q.nnuK_q2);
+    c.nFK = lmul(lmul(r, ie), q.nFK_q);
+    c.c0 = lfma(q_nquarter(q), c.nnuK, q_half(q));
     c.c0sq = lmul(c.c0, c.c0);
-    c.c1 = lmul(lset<L>(R(-0.5)), c.nFK);
-    const L d = lfma(lset<L>(R(-0.5)), c.nnuK, lset<L>(R(1)));  // 2 c0
+    c.c1 = lmul(q_nhalf(q), c.nFK);
+    const L d = lfma(q_nhalf(q), c.nnuK, q_one(q));  // 2 c0
     c.ih = lrcp(d);
-    c.il = lmul(c.ih, lfma(lneg(d), c.ih, lset<L>(R(1))));
-    if constexpr (sizeof(R) == 4) c.il = lfma(c.ih, lset<L>(k.gain), c.il);
+    c.il = lmul(c.ih, lfma(lneg(d), c.ih, q_one(q)));
+    if constexpr (sizeof(R) == 4) c.il = lfma(c.ih, q.gain, c.il);
     c.ci = lneg(lmul(c.c1, c.ih));
-    c.e2 = lmul(ie, lset<L>(k.e2_ie));
-    c.e3 = lmul(ie, lset<L>(k.e3_ie));
-    c.re = lmul(ie, lset<L>(k.rho0));
-    c.qu = lmul(ie, lset<L>(k.qu_ie));
-    c.qF = lmul(ie, lset<L>(k.qF_ie));
-    c.cu2 = lmul(ie, lset<L>(k.cu2_ie));
-    c.cuF = lmul(ie, lset<L>(k.cuF_ie));
-    c.b = lfma(lset<L>(R(0.5)), ie, lset<L>(k.b_0));
-    c.nb = lfma(lset<L>(R(-0.5)), ie, lset<L>(-k.b_0));
-    c.ug = lmul(c.b, lset<L>(k.ug_b));
-    c.kc = lmul(ie, lset<L>(k.kc_ie));
+    c.e2 = lmul(ie, q.e2_ie);
+    c.e3 = lmul(ie, q.e3_ie);
+    c.re = lmul(ie, q.rho0);
+    c.qu = lmul(ie, q.qu_ie);
+    c.qF = lmul(ie, q.qF_ie);
+    c.cu2 = lmul(ie, q.cu2_ie);
+    c.cuF = lmul(ie, q.cuF_ie);
+    c.b = lfma(q_half(q), ie, q.b_0);
+    c.nb = lfma(q_nhalf(q), ie, lneg(q.b_0));
+    c.ug = lmul(c.b, q.ug_b);
+    c.kc = lmul(ie, q.kc_ie);
     return c;
 }
 
 // Constants of node (x, y).
 template <class R>
 __device__ __forceinline__ Cell<R> node_cell(const KConst<R>& k, int x, int y) {
-    return k.eps_field ? field_cell<R>(k, k.eps_field[(long long)y * k.nx + x]) : uniform_cell<R>(k);
+    return k.eps_field ? field_cell<R>(k, k.eps_field[(long long)y * k.nx + x]) : k.cell;
 }
 
 // eps a_y of a node in row y: uniform porosity without a profile has it as a
 // constant.
-template <class L, class R>
-__device__ __forceinline__ L eps_ay(const KConst<R>& k, const Cell<L>& c, int y) {
-    return k.ay_row || k.eps_field ? lmul(c.eps, lset<L>(row_ay(k, y))) : lset<L>(k.eay);
+template <class L, class R, class Q>
+__device__ __forceinline__ L eps_ay(const KConst<R>& k, const Q& q, const Cell<L>& c, int y) {
+    return k.ay_row || k.eps_field ? lmul(c.eps, lset<L>(row_ay(k, y))) : q.eay;
 }
 
 // ------------------------------------------------------------------ moments
@@ -196,18 +298,19 @@ __device__ __forceinline__ L core_hsum_rest(const L* h) {
     return ladd(rest(A, B), rest(ladd(A, B), h[0]));
 }
 // T - T0 from that sum: (sum + Q/2)/sigma.
-template <class L, class R>
-__device__ __forceinline__ L core_theta(const KConst<R>& k, L hsum) {
-    return lfma(hsum, lset<L>(k.inv_sigma), lset<L>(k.hq_sigma));
+template <class L, class Q>
+__device__ __forceinline__ L core_theta(const Q& q, L hsum) {
+    return lfma(hsum, q.inv_sigma, q.hq_sigma);
 }
 
-template <class L, class R>
-__device__ __forceinline__ CoreState<L> core_moments(const KConst<R>& k, const Cell<L>& c, L eay, const L* f,
+template <class L, class Q>
+__device__ __forceinline__ CoreState<L> core_moments(const Q& q, const Cell<L>& c, L eay, const L* f,
                                                      const L* h) {
+    using R = typename LaneReal<L>::type;
     CoreState<L> s;
-    const L half = lset<L>(R(0.5));
-    s.th = core_theta(k, core_hsum(h));
-    s.T = ladd(lset<L>(k.T0), s.th);
+    const L half = q_half(q);
+    s.th = core_theta(q, core_hsum(h));
+    s.T = ladd(q.T0, s.th);
     const L s13 = ladd(f[1], f[3]), s24 = ladd(f[2], f[4]), s57 = ladd(f[5], f[7]), s68 = ladd(f[6], f[8]);
     const L d57 = lsub(f[5], f[7]), d86 = lsub(f[8], f[6]);
     const L mx = ladd(lsub(f[1], f[3]), ladd(d57, d86));
@@ -218,7 +321,7 @@ __device__ __forceinline__ CoreState<L> core_moments(const KConst<R>& k, const C
     const L sf = ladd(s13, Pyy);
     s.Pxy = lsub(s57, s68);
     const L eGy = lfma(c.eg, s.th, eay);  // eps G_y
-    const L ir = lset<L>(k.inv_rho0);
+    const L ir = q.inv_rho0;
     const L vx = lfma(mx, ir, c.heax);
     const L vy = lfma(my, ir, lmul(half, eGy));
     const L vmag = lsqrt(lfma(vx, vx, lmul(vy, vy)));
@@ -230,9 +333,9 @@ __device__ __forceinline__ CoreState<L> core_moments(const KConst<R>& k, const C
         // ih + il = 1/(2 c0).  v iden would carry the rounding of den, the same
         // at every step where c1 |v| is small: a gain or loss of momentum of up
         // to 1e-7 a step that builds up.
-        const L q = lfma(lmul(c.ci, um), iden, c.il);
-        s.ux = lfma(vx, c.ih, lmul(vx, q));
-        s.uy = lfma(vy, c.ih, lmul(vy, q));
+        const L rest = lfma(lmul(c.ci, um), iden, c.il);
+        s.ux = lfma(vx, c.ih, lmul(vx, rest));
+        s.uy = lfma(vy, c.ih, lmul(vy, rest));
     } else {
         s.ux = lmul(vx, iden);
         s.uy = lmul(vy, iden);
@@ -243,18 +346,18 @@ __device__ __forceinline__ CoreState<L> core_moments(const KConst<R>& k, const C
     s.Fy = lfma(nd, s.uy, eGy);
     const L uF = lfma(s.ux, s.Fx, lmul(s.uy, s.Fy));
     L ep = lfma(c.e2, uF, lmul(c.e3, uu));
-    if constexpr (sizeof(R) == 4) ep = lfma(lset<L>(k.e1_lo), sf, ep);
-    s.ep = lfma(lset<L>(k.e1), sf, ep);
+    if constexpr (sizeof(R) == 4) ep = lfma(q.e1_lo, sf, ep);
+    s.ep = lfma(q.e1, sf, ep);
     s.Px = lsub(Pxx, s.ep);
     s.Py = lsub(Pyy, s.ep);
     // grad T: (a I - b u u^T) grad T = N
     const L h57 = lsub(h[5], h[7]), h86 = lsub(h[8], h[6]);
     const L hx = ladd(lsub(h[1], h[3]), ladd(h57, h86));
     const L hy = ladd(lsub(h[2], h[4]), lsub(h57, h86));
-    const L qT = lsub(lset<L>(k.hq_sigma), s.T), Th = lmul(half, s.T);
+    const L qT = lsub(q.hq_sigma, s.T), Th = lmul(half, s.T);
     const L Nx = lfma(s.ux, qT, lfma(Th, s.Fx, hx));
     const L Ny = lfma(s.uy, qT, lfma(Th, s.Fy, hy));
-    const L a = lfma(lset<L>(k.a_ep), s.ep, lset<L>(k.a_const));
+    const L a = lfma(q.a_ep, s.ep, q.a_const);
     const L d = lfma(c.nb, uu, a);
     const L r = lrcp(lmul(a, d));  // 1/a = d r, 1/d = a r
     const L ia = lmul(d, r);
@@ -269,105 +372,104 @@ template <class L>
 struct Shear {
     L xx, yy, xy;
 };
-template <class L, class R>
-__device__ __forceinline__ Shear<L> core_shear(const KConst<R>& k, const Cell<L>& c, const CoreState<L>& s) {
-    const L D = lset<L>(k.invD);
+template <class L, class Q>
+__device__ __forceinline__ Shear<L> core_shear(const Q& q, const Cell<L>& c, const CoreState<L>& s) {
+    const L D = q.invD;
     const L dx = lsub(s.Fx, s.ux), dy = lsub(s.Fy, s.uy);
     const L rx = lmul(c.re, s.ux), ry = lmul(c.re, s.uy);
     Shear<L> S;
     S.xx = lmul(D, lfma(rx, dx, s.Px));
     S.yy = lmul(D, lfma(ry, dy, s.Py));
-    S.xy = lmul(D, lfma(lset<L>(R(0.5)), lfma(rx, dy, lmul(ry, dx)), s.Pxy));
+    S.xy = lmul(D, lfma(q_half(q), lfma(rx, dy, lmul(ry, dx)), s.Pxy));
     return S;
 }
 
 // The form Q of the even flow part (Q2 = 2 Q_xy): from the pulled second
 // moments (interior nodes) ...
-template <class L, class R>
-__device__ __forceinline__ void core_form(const KConst<R>& k, const Cell<L>& c, const CoreState<L>& s, L& Qxx, L& Qyy,
+template <class L, class Q>
+__device__ __forceinline__ void core_form(const Q& q, const Cell<L>& c, const CoreState<L>& s, L& Qxx, L& Qyy,
                                           L& Q2) {
-    const L al = lset<L>(k.aS);
+    const L al = q.aS;
     const L tx = lfma(c.qu, s.ux, lmul(c.qF, s.Fx)), ty = lfma(c.qu, s.uy, lmul(c.qF, s.Fy));
     Qxx = lfma(s.ux, tx, lmul(al, s.Px));
     Qyy = lfma(s.uy, ty, lmul(al, s.Py));
-    Q2 = lfma(s.ux, ty, lfma(s.uy, tx, lmul(lset<L>(k.aS2), s.Pxy)));
+    Q2 = lfma(s.ux, ty, lfma(s.uy, tx, lmul(q.aS2, s.Pxy)));
 }
 // ... or from an explicit shear rate (walls, moment state).
-template <bool SOURCES, class L, class R>
-__device__ __forceinline__ void shear_form(const KConst<R>& k, const Cell<L>& c, L ux, L uy, L Fx, L Fy,
+template <bool SOURCES, class L, class Q>
+__device__ __forceinline__ void shear_form(const Q& q, const Cell<L>& c, L ux, L uy, L Fx, L Fy,
                                            const Shear<L>& S, L& Qxx, L& Qyy, L& Q2) {
-    const L fs = lset<L>(k.f_ScS);
+    const L fs = q.f_ScS;
     const L tx = SOURCES ? lfma(c.cu2, ux, lmul(c.cuF, Fx)) : lmul(c.cu2, ux);
     const L ty = SOURCES ? lfma(c.cu2, uy, lmul(c.cuF, Fy)) : lmul(c.cu2, uy);
     Qxx = lfma(ux, tx, lmul(fs, S.xx));
     Qyy = lfma(uy, ty, lmul(fs, S.yy));
-    Q2 = lfma(ux, ty, lfma(uy, tx, lmul(lset<L>(k.f_ScS2), S.xy)));
+    Q2 = lfma(ux, ty, lfma(uy, tx, lmul(q.f_ScS2, S.xy)));
 }
 
 // Collision: f* = (1 - 1/tau) f + f^eq/tau + F_i and g* likewise, from the
 // state and the form Q.  TAU1: tau_f = tau_T = 1 (f, h are not read); then
 // wscale multiplies every output (the FP16 storage scale).  SOURCES = false
 // keeps the equilibria alone.
-template <bool TAU1, bool SOURCES, class L, class R>
-__device__ __forceinline__ void core_emit(const KConst<R>& k, const Cell<L>& c, const CoreState<L>& s, L Qxx, L Qyy,
-                                          L Q2, const L* f, const L* h, L* fo, L* ho, R wscale) {
-    const L w1 = lset<L>(wscale * (R(1) / R(9)));
-    const L nthird = lset<L>(R(-1) / R(3));
+template <bool TAU1, bool SOURCES, class L, class Q>
+__device__ __forceinline__ void core_emit(const Q& q, const Cell<L>& c, const CoreState<L>& s, L Qxx, L Qyy,
+                                          L Q2, const L* f, const L* h, L* fo, L* ho,
+                                          typename LaneReal<L>::type wscale) {
+    const CoreWeights<L> w_ = core_weights(q, wscale);
+    const L w1 = w_.w1;
+    const L nthird = q_nthird(q);
     // out_i, out_j = w (e +- d) of two opposite directions.  The smaller of
     // the two parts is scaled by w first, so that each output is rounded once
     // at its own size: in the flow e ~ u^2 < d ~ u, in the temperature d < e.
-    auto put_f = [&](int i, int j, const L& w, const L& e, const L& d) {
-        const L b = lmul(w, e), n = lneg(w);
-        fo[i] = lfma(w, d, TAU1 ? b : lfma(lset<L>(k.omf), f[i], b));
-        fo[j] = lfma(n, d, TAU1 ? b : lfma(lset<L>(k.omf), f[j], b));
+    auto put_f = [&](int i, int j, const L& w, const L& n, const L& e, const L& d) {
+        const L b = lmul(w, e);
+        fo[i] = lfma(w, d, TAU1 ? b : lfma(q.omf, f[i], b));
+        fo[j] = lfma(n, d, TAU1 ? b : lfma(q.omf, f[j], b));
     };
     {
         const L tr = ladd(Qxx, Qyy);
-        const L E = lfma(nthird, tr, lmul(lset<L>(k.fA_ep), s.ep));
+        const L E = lfma(nthird, tr, lmul(q.fA_ep, s.ep));
         const L Ed = ladd(E, tr);
-        const L fu = lset<L>(k.f_cu), fF = lset<L>(k.f_cF);
+        const L fu = q.f_cu, fF = q.f_cF;
         const L Dx = SOURCES ? lfma(fu, s.ux, lmul(fF, s.Fx)) : lmul(fu, s.ux);
         const L Dy = SOURCES ? lfma(fu, s.uy, lmul(fF, s.Fy)) : lmul(fu, s.uy);
-        // the flow's own diagonal weight, rounded to nearest: 2 w_1 + 4 w_5 is
-        // then within 7.5e-9 of 1/3, which scales the momentum in each step
-        // (w_diag, fitted to the sum of all nine, is 1.5e-8 off)
-        const L w5 = lset<L>(wscale * (R(1) / R(36)));
-        put_f(1, 3, w1, ladd(E, Qxx), Dx);
-        put_f(2, 4, w1, ladd(E, Qyy), Dy);
-        put_f(5, 7, w5, ladd(Ed, Q2), SOURCES ? ladd(Dx, Dy) : lfma(fu, s.uy, Dx));
-        put_f(6, 8, w5, lsub(Ed, Q2), SOURCES ? lsub(Dy, Dx) : lfma(lset<L>(-k.f_cu), s.ux, Dy));
+        const L w5 = w_.w5f;
+        put_f(1, 3, w1, w_.n1, ladd(E, Qxx), Dx);
+        put_f(2, 4, w1, w_.n1, ladd(E, Qyy), Dy);
+        put_f(5, 7, w5, w_.n5f, ladd(Ed, Q2), SOURCES ? ladd(Dx, Dy) : lfma(fu, s.uy, Dx));
+        put_f(6, 8, w5, w_.n5f, lsub(Ed, Q2), SOURCES ? lsub(Dy, Dx) : lfma(lneg(q.f_cu), s.ux, Dy));
     }
     {
         // even part: sigma theta plus small terms, summed among themselves first
         const L T = s.T, Tep = lmul(T, s.ep);
-        const L th = lmul(lset<L>(k.h_sig), s.th);
+        const L th = lmul(q.h_sig, s.th);
         const L kc = lmul(c.kc, T);
         const L kx = lmul(kc, s.ux), ky = lmul(kc, s.uy);
         const L tr = lfma(kx, s.ux, lmul(ky, s.uy));
-        const L m0 = SOURCES ? lfma(nthird, tr, lset<L>(k.h_kQ)) : lmul(nthird, tr);
+        const L m0 = SOURCES ? lfma(nthird, tr, q.h_kQ) : lmul(nthird, tr);
         // h + (w sum h - h)/tau + w (small +- d): the difference is small, so
         // the output is rounded once at its own size here too; sigma theta =
         // sum h + Q/2, and what the sum in R misses joins the small terms
-        const L itT = lset<L>(R(1) - k.omT);
+        const L itT = lsub(q_one(q), q.omT);
         L tr0, m1 = m0;
         if constexpr (!TAU1) {
             tr0 = core_hsum(h);
-            m1 = lfma(itT, ladd(core_hsum_rest(h), lset<L>(k.half_Q)), m0);
+            m1 = lfma(itT, ladd(core_hsum_rest(h), q.half_Q), m0);
         }
-        const L m = lfma(lset<L>(k.h_pT), Tep, m1);
-        const L md = SOURCES ? ladd(m, tr) : lfma(lset<L>(R(1)), tr, m);
+        const L m = lfma(q.h_pT, Tep, m1);
+        const L md = SOURCES ? ladd(m, tr) : lfma(q_one(q), tr, m);
         L Vx, Vy;
         if constexpr (SOURCES) {
-            const L K = lfma(lset<L>(k.h_u3), T, lfma(c.ug, lfma(s.ux, s.gx, lmul(s.uy, s.gy)), lset<L>(k.h_uQ)));
-            const L hg = lfma(lset<L>(k.h_Wr), s.ep, lset<L>(k.h_g)), hT = lmul(lset<L>(k.h_W), T);
+            const L K = lfma(q.h_u3, T, lfma(c.ug, lfma(s.ux, s.gx, lmul(s.uy, s.gy)), q.h_uQ));
+            const L hg = lfma(q.h_Wr, s.ep, q.h_g), hT = lmul(q.h_W, T);
             Vx = lfma(K, s.ux, lfma(hg, s.gx, lmul(hT, s.Fx)));
             Vy = lfma(K, s.uy, lfma(hg, s.gy, lmul(hT, s.Fy)));
         } else {
-            const L K = lmul(lset<L>(k.h_u3), T), hg = lset<L>(k.h_g);
+            const L K = lmul(q.h_u3, T), hg = q.h_g;
             Vx = lfma(K, s.ux, lmul(hg, s.gx));
             Vy = lfma(K, s.uy, lmul(hg, s.gy));
         }
-        const L w5 = lset<L>(wscale * w_diag<R>());
+        const L w5 = w_.w5h;
         auto relax = [&](const L& w, const L& small, const L& in) {
             return ladd(in, lfma(itT, lfma(w, tr0, lneg(in)), lmul(w, small)));
         };
@@ -383,26 +485,25 @@ __device__ __forceinline__ void core_emit(const KConst<R>& k, const Cell<L>& c, 
         };
         put_h(1, 3, w1, lfma(kx, s.ux, m), Vx);
         put_h(2, 4, w1, lfma(ky, s.uy, m), Vy);
-        const L k2 = lmul(lset<L>(R(2)), kx);
+        const L k2 = lmul(q_two(q), kx);
         put_h(5, 7, w5, lfma(k2, s.uy, md), ladd(Vx, Vy));
         put_h(6, 8, w5, lfma(lneg(k2), s.uy, md), lsub(Vy, Vx));
-        const L w0 = lset<L>(wscale * (R(4) / R(9)));
-        const L pT = lset<L>(wscale * k.h0_pT);
+        const L w0 = w_.w0;
+        const L pT = w_.pT;
         if constexpr (TAU1) ho[0] = lfma(w0, th, lfma(w0, m0, lmul(pT, Tep)));
         else ho[0] = ladd(h[0], lfma(itT, lfma(w0, tr0, lneg(h[0])), lfma(w0, m1, lmul(pT, Tep))));
     }
 }
 
-// Interior node: moments, then the collision.  The rest direction's thermal
-// value is finite only if T and u are, so it stands for both.
-template <bool TAU1, class L, class R>
-__device__ __forceinline__ void core_interior(const KConst<R>& k, const Cell<L>& c, L eay, const L* f, const L* h,
-                                              L* fo, L* ho, R wscale = R(1)) {
-    const CoreState<L> s = core_moments(k, c, eay, f, h);
+// Interior node: moments, then the collision.  (The rest direction's thermal
+// value ho[0] is finite only if T and u are: the caller's watchdog looks at it.)
+template <bool TAU1, class L, class Q>
+__device__ __forceinline__ void core_interior(const Q& q, const Cell<L>& c, L eay, const L* f, const L* h, L* fo, L* ho,
+                                              typename LaneReal<L>::type wscale = 1) {
+    const CoreState<L> s = core_moments(q, c, eay, f, h);
     L Qxx, Qyy, Q2;
-    core_form(k, c, s, Qxx, Qyy, Q2);
-    core_emit<TAU1, true>(k, c, s, Qxx, Qyy, Q2, f, h, fo, ho, wscale);
-    if (!lfinite(ho[0])) atomicOr(k.flag, 1);
+    core_form(q, c, s, Qxx, Qyy, Q2);
+    core_emit<TAU1, true>(q, c, s, Qxx, Qyy, Q2, f, h, fo, ho, wscale);
 }
 
 // Wall node at tau_f = tau_T = 1 (Sec. 3.4): there the extrapolated
@@ -410,24 +511,24 @@ __device__ __forceinline__ void core_interior(const KConst<R>& k, const Cell<L>&
 // collision of its boundary state b alone.  s, S: state and shear rate of
 // x_f (on entry s; b on return), cs / cb: constants of x_f and of the node,
 // thff: T(x_ff) - T0, thb: the Dirichlet T_b - T0 where `given`.
-template <class L, class R>
-__device__ __forceinline__ void core_boundary(const KConst<R>& k, const Cell<L>& cs, const Cell<L>& cb, L eay_b,
-                                              R ubx, R uby, R ubm, bool given, bool fixgx, bool fixgy, R thb, L thff,
-                                              CoreState<L>& s) {
-    s.ux = lset<L>(ubx);
-    s.uy = lset<L>(uby);
+template <class R>
+__device__ __forceinline__ void core_boundary(const KConst<R>& k, const Cell<R>& cs, const Cell<R>& cb, R eay_b,
+                                              R ubx, R uby, R ubm, bool given, bool fixgx, bool fixgy, R thb, R thff,
+                                              CoreState<R>& s) {
+    s.ux = ubx;
+    s.uy = uby;
     if (given) {
-        s.th = lset<L>(thb);
+        s.th = thb;
     } else {
         // Eq. (TNEESApGra) with zero normal gradient
-        s.th = lmul(lset<L>(R(1) / R(3)), lfma(lset<L>(R(4)), s.th, lneg(thff)));
-        if (fixgx) s.gx = lset<L>(R(0));
-        if (fixgy) s.gy = lset<L>(R(0));
+        s.th = lmul(R(1) / R(3), lfma(R(4), s.th, lneg(thff)));
+        if (fixgx) s.gx = R(0);
+        if (fixgy) s.gy = R(0);
     }
-    s.T = ladd(lset<L>(k.T0), s.th);
+    s.T = ladd(k.T0, s.th);
     // p(x_f) at the wall node's own porosity
     if (k.eps_field) s.ep = lmul(lmul(s.ep, cs.ie), cb.eps);
-    const L nd = lfma(cb.nFK, lset<L>(ubm), cb.nnuK);
+    const R nd = lfma(cb.nFK, ubm, cb.nnuK);
     s.Fx = lfma(nd, s.ux, cb.eax);
     s.Fy = lfma(nd, s.uy, lfma(cb.eg, s.th, eay_b));
 }

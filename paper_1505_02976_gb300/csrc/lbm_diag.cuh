@@ -43,7 +43,7 @@ __device__ __forceinline__ void node_u_th(const KConst<R>& k, const S* __restric
     Pops<R> P;
     pull(k, src, x, y, P);
     const Cell<R> c = node_cell(k, x, y);
-    const CoreState<R> s = core_moments(k, c, eps_ay(k, c, y), P.f, P.h);
+    const CoreState<R> s = core_moments(k, c, eps_ay(k, k, c, y), P.f, P.h);
     if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
     *ux = s.ux;
     *uy = s.uy;

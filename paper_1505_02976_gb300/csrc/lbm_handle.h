@@ -29,6 +29,8 @@ struct lbm_handle {
     bool tma, tma_ready;
     CUtensorMap tmap[2];
     int tma_rows;
+    int sms;
+    bool two_steps;  // FP32 populations: pairs of steps go through launch_two_steps
     bool nonfinite, timeout;
     lbm::KConst<double> k64;
     lbm::KConst<float> k32;

@@ -75,7 +75,7 @@ __device__ __forceinline__ void expand_moments(const KConst<R>& k, const Cell<R>
 template <class R, bool EPS_FIELD>
 __device__ __forceinline__ Cell<R> moment_cell(const KConst<R>& k, int x, int y) {
     if constexpr (EPS_FIELD) return field_cell<R>(k, node_eps(k, x, y));
-    else return uniform_cell<R>(k);
+    else return k.cell;
 }
 
 // Plane strides are 32-bit (9 planes of ny * pitch < 2^31 elements).
@@ -146,7 +146,7 @@ __device__ __forceinline__ Expanded<R> expand_node(const KConst<R>& k, const R* 
     if (!ok) return e;
     R fo[9], ho[9];
     const Cell<R> c = moment_cell<R, EPS_FIELD>(k, xe, r);
-    expand_moments<R, SOURCES>(k, c, eps_ay(k, c, r), m, fo, ho);
+    expand_moments<R, SOURCES>(k, c, eps_ay(k, k, c, r), m, fo, ho);
     e.up[0] = fo[2]; e.up[1] = fo[5]; e.up[2] = fo[6];
     e.up[3] = ho[2]; e.up[4] = ho[5]; e.up[5] = ho[6];
     e.hz[0] = fo[1]; e.hz[1] = fo[3]; e.hz[2] = ho[0]; e.hz[3] = ho[1]; e.hz[4] = ho[3];
@@ -237,7 +237,7 @@ k_step_m(const __grid_constant__ KConst<R> k, const R* __restrict__ src, R* dst,
             R mo[kMPlanes] = {};
             if (out_col && !wall_col) {
                 const Cell<R> c = moment_cell<R, EPS_FIELD>(k, x, y);
-                const CoreState<R> s = core_moments(k, c, eps_ay(k, c, y), f, h);
+                const CoreState<R> s = core_moments(k, c, eps_ay(k, k, c, y), f, h);
                 const Shear<R> S = core_shear(k, c, s);
                 if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
                 mo[MP] = lmul(s.ep, c.ie);
@@ -290,7 +290,7 @@ __global__ void k_expand_m(const __grid_constant__ KConst<R> k, const R* __restr
     for (int q = 0; q < kMPlanes; ++q) m[q] = src[q * k.plane + at];
     const Cell<R> c = node_cell(k, x, y);
     R fo[9], ho[9];
-    expand_moments<R, SOURCES>(k, c, eps_ay(k, c, y), m, fo, ho);
+    expand_moments<R, SOURCES>(k, c, eps_ay(k, k, c, y), m, fo, ho);
 #pragma unroll
     for (int i = 1; i < 9; ++i) dst[(i - 1) * k.plane + at] = fo[i];
 #pragma unroll

@@ -46,10 +46,11 @@ __device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __r
     for (int i = 0; i < 9; ++i) h[i] = load_pop<S, R>(c + ((8 + i) * pl + o[i]), sc);
     Cell<R> cell;
     if constexpr (EPS_FIELD) cell = field_cell<R>(k, k.eps_field[(long long)y * k.nx + x]);
-    else cell = uniform_cell<R>(k);
+    else cell = k.cell;
     R fo[9], ho[9];
     constexpr bool prescale = TAU1 && std::is_same<S, __half>::value;
-    core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo, ho, prescale ? R(k.inv_scale) : R(1));
+    core_interior<TAU1>(k, cell, eps_ay(k, k, cell, y), f, h, fo, ho, prescale ? R(k.inv_scale) : R(1));
+    if (!lfinite(ho[0])) atomicOr(k.flag, 1);
     Dither dither((uint32_t)at, step);
     store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
 }
@@ -77,10 +78,10 @@ __device__ __forceinline__ void wall_node_tau1(const KConst<R>& k, const Source&
         thff = core_theta(k, core_hsum(Q.h));
     }
     const Cell<R> cs = node_cell(k, w.xs, w.ys), cb = node_cell(k, x, y);
-    CoreState<R> s = core_moments(k, cs, eps_ay(k, cs, w.ys), P.f, P.h);
+    CoreState<R> s = core_moments(k, cs, eps_ay(k, k, cs, w.ys), P.f, P.h);
     const Shear<R> S_ = core_shear(k, cs, s);
     const R thb = w.tside >= 0 ? k.T_bc[w.tside] - k.T0 : R(0);
-    core_boundary(k, cs, cb, eps_ay(k, cb, y), k.u_bc[w.uside][0], k.u_bc[w.uside][1], k.u_abs[w.uside], w.tside >= 0,
+    core_boundary(k, cs, cb, eps_ay(k, k, cb, y), k.u_bc[w.uside][0], k.u_bc[w.uside][1], k.u_abs[w.uside], w.tside >= 0,
                   w.fixgx != 0, w.fixgy != 0, thb, thff, s);
     R Qxx, Qyy, Q2;
     shear_form<true>(k, cb, s.ux, s.uy, s.Fx, s.Fy, S_, Qxx, Qyy, Q2);

@@ -257,8 +257,9 @@ __device__ __forceinline__ bool staged_rows(const KConst<float>& k, const S* __r
             float fo[9], ho[9];
             Cell<float> cell;
             if constexpr (EPS_FIELD) cell = field_cell<float>(k, node_eps(k, x, y));
-            else cell = uniform_cell<float>(k);
-            core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo, ho, prescale ? k.inv_scale : 1.0f);
+            else cell = k.cell;
+            core_interior<TAU1>(k, cell, eps_ay(k, k, cell, y), f, h, fo, ho, prescale ? k.inv_scale : 1.0f);
+            if (!lfinite(ho[0])) atomicOr(k.flag, 1);
             const int at = y * k.pitch + x;
             Dither dither((uint32_t)at, step);
             store_planes<S, float>(dst + at, k.plane32, fo, ho, prescale ? 1.0f : k.inv_scale, &dither, hot);
@@ -283,7 +284,7 @@ __device__ __forceinline__ bool staged_rows(const KConst<float>& k, const S* __r
 // per plane (a pair with a wall or out-of-range member stores its interior
 // node alone, with the same rounding).
 template <bool EPS_FIELD, bool TAU1>
-__device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const __half* __restrict__ src,
+__device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const PairConst& pc, const __half* __restrict__ src,
                                                  __half* __restrict__ dst, int x0, int y0, int rows, uint32_t step,
                                                  const __half* stage, uint64_t* bar, bool hot = false) {
     using L = TmaLayout<__half>;
@@ -343,8 +344,8 @@ __device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const _
                 for (int i = 1; i < 9; ++i) f2[i] = lmul(__half22float2(pk[i - 1]), sc);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) h2[i] = lmul(__half22float2(pk[8 + i]), sc);
-                const Cell<float2> cell = uniform_cell<float2>(k);
-                core_interior<true>(k, cell, eps_ay(k, cell, y), f2, h2, fo2, ho2, k.inv_scale);
+                core_interior<true>(pc, pc.cell, eps_ay(k, pc, pc.cell, y), f2, h2, fo2, ho2);
+                if (!lfinite(ho2[0])) atomicOr(k.flag, 1);
                 const Dither dither((uint32_t)at, step);
                 uint32_t* wd = reinterpret_cast<uint32_t*>(dst + at);
                 const int pw = k.plane32 >> 1;
@@ -379,8 +380,9 @@ __device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const _
             for (int i = 0; i < 9; ++i) h[i] = (n == 0 ? __low2float(pk[8 + i]) : __high2float(pk[8 + i])) * k.scale;
             Cell<float> cell;
             if constexpr (EPS_FIELD) cell = field_cell<float>(k, node_eps(k, xa + n, y));
-            else cell = uniform_cell<float>(k);
-            core_interior<TAU1>(k, cell, eps_ay(k, cell, y), f, h, fo[n], ho[n], TAU1 ? k.inv_scale : 1.0f);
+            else cell = k.cell;
+            core_interior<TAU1>(k, cell, eps_ay(k, k, cell, y), f, h, fo[n], ho[n], TAU1 ? k.inv_scale : 1.0f);
+            if (!lfinite(ho[n][0])) atomicOr(k.flag, 1);
         }
         if (act0 && act1) {
             const Dither dither((uint32_t)at, step);
@@ -410,7 +412,8 @@ __device__ __forceinline__ void staged_rows_pair(const KConst<float>& k, const _
 // so that the blocks the hardware starts last are plain interior ones.
 template <class S, bool EPS_FIELD, bool TAU1>
 __global__ void __launch_bounds__(kTBand, TmaBlocks<S>::value)
-k_step_tma(const __grid_constant__ KConst<float> k, const __grid_constant__ CUtensorMap tm,
+k_step_tma(const __grid_constant__ KConst<float> k, const __grid_constant__ PairConst pc,
+           const __grid_constant__ CUtensorMap tm,
            const S* __restrict__ src, S* __restrict__ dst, int rows, uint32_t step) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -436,7 +439,7 @@ k_step_tma(const __grid_constant__ KConst<float> k, const __grid_constant__ CUte
     asm volatile("griddepcontrol.wait;" ::: "memory");
     staged_issue_warps<S>(&tm, stage, bar, x0, y0, rows, k.ny);
     if constexpr (std::is_same<S, __half>::value)
-        staged_rows_pair<EPS_FIELD, TAU1>(k, src, dst, x0, y0, rows, step, stage, bar, hot);
+        staged_rows_pair<EPS_FIELD, TAU1>(k, pc, src, dst, x0, y0, rows, step, stage, bar, hot);
     else
         staged_rows<S, EPS_FIELD, TAU1>(k, src, dst, x0, y0, rows, step, stage, bar, 0u, hot);
 }
@@ -697,7 +700,9 @@ static cudaError_t launch_tma(const cudaLaunchConfig_t& cfg, const KConst<float>
                               const S* src, S* dst, int rows, uint32_t step) {
     cudaError_t e = allow_tma_smem<S, E, T>();
     if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, k_step_tma<S, E, T>, k, tm, src, dst, rows, step);
+    // (read by the FP16 form alone; its outputs take the storage scale)
+    const PairConst pc = make_pair_const(k, k.inv_scale);
+    return cudaLaunchKernelEx(&cfg, k_step_tma<S, E, T>, k, pc, tm, src, dst, rows, step);
 }
 
 template <class S>
