@@ -18,24 +18,6 @@ namespace lbm {
 template <class R> struct BatchOccupancy { static constexpr int blocks = LBM_BATCH_BLOCKS; };
 template <> struct BatchOccupancy<double> { static constexpr int blocks = 3; };
 
-// Wall node idx of a cavity in perimeter order: S row, N row, W column, E
-// column (walled sides only; the columns skip the rows' corner nodes).
-template <class R>
-__device__ __forceinline__ void perimeter_node(const KConst<R>& k, int idx, int& x, int& y) {
-    const bool wS = k.bc[SS] != BC_PERIODIC, wN = k.bc[SN] != BC_PERIODIC;
-    const int nS = wS ? k.nx : 0, nN = wN ? k.nx : 0;
-    const int y0 = wS ? 1 : 0, y1 = wN ? k.ny - 1 : k.ny;
-    const int nW = k.bc[SW] != BC_PERIODIC ? y1 - y0 : 0;
-    if (idx < nS) { x = idx; y = 0; return; }
-    idx -= nS;
-    if (idx < nN) { x = idx; y = k.ny - 1; return; }
-    idx -= nN;
-    if (idx < nW) { x = 0; y = y0 + idx; return; }
-    idx -= nW;
-    x = k.nx - 1;
-    y = y0 + idx;
-}
-
 // Batched step: a grid of resident blocks walks a work list drawn from many
 // cavities of different size and parameters.  Each block takes one
 // contiguous, cost-balanced range of the list (items are sorted by cavity,

@@ -15,25 +15,44 @@ namespace lbm {
 
 
 
-// The fused step: one thread per node; interior nodes take the fast path,
-// wall nodes the NEES path.  TAU1: tau_f = tau_T = 1 (the paper's default,
+// The fused step: one thread per node.  The first `wall_blocks` blocks take the
+// wall nodes in perimeter order (the NEES path), the others the interior nodes
+// row by row, bx blocks a row: a warp then runs one of the two paths, where a
+// warp with both would run them one after the other, and the wall nodes'
+// longer chain starts first.  TAU1: tau_f = tau_T = 1 (the paper's default,
 // Sec. 4), where the (1 - 1/tau) terms vanish.
+// FP64 is bound by its pipe (two lanes a cycle and SM): 700 x 517 takes 126 us a
+// step, 0.95 of the measured FP64 rate for its 182 FP64 instructions a warp and
+// node (165 us with the wall nodes inside the rows' warps, 267 with the
+// direction-by-direction arithmetic too); blocks of one warp end most evenly
+// (130 us in blocks of four).  A lattice that leaves SMs empty is bound by one
+// warp's chain, and blocks of one warp put every warp on an SM of its own: 32^2
+// 8.7 us a step (10.0 in blocks of four; 17.3 with the wall nodes inside, 38
+// before).
 template <class R, class S, bool EPS_FIELD, bool TAU1>
 __global__ void __launch_bounds__(kStepBlock, StepOccupancy<R>::blocks)
-k_step(const __grid_constant__ KConst<R> k, const S* __restrict__ src, S* __restrict__ dst, uint32_t step) {
-    // Programmatic dependent launch: let the next step's blocks be scheduled
-    // while this grid drains, and wait here until the previous step's grid
+k_step(const __grid_constant__ KConst<R> k, const S* __restrict__ src, S* __restrict__ dst, int wall_blocks, int bx,
+       uint32_t step) {
+    // Programmatic dependent launch: wait here until the previous step's grid
     // has completed and its writes are visible (no-op without the launch
-    // attribute).  Both are hardware-managed; nothing spins.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // attribute), then let the next step's blocks be scheduled while this grid
+    // runs.  Both are hardware-managed; nothing spins.  The other order lets a
+    // whole queue of later steps take their places on the SMs: FP64 80^2 8.9 us
+    // a step against 19.4.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int x = blockIdx.x * kStepBlock + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= k.nx) return;
-    if (is_wall(k, x, y)) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if ((int)blockIdx.x < wall_blocks) {
+        const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+        if (n >= perimeter_nodes(k)) return;
+        int x, y;
+        perimeter_node(k, n, x, y);
         wall_update(k, src, dst, x, y, step);
         return;
     }
+    const unsigned b = blockIdx.x - wall_blocks;
+    const int y = (int)(b / (unsigned)bx);
+    const int x = (int)((b - (unsigned)y * bx) * blockDim.x + threadIdx.x);
+    if (x >= k.nx || is_wall(k, x, y)) return;
     interior_update<R, S, EPS_FIELD, TAU1>(k, src, dst, x, y, step);
 }
 
@@ -60,12 +79,34 @@ __global__ void k_init(const __grid_constant__ KConst<R> k, S* __restrict__ dst,
 
 // ------------------------------------------------------------------ launchers
 
+// Multiprocessors of the current device (asked once per device).
+static int device_sms() {
+    constexpr int kMaxDev = 64;
+    static int known[kMaxDev] = {};
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev < kMaxDev && known[dev] > 0) return known[dev];
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
+    if (dev < kMaxDev) known[dev] = sms;
+    return sms;
+}
+
 template <class R, class S>
 cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = row_grid(k.nx, k.ny, kStepBlock);
-    cfg.blockDim = dim3(kStepBlock);
-    cfg.dynamicSmemBytes = 0;
+    // blocks of one warp in FP64, and while whole blocks would not fill the GPU twice
+    const long long full = (long long)((k.nx + kStepBlock - 1) / kStepBlock) * k.ny;
+    const int block = sizeof(R) == 8 || full < 2LL * device_sms() ? 32 : kStepBlock;
+    const int bx = (k.nx + block - 1) / block, wall_blocks = (perimeter_nodes(k) + block - 1) / block;
+    cfg.gridDim = dim3((unsigned)(wall_blocks + (long long)bx * k.ny));
+    cfg.blockDim = dim3((unsigned)block);
+    // The blocks of a dependent launch fill SM after SM up to the kernel's
+    // occupancy (12 blocks of one warp), which leaves SMs idle where the grid
+    // is smaller: unused shared memory keeps each SM to its share of the
+    // blocks.  FP64 130^2 13.2 -> 12.0, 201^2 21.6 -> 18.9 us a step; with
+    // fewer than four blocks an SM the launches overlap less and it costs 0.5 us.
+    const long long per = (cfg.gridDim.x + device_sms() - 1) / device_sms();
+    cfg.dynamicSmemBytes = sizeof(R) == 8 && per >= 4 && per < 12 ? (size_t)(227 / per - 1) * 1024 : 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -74,10 +115,10 @@ cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step,
     cfg.numAttrs = 1;
     const bool tau1 = k.omf == R(0) && k.omT == R(0);
     if (k.eps_field)
-        return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, true, true>, k, src, dst, step)
-                    : cudaLaunchKernelEx(&cfg, k_step<R, S, true, false>, k, src, dst, step);
-    return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, false, true>, k, src, dst, step)
-                : cudaLaunchKernelEx(&cfg, k_step<R, S, false, false>, k, src, dst, step);
+        return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, true, true>, k, src, dst, wall_blocks, bx, step)
+                    : cudaLaunchKernelEx(&cfg, k_step<R, S, true, false>, k, src, dst, wall_blocks, bx, step);
+    return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, false, true>, k, src, dst, wall_blocks, bx, step)
+                : cudaLaunchKernelEx(&cfg, k_step<R, S, false, false>, k, src, dst, wall_blocks, bx, step);
 }
 
 template <class R, class S>

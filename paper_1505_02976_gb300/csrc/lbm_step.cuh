@@ -55,6 +55,32 @@ __device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __r
     store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
 }
 
+// Wall node idx of a lattice in perimeter order: S row, N row, W column, E
+// column (walled sides only; the columns skip the rows' corner nodes).
+template <class R>
+__device__ __forceinline__ void perimeter_node(const KConst<R>& k, int idx, int& x, int& y) {
+    const bool wS = k.bc[SS] != BC_PERIODIC, wN = k.bc[SN] != BC_PERIODIC;
+    const int nS = wS ? k.nx : 0, nN = wN ? k.nx : 0;
+    const int y0 = wS ? 1 : 0, y1 = wN ? k.ny - 1 : k.ny;
+    const int nW = k.bc[SW] != BC_PERIODIC ? y1 - y0 : 0;
+    if (idx < nS) { x = idx; y = 0; return; }
+    idx -= nS;
+    if (idx < nN) { x = idx; y = k.ny - 1; return; }
+    idx -= nN;
+    if (idx < nW) { x = 0; y = y0 + idx; return; }
+    idx -= nW;
+    x = k.nx - 1;
+    y = y0 + idx;
+}
+
+// Number of wall nodes in that order.
+template <class R>
+__host__ __device__ inline int perimeter_nodes(const KConst<R>& k) {
+    const int wS = k.bc[SS] != BC_PERIODIC, wN = k.bc[SN] != BC_PERIODIC;
+    const int inner = k.ny - wS - wN;
+    return (wS + wN) * k.nx + ((k.bc[SW] != BC_PERIODIC) + (k.bc[SE] != BC_PERIODIC)) * inner;
+}
+
 // Where a wall node's update takes its pulled values from: the population
 // buffer src in global memory.
 template <class R, class S>
@@ -83,9 +109,14 @@ __device__ __forceinline__ void wall_node_tau1(const KConst<R>& k, const Source&
     const R thb = w.tside >= 0 ? k.T_bc[w.tside] - k.T0 : R(0);
     core_boundary(k, cs, cb, eps_ay(k, k, cb, y), k.u_bc[w.uside][0], k.u_bc[w.uside][1], k.u_abs[w.uside], w.tside >= 0,
                   w.fixgx != 0, w.fixgy != 0, thb, thff, s);
-    R Qxx, Qyy, Q2;
-    shear_form<true>(k, cb, s.ux, s.uy, s.Fx, s.Fy, S_, Qxx, Qyy, Q2);
-    core_emit<true, true>(k, cb, s, Qxx, Qyy, Q2, P.f, P.h, fo, ho, R(1));
+    if (k.u_abs[w.uside] == R(0)) {
+        core_emit<true, true, true>(k, cb, s, lmul(k.f_ScS, S_.xx), lmul(k.f_ScS, S_.yy), lmul(k.f_ScS2, S_.xy), P.f,
+                                    P.h, fo, ho, R(1));
+    } else {
+        R Qxx, Qyy, Q2;
+        shear_form<true>(k, cb, s.ux, s.uy, s.Fx, s.Fy, S_, Qxx, Qyy, Q2);
+        core_emit<true, true>(k, cb, s, Qxx, Qyy, Q2, P.f, P.h, fo, ho, R(1));
+    }
     if (!lfinite(ho[0])) atomicOr(k.flag, 1);
 }
 
