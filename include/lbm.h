@@ -314,8 +314,9 @@ lbm_status lbm_set_state(lbm_handle* h, const double* f, const double* g, int on
  *                       needs a porosity field set by lbm_set_fields),
  *   dloss_dTbc[4]       d loss / d (Dirichlet wall temperature) per side
  *                       W, E, S, N (host; NULL allowed).
- * States are recomputed from checkpoints kept every `segment` steps
- * (0 = ceil(sqrt(n_steps))): memory for about 2 sqrt(n_steps) states is
+ * States are recomputed from checkpoints kept every `segment` steps (0 =
+ * ceil(sqrt(n_steps)), or every state kept while n_steps states take at most
+ * 256 MB): memory for about 2 sqrt(n_steps) states, or those 256 MB, is
  * allocated on the handle's stream for the duration of the call and freed
  * before it returns.  FP64 or FP32 storage; the adjoint arithmetic is that of
  * the storage type, the gradients are accumulated in FP64.  The derivatives

@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lbm_core.cuh"
@@ -285,18 +286,19 @@ __device__ __forceinline__ R porosity_adjoint(const KConst<R>& k, R ie, const Ce
 // theirs in Vff.
 template <class R>
 __device__ __forceinline__ R pending_ff(const KConst<R>& k, const R* __restrict__ Vff, int sx, int sy) {
-    const bool wW = k.bc[SW] != BC_PERIODIC, wE = k.bc[SE] != BC_PERIODIC, wS = k.bc[SS] != BC_PERIODIC,
-               wN = k.bc[SN] != BC_PERIODIC;
+    const bool wW = k.bc[SW] != BC_PERIODIC, wS = k.bc[SS] != BC_PERIODIC;
     if (!wW) sx = sx < 0 ? sx + k.nx : (sx >= k.nx ? sx - k.nx : sx);
     if (!wS) sy = sy < 0 ? sy + k.ny : (sy >= k.ny ? sy - k.ny : sy);
     const bool inx = wW ? sx >= 1 && sx <= k.nx - 2 : true, iny = wS ? sy >= 1 && sy <= k.ny - 2 : true;
     if (!inx || !iny) return R(0);
     R v = R(0);
-    const bool W2 = wW && sx == 2, E2 = wE && sx == k.nx - 3, S2 = wS && sy == 2, N2 = wN && sy == k.ny - 3;
+    const bool W2 = k.bc[SW] == BC_ADIABATIC && sx == 2, E2 = k.bc[SE] == BC_ADIABATIC && sx == k.nx - 3;
+    const bool S2 = k.bc[SS] == BC_ADIABATIC && sy == 2, N2 = k.bc[SN] == BC_ADIABATIC && sy == k.ny - 3;
     if (W2) v += Vff[at_of(k, 0, sy)];
     if (E2) v += Vff[at_of(k, k.nx - 1, sy)];
     if (S2) v += Vff[at_of(k, sx, 0)];
     if (N2) v += Vff[at_of(k, sx, k.ny - 1)];
+    // a corner is adiabatic when both its walls are
     if (W2 && S2) v += Vff[at_of(k, 0, 0)];
     if (E2 && S2) v += Vff[at_of(k, k.nx - 1, 0)];
     if (W2 && N2) v += Vff[at_of(k, 0, k.ny - 1)];
@@ -321,33 +323,79 @@ __device__ __forceinline__ void load_lambda(const KConst<R>& k, const R* __restr
     }
 }
 
+// Interior nodes (columns x0 .. x0 + nxi - 1, rows likewise), those beside a wall
+// (the ring: S and N rows, then the W and E columns without them) and the
+// others numbered apart; x, y hold x0, y0 on entry.
+struct Interior {
+    bool wx, wy;
+    int nxi, nyi, rows, cols;  // rows, cols: without the ring
+    template <class R>
+    __host__ __device__ explicit Interior(const KConst<R>& k)
+        : wx(k.bc[SW] != BC_PERIODIC), wy(k.bc[SS] != BC_PERIODIC), nxi(k.nx - (wx ? 2 : 0)), nyi(k.ny - (wy ? 2 : 0)),
+          rows(nyi - (wy ? 2 : 0)), cols(nxi - (wx ? 2 : 0)) {}
+    __host__ __device__ int ring() const { return (wy ? 2 * nxi : 0) + (wx ? 2 * rows : 0); }
+    __host__ __device__ long long inner() const { return (long long)rows * cols; }
+    __device__ __forceinline__ void ring_node(int n, int& x, int& y) const {
+        if (wy) {
+            if (n < nxi) { x += n; return; }
+            n -= nxi;
+            if (n < nxi) { x += n; y += nyi - 1; return; }
+            n -= nxi;
+        }
+        y += (wy ? 1 : 0) + (n < rows ? n : n - rows);
+        if (n >= rows) x += nxi - 1;
+    }
+    __device__ __forceinline__ void inner_node(long long n, int& x, int& y) const {
+        const int r = (int)(n / cols);
+        x += (wx ? 1 : 0) + (int)(n - (long long)r * cols);
+        y += (wy ? 1 : 0) + r;
+    }
+};
+
 // One adjoint step.  state: s_n; lam, Vff: adjoints of s_{n+1}; lam_prev,
 // Vff_prev: those of s_n (places no interior node pulls are never written and
-// stay 0).  Threads run over the interior nodes, x fastest.  ff: some wall is
-// adiabatic.  early: the state was complete before the previous launch began,
-// so it may be read before the grid dependency is resolved.
+// stay 0).  ff: some wall is adiabatic.  early: the state was complete before
+// the previous launch began, so it may be read before the grid dependency is
+// resolved.
+// The first ring_blocks blocks take the nodes beside a wall, 32 a block: their
+// first warp the node's own collision, their second one those of the wall nodes
+// it feeds, at the same time (in one thread the second chain follows the first,
+// and every warp of a small lattice holds such a node); the first warp adds
+// the two and goes on.  The other blocks take 64 nodes.
 // Bound: 256^2 FP32 fits L2 and one wave of warps; the step takes about the
-// latency of its chain (loads, ~700 dependent operations, stores).  Blocks of
-// 64 threads (32 in FP64, whose pipe serves two lanes a cycle and SM) spread
-// small lattices over more SMs.  Before, 9 to 11 forward-mode passes a node in
-// a thread each, then a combining and a gathering launch: whole calls with 256
-// steps at 256^2 FP32 took 38.0 ms against 8.8 ms, with 100 steps at 65 x 49
-// FP64 45.7 against 10.8 ms (forward and recomputed steps included).
-template <class R> struct AdjLaunch { static constexpr int block = 64, blocks = 8; };
-template <> struct AdjLaunch<double> { static constexpr int block = 32, blocks = 8; };
+// latency of its chain (loads, ~600 dependent operations, stores).  Before, 9
+// to 11 forward-mode passes a node in a thread each, then a combining and a
+// gathering launch: whole calls with 256 steps at 256^2 FP32 took 38.0 ms
+// against 7.0 ms, with 100 steps at 65 x 49 FP64 45.7 against 6.6 ms (forward and
+// recomputed steps included; 7.5 and 8.4 ms with the wall nodes' chains in the
+// threads of the nodes they hang on).
+constexpr int kAdjNodes = 64, kAdjRing = 32;
+template <class R> struct AdjLaunch { static constexpr int blocks = 8; };
+template <> struct AdjLaunch<double> { static constexpr int blocks = 4; };
 
 template <class R, class S, bool TAU1>
-__global__ void __launch_bounds__(AdjLaunch<R>::block, AdjLaunch<R>::blocks)
+__global__ void __launch_bounds__(kAdjNodes, AdjLaunch<R>::blocks)
 k_adj_step(const __grid_constant__ KConst<R> k, const S* __restrict__ state, const R* __restrict__ lam,
            const R* __restrict__ Vff, R* __restrict__ lam_prev, R* __restrict__ Vff_prev, double* __restrict__ g_eps,
-           double* __restrict__ g_tb, bool ff, bool early) {
+           double* __restrict__ g_tb, int ring_blocks, bool ff, bool early) {
+    constexpr int kShared = TAU1 ? 10 : 27;
+    __shared__ R part[kShared][kAdjRing];  // what the wall nodes add, per node of the ring
     if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const bool wx = k.bc[SW] != BC_PERIODIC, wy = k.bc[SS] != BC_PERIODIC;
-    const int x0 = wx ? 1 : 0, y0 = wy ? 1 : 0, nxi = k.nx - 2 * x0, nyi = k.ny - 2 * y0;
-    const long long n = (long long)blockIdx.x * AdjLaunch<R>::block + threadIdx.x;
-    const bool live = n < (long long)nxi * nyi;
-    const int yi = live ? (int)(n / nxi) : 0;
-    const int x = x0 + (live ? (int)(n - (long long)yi * nxi) : 0), y = y0 + yi;
+    const Interior in(k);
+    const bool ring = (int)blockIdx.x < ring_blocks;
+    const bool walls = ring && threadIdx.x >= kAdjRing;  // this thread's role
+    const int slot = threadIdx.x & (kAdjRing - 1);
+    int x = in.wx ? 1 : 0, y = in.wy ? 1 : 0;
+    bool live;
+    if (ring) {
+        const int n = (int)blockIdx.x * kAdjRing + slot;
+        live = n < in.ring();
+        if (live) in.ring_node(n, x, y);
+    } else {
+        const long long n = (long long)((int)blockIdx.x - ring_blocks) * kAdjNodes + threadIdx.x;
+        live = n < in.inner();
+        if (live) in.inner_node(n, x, y);
+    }
     Pops<R> P;
     pull(k, state, x, y, P);
     const AdjState<R> s = adjoint_state(k, node_eps(k, x, y), row_ay(k, y), P.f, P.h);
@@ -355,21 +403,27 @@ k_adj_step(const __grid_constant__ KConst<R> k, const S* __restrict__ state, con
     // only now may the next step's blocks start: their early reads then come
     // after the launch before this one
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!live) return;
     StateBar<R> B = {};
     CellBar<R> C = {};
     R lf[9], lh[9], vf[9], vh[9];
-    load_lambda(k, lam, Vff, ff, x, y, lf, lh);
-    emit_adjoint<true>(k, s.ie, R(1) - k.omf, R(1) - k.omT, s.ux, s.uy, s.Fx, s.Fy, s.ep, s.T, s.gx, s.gy, lf, lh, B, C);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        vf[i] = TAU1 ? R(0) : k.omf * lf[i];
-        vh[i] = TAU1 ? R(0) : k.omT * lh[i];
+    for (int i = 0; i < 9; ++i) vf[i] = vh[i] = R(0);
+    if (live && !walls) {
+        load_lambda(k, lam, Vff, ff, x, y, lf, lh);
+        emit_adjoint<true>(k, s.ie, TAU1 ? R(1) : R(1) - k.omf, TAU1 ? R(1) : R(1) - k.omT, s.ux, s.uy, s.Fx, s.Fy, s.ep,
+                           s.T, s.gx, s.gy, lf, lh, B, C);
+        if constexpr (!TAU1) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                vf[i] = k.omf * lf[i];
+                vh[i] = k.omT * lh[i];
+            }
+        }
     }
-    // wall nodes whose x_f this node is
-    const int bx = wx && x == 1 ? 0 : (wx && x == k.nx - 2 ? k.nx - 1 : -1);
-    const int by = wy && y == 1 ? 0 : (wy && y == k.ny - 2 ? k.ny - 1 : -1);
-    if (bx >= 0 || by >= 0) {
+    if (live && walls) {
+        // the wall nodes whose x_f this node is
+        const int bx = in.wx && x == 1 ? 0 : (in.wx && x == k.nx - 2 ? k.nx - 1 : -1);
+        const int by = in.wy && y == 1 ? 0 : (in.wy && y == k.ny - 2 ? k.ny - 1 : -1);
 #pragma unroll 1
         for (int m = 0; m < 3; ++m) {
             const int X = m == 1 ? x : bx, Y = m == 0 ? y : by;  // W/E side, S/N side, corner
@@ -429,7 +483,32 @@ k_adj_step(const __grid_constant__ KConst<R> k, const S* __restrict__ state, con
                 }
             }
         }
+        R* o = &part[0][slot];
+        const R v[10] = {B.th, B.ep, B.Sxx, B.Syy, B.Sxy, B.gx, B.gy, C.ie, B.ux, B.uy};
+#pragma unroll
+        for (int q = 0; q < 10; ++q) o[q * kAdjRing] = v[q];
+        if constexpr (!TAU1) {
+#pragma unroll
+            for (int i = 1; i < 9; ++i) o[(9 + i) * kAdjRing] = vf[i];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) o[(18 + i) * kAdjRing] = vh[i];
+        }
     }
+    if (ring) {
+        __syncthreads();
+        if (walls) return;
+        const R* o = &part[0][slot];
+        R* b[10] = {&B.th, &B.ep, &B.Sxx, &B.Syy, &B.Sxy, &B.gx, &B.gy, &C.ie, &B.ux, &B.uy};
+#pragma unroll
+        for (int q = 0; q < 10; ++q) *b[q] += live ? o[q * kAdjRing] : R(0);
+        if constexpr (!TAU1) {
+#pragma unroll
+            for (int i = 1; i < 9; ++i) vf[i] += live ? o[(9 + i) * kAdjRing] : R(0);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) vh[i] += live ? o[(18 + i) * kAdjRing] : R(0);
+        }
+    }
+    if (!live) return;
     const SumsBar<R> m = moments_adjoint(k, s, B, C);
     if (k.eps_field) g_eps[(long long)y * k.nx + x] += double(porosity_adjoint(k, s.ie, C));
     // pulled value i of this node came from (x, y) - c_i
@@ -471,13 +550,14 @@ __global__ void k_adj_seed(const __grid_constant__ KConst<R> k, const double* __
 template <class R, class S>
 cudaError_t launch_adj_step(const KConst<R>& k, const S* state, const R* lam, const R* Vff, R* lam_prev, R* Vff_prev,
                             double* g_eps, double* g_tb, bool early, cudaStream_t st) {
-    const int wx = k.bc[SW] != BC_PERIODIC ? 1 : 0, wy = k.bc[SS] != BC_PERIODIC ? 1 : 0;
-    const long long n = (long long)(k.nx - 2 * wx) * (k.ny - 2 * wy);
+    const Interior in(k);
+    const int ring_blocks = (in.ring() + kAdjRing - 1) / kAdjRing;
+    const long long blocks = ring_blocks + (in.inner() + kAdjNodes - 1) / kAdjNodes;
     bool ff = false;
     for (int s = 0; s < 4; ++s) ff = ff || k.bc[s] == BC_ADIABATIC;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n + AdjLaunch<R>::block - 1) / AdjLaunch<R>::block));
-    cfg.blockDim = dim3(AdjLaunch<R>::block);
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kAdjNodes);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -485,8 +565,8 @@ cudaError_t launch_adj_step(const KConst<R>& k, const S* state, const R* lam, co
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (k.omf == R(0) && k.omT == R(0))
-        return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, true>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ff, early);
-    return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, false>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ff, early);
+        return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, true>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ring_blocks, ff, early);
+    return cudaLaunchKernelEx(&cfg, k_adj_step<R, S, false>, k, state, lam, Vff, lam_prev, Vff_prev, g_eps, g_tb, ring_blocks, ff, early);
 }
 
 template <class R>
@@ -531,15 +611,38 @@ HostWall host_classify(const lbm_params& p, int x, int y) {
 
 namespace {
 
+// lbm_adjoint keeps every state (segment = 0) while together they take no more.
+constexpr size_t kKeepBytes = (size_t)256 << 20;
+
+// Steps that one launch takes of the next `left`: two on FP32 lattices that have
+// the two-step kernel.
+template <class S>
+int64_t steps_of_launch(const lbm_handle* h, int64_t left) {
+    return std::is_same<S, float>::value && h->two_steps && left >= 2 ? 2 : 1;
+}
+// m = 1 or 2 steps from src to dst; with two, the state between them to mid
+// (or nowhere, if null).
+template <class R, class S>
+cudaError_t launch_steps(const lbm_handle* h, const lbm::KConst<R>& k, int64_t m, const S* src, S* mid, S* dst,
+                         int64_t step, cudaStream_t st) {
+    if constexpr (std::is_same<S, float>::value)
+        if (m == 2) return lbm::launch_two_steps(k, src, mid, dst, (uint32_t)(step / 2), h->sms, st);
+    return lbm::launch_step(k, src, dst, (uint32_t)step, st);
+}
+
 template <class R, class S>
 lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_t seg_len, int side, double* loss,
                        double* dloss_deps, double* dloss_dTbc) {
     cudaStream_t st = h->stream;
     const lbm_params& p = h->prm;
     const size_t N = (size_t)p.nx * p.ny;
-    const int64_t K = seg_len > 0 ? seg_len : (int64_t)ceil(sqrt((double)n));
+    const size_t sb = h->L.buf_bytes;  // one state
+    // few and small states are all kept as the forward pass computes them, and
+    // nothing is recomputed (65 x 49 FP64, 100 steps: 4.7 ms a call
+    // against 5.7 with checkpoints)
+    const bool keep = seg_len == 0 && (double)sb * (double)n <= (double)kKeepBytes;
+    const int64_t K = keep ? n : (seg_len > 0 ? seg_len : (int64_t)ceil(sqrt((double)n)));
     const int64_t nseg = (n + K - 1) / K;
-    const size_t sb = h->L.buf_bytes;                               // one state
     const size_t lam_bytes = 17 * (size_t)k.plane * sizeof(R);    // one adjoint state
     std::vector<void*> allocs;
     auto fail_free = [&](lbm_status s, const std::string& m) {
@@ -553,7 +656,7 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
         allocs.push_back(a);
         return a;
     };
-    char* ckpt = (char*)alloc(sb * (size_t)nseg);
+    char* ckpt = (char*)alloc(keep ? 256 : sb * (size_t)nseg);
     char* segs = (char*)alloc(sb * (size_t)K);
     R* lam0 = (R*)alloc(lam_bytes);
     R* lam1 = (R*)alloc(lam_bytes);
@@ -571,15 +674,23 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
 
     // forward, keeping a checkpoint at the start of every segment
     const int64_t step0 = h->steps;
-    for (int64_t t = 0; t < n; ++t) {
+    auto kept = [&](int64_t t) { return (S*)(segs + sb * (size_t)t); };  // state t of the segment in hand
+    for (int64_t t = 0; t < n;) {
         if (t % K == 0)
-            if (cudaMemcpyAsync(ckpt + sb * (size_t)(t / K), h->buf(h->cur), sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            if (cudaMemcpyAsync(keep ? segs : ckpt + sb * (size_t)(t / K), h->buf(h->cur), sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
                 return fail_free(LBM_ERR_CUDA, "checkpoint copy");
-        cudaError_t e = lbm::launch_step(k, (const S*)h->buf(h->cur), (S*)h->buf(1 - h->cur), (uint32_t)(step0 + t), st);
+        // as many steps as one launch takes, up to the next checkpoint
+        const int64_t m = steps_of_launch<S>(h, std::min(K - t % K, n - t));
+        const bool last = t + m == n;  // the handle ends at step n
+        cudaError_t e = keep ? launch_steps(h, k, m, (const S*)kept(t), m == 2 ? kept(t + 1) : (S*)nullptr,
+                                            last ? (S*)h->buf(1 - h->cur) : kept(t + m), step0 + t, st)
+                             : launch_steps(h, k, m, (const S*)h->buf(h->cur), (S*)nullptr, (S*)h->buf(1 - h->cur),
+                                            step0 + t, st);
         if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, std::string("step kernel: ") + cudaGetErrorString(e));
-        h->cur = 1 - h->cur;
-        ++h->steps;
+        if (!keep || last) h->cur = 1 - h->cur;
+        h->steps += m;
         ++h->launches;
+        t += m;
     }
     // loss
     cudaError_t e = lbm::launch_nusselt(k, h->diag, (const S*)h->buf(h->cur), side, h->nu(), h->out(), st);
@@ -622,16 +733,17 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
     R* ln = lam1;
     for (int64_t sgi = nseg - 1; sgi >= 0; --sgi) {
         const int64_t t0 = sgi * K, len = std::min<int64_t>(K, n - t0);
-        if (cudaMemcpyAsync(segs, ckpt + sb * (size_t)sgi, sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        if (!keep && cudaMemcpyAsync(segs, ckpt + sb * (size_t)sgi, sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
             return fail_free(LBM_ERR_CUDA, "checkpoint restore");
-        for (int64_t t = 1; t < len; ++t) {
-            e = lbm::launch_step(k, (const S*)(segs + sb * (size_t)(t - 1)), (S*)(segs + sb * (size_t)t),
-                                 (uint32_t)(step0 + t0 + t - 1), st);
+        for (int64_t t = keep ? len : 1; t < len;) {
+            const int64_t m = steps_of_launch<S>(h, len - t);
+            e = launch_steps(h, k, m, (const S*)kept(t - 1), m == 2 ? kept(t) : (S*)nullptr, kept(t + m - 1), step0 + t0 + t - 1, st);
             if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, "recompute step");
+            t += m;
         }
         for (int64_t t = len - 1; t >= 0; --t) {
             // the first launch after the recomputation waits before it reads the state
-            e = lbm::launch_adj_step(k, (const S*)(segs + sb * (size_t)t), lc, ff0, ln, ff1, g_eps, g_tb, t < len - 1, st);
+            e = lbm::launch_adj_step(k, (const S*)kept(t), lc, ff0, ln, ff1, g_eps, g_tb, keep || t < len - 1, st);
             if (e != cudaSuccess) return fail_free(LBM_ERR_CUDA, std::string("adjoint kernel: ") + cudaGetErrorString(e));
             std::swap(lc, ln);
             std::swap(ff0, ff1);

@@ -376,7 +376,7 @@ lbm_status lbm_step(lbm_handle* h, int64_t n) {
     for (int64_t i = 0; i < n; ++i) {
         const int src = h->cur, dst = 1 - h->cur;
         if (h->two_steps && n - i >= 2) {
-            const cudaError_t e = lbm::launch_two_steps(h->k32, (const float*)h->buf(src), (float*)h->buf(dst),
+            const cudaError_t e = lbm::launch_two_steps(h->k32, (const float*)h->buf(src), nullptr, (float*)h->buf(dst),
                                                         (uint32_t)h->launches, h->sms, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "two-step kernel");
             h->cur = dst;

@@ -132,10 +132,12 @@ template <class S>
 cudaError_t launch_step_tma(const KConst<float>& k, const CUtensorMap& tm, const S* src, S* dst, int rows,
                             uint32_t step, cudaStream_t st);
 // Two steps of an FP32 lattice in one launch (lbm_tile.cu; lattices of at
-// least 8 x 8 nodes, any sides); `launch` alternates the sweep's direction,
+// least 8 x 8 nodes, any sides) from src to dst; mid (or nullptr) receives the
+// state between them; `launch` alternates the sweep's direction,
 // sms: multiprocessors of the device.
 bool two_steps_supported(const KConst<float>& k);
-cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* dst, uint32_t launch, int sms, cudaStream_t st);
+cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* mid, float* dst, uint32_t launch, int sms,
+                             cudaStream_t st);
 // Work item of the staged batched step: the band of 128 columns from x0 and
 // the segment of rows from y0 of a cavity ny rows high.
 struct StagedItem {

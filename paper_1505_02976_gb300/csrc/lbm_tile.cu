@@ -85,7 +85,8 @@ struct TileSource {
 };
 
 template <bool TAU1>
-__device__ __noinline__ void tile_wall_1(const KConst<float>& k, const float* __restrict__ src, float* slot, int x, int y) {
+__device__ __noinline__ void tile_wall_1(const KConst<float>& k, const float* __restrict__ src, float* slot, float* mid,
+                                         int x, int y) {
     float fo[9], ho[9];
     if constexpr (TAU1) wall_node_tau1(k, GlobalSource<float, float>{src}, x, y, fo, ho);
     else wall_node_generic(k, GlobalSource<float, float>{src}, x, y, fo, ho);
@@ -93,6 +94,7 @@ __device__ __noinline__ void tile_wall_1(const KConst<float>& k, const float* __
     for (int i = 1; i < 9; ++i) slot[(i - 1) * kTileCols] = fo[i];
 #pragma unroll
     for (int i = 0; i < 9; ++i) slot[(8 + i) * kTileCols] = ho[i];
+    if (mid) store_node(k, mid, (long long)y * k.pitch + x, fo, ho);
 }
 
 template <bool TAU1>
@@ -131,10 +133,11 @@ struct TileWalls {
 };
 
 // Two steps of one tile: output columns X0 .. X1 - 1 (X0 even), rows Y0 .. Y1 - 1.
+// mid (or nullptr): where the state after the first step goes as well.
 template <bool EPS_FIELD, bool TAU1>
 __device__ __forceinline__ void tile_two_steps(const KConst<float>& k, const PairConst& pc, const float* __restrict__ src,
-                                               float* __restrict__ dst, float* slots, int X0, int X1, int Y0, int Y1,
-                                               int warps, bool hot) {
+                                               float* __restrict__ mid, float* __restrict__ dst, float* slots,
+                                               int X0, int X1, int Y0, int Y1, int warps, bool hot) {
     // the first `warps` warps take the rows; the others, if there are any, the wall nodes
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int wall_threads = (int)blockDim.x > 32 * warps ? (int)blockDim.x - 32 * warps : (int)blockDim.x;
@@ -196,6 +199,21 @@ __device__ __forceinline__ void tile_two_steps(const KConst<float>& k, const Pai
             }
             core_interior<TAU1>(pc, c, eps_ay(k, pc, c, y), f, h, fo, ho);
             if ((va && !lfinite(ho[0].x)) || (vb && !lfinite(ho[0].y))) atomicOr(k.flag, 1);
+            if (mid && yy >= Y0 && yy < Y1) {
+                float* m = mid + (y * pitch + x);
+                if (va && x >= X0) {
+#pragma unroll
+                    for (int i = 1; i < 9; ++i) m[(i - 1) * pl] = fo[i].x;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) m[(8 + i) * pl] = ho[i].x;
+                }
+                if (vb && x + 1 < X1) {
+#pragma unroll
+                    for (int i = 1; i < 9; ++i) m[(i - 1) * pl + 1] = fo[i].y;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) m[(8 + i) * pl + 1] = ho[i].y;
+                }
+            }
             float* d = slots + (yy - Y0 + 1) * kTileRowElems + 2 * lane;
             if (va && vb) {
 #pragma unroll
@@ -216,9 +234,10 @@ __device__ __forceinline__ void tile_two_steps(const KConst<float>& k, const Pai
             int X, Y;
             W.at(n, X, Y);
             float* slot = slots + (Y - Y0 + 1) * kTileRowElems + (X - X0 + 1);
+            float* own = X >= X0 && X < X1 && Y >= Y0 && Y < Y1 ? mid : nullptr;
             if (!wx) X = X < 0 ? X + nx : (X >= nx ? X - nx : X);
             if (!wy) Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
-            tile_wall_1<TAU1>(k, src, slot, X, Y);
+            tile_wall_1<TAU1>(k, src, slot, own, X, Y);
         }
     }
     __syncthreads();
@@ -299,17 +318,22 @@ struct TileSplit {
 
 template <bool EPS_FIELD, bool TAU1>
 __global__ void __launch_bounds__(kTileMaxThreads, 2)
-k_tile(const __grid_constant__ KConst<float> k, const __grid_constant__ PairConst pc, const float* __restrict__ src, float* __restrict__ dst, TileSplit sx,
-       TileSplit sy, int warps, uint32_t launch) {
+k_tile(const __grid_constant__ KConst<float> k, const __grid_constant__ PairConst pc, const float* __restrict__ src, float* __restrict__ mid,
+       float* __restrict__ dst, TileSplit sx, TileSplit sy, int warps, bool early, uint32_t launch) {
     extern __shared__ __align__(16) float slots[];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // early: let the next launch's blocks in as soon as this one's have all
+    // started.  Small lattices' blocks do it only once the previous launch is
+    // done: otherwise a queue of later launches takes their places on the SMs
+    // (128^2 2.9 -> 2.6 us a step; 2048^2 58 -> 60, so large ones keep it).
+    if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // bottom-up and top-down in turn, so that a launch first reads the rows
     // the previous one wrote last, while they are in L2
     const int by = (launch & 1u) ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
     const int X0 = sx.begin(blockIdx.x), X1 = sx.begin(blockIdx.x + 1), Y0 = sy.begin(by), Y1 = sy.begin(by + 1);
     const bool hot = (long long)(gridDim.y - blockIdx.y) * (Y1 - Y0) * k.nx <= k.l2_hot;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    tile_two_steps<EPS_FIELD, TAU1>(k, pc, src, dst, slots, X0, X1, Y0, Y1, warps, hot);
+    if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    tile_two_steps<EPS_FIELD, TAU1>(k, pc, src, mid, dst, slots, X0, X1, Y0, Y1, warps, hot);
 }
 
 // The fewest tiles of at most `most` units.
@@ -334,17 +358,17 @@ static cudaError_t allow_tile_smem() {
 }
 
 template <bool E, bool T>
-static cudaError_t launch_tile(cudaLaunchConfig_t& cfg, const KConst<float>& k, const float* src, float* dst,
-                               const TileSplit& sx, const TileSplit& sy, int warps, uint32_t launch) {
+static cudaError_t launch_tile(cudaLaunchConfig_t& cfg, const KConst<float>& k, const float* src, float* mid,
+                               float* dst, const TileSplit& sx, const TileSplit& sy, int warps, bool early, uint32_t launch) {
     cudaError_t e = allow_tile_smem<E, T>();
     if (e != cudaSuccess) return e;
     const PairConst pc = make_pair_const(k, 1.0f);
-    return cudaLaunchKernelEx(&cfg, k_tile<E, T>, k, pc, src, dst, sx, sy, warps, launch);
+    return cudaLaunchKernelEx(&cfg, k_tile<E, T>, k, pc, src, mid, dst, sx, sy, warps, early, launch);
 }
 
 bool two_steps_supported(const KConst<float>& k) { return k.nx >= 8 && k.ny >= 8; }
 
-cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* dst, uint32_t launch, int sms,
+cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* mid, float* dst, uint32_t launch, int sms,
                              cudaStream_t st) {
     if (!two_steps_supported(k)) return cudaErrorInvalidValue;
     const TileSplit sx = tile_split(k.nx, 2, kTilePairs);
@@ -352,6 +376,7 @@ cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* ds
     const TileShape shape = small ? kTileSmall : kTileLarge;
     const TileSplit sy = tile_split(k.ny, 1, shape.rows);
     const int warps = shape.warps;
+    const bool early = !small;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)sx.n, (unsigned)sy.n);
     cfg.blockDim = dim3((unsigned)(32 * (shape.warps + shape.wall_warps)));
@@ -363,8 +388,8 @@ cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* ds
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const bool tau1 = k.omf == 0.f && k.omT == 0.f;
-    if (k.eps_field) return tau1 ? launch_tile<true, true>(cfg, k, src, dst, sx, sy, warps, launch) : launch_tile<true, false>(cfg, k, src, dst, sx, sy, warps, launch);
-    return tau1 ? launch_tile<false, true>(cfg, k, src, dst, sx, sy, warps, launch) : launch_tile<false, false>(cfg, k, src, dst, sx, sy, warps, launch);
+    if (k.eps_field) return tau1 ? launch_tile<true, true>(cfg, k, src, mid, dst, sx, sy, warps, early, launch) : launch_tile<true, false>(cfg, k, src, mid, dst, sx, sy, warps, early, launch);
+    return tau1 ? launch_tile<false, true>(cfg, k, src, mid, dst, sx, sy, warps, early, launch) : launch_tile<false, false>(cfg, k, src, mid, dst, sx, sy, warps, early, launch);
 }
 
 }  // namespace lbm
