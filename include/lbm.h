@@ -358,7 +358,8 @@ int64_t lbm_kernel_launches(const lbm_handle* h);
 typedef struct lbm_batch lbm_batch;
 
 typedef enum {
-    LBM_BATCH_FUSED = 0,     /* one kernel launch per step for all cavities */
+    LBM_BATCH_FUSED = 0,     /* one kernel launch per step for all cavities (per two steps
+                                of a staged batch whose cavities have 8 x 8 nodes or more) */
     LBM_BATCH_GRAPH = 1,     /* the same launches replayed from a captured CUDA graph
                                 (50 steps per graph; needs a non-default stream) */
     LBM_BATCH_PER_CASE = 2,  /* one single-lattice launch per cavity per step */
@@ -430,7 +431,8 @@ lbm_status lbm_batch_moments(lbm_batch* b, int32_t cavity, double* p, double* ux
 
 int64_t lbm_batch_steps_done(const lbm_batch* b);
 
-/* Kernel launches issued for steps (a graph replay counts its 50 launches). */
+/* Kernel launches issued for steps (a graph replay counts its launches: 50, or
+ * 25 of two steps). */
 int64_t lbm_batch_kernel_launches(const lbm_batch* b);
 
 /* As lbm_check_guards, for the batch workspace (both population buffers,

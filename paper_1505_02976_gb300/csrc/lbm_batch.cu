@@ -19,7 +19,7 @@ namespace {
 
 thread_local std::string g_batch_create_error;
 constexpr int kTiles[3] = {32, 64, 128};
-constexpr int kGraphChunk = 50;  // steps per captured graph (even: the ping-pong parity returns)
+constexpr int kGraphChunk = 50;  // steps per captured graph
 constexpr int kMaxGrid = 1 << 16;
 constexpr double kWallCost = 4.0;  // a packed wall node costs about 4 interior nodes (out-of-line path)
 
@@ -56,6 +56,11 @@ struct lbm_batch {
     // cavity, segment-major), the per-cavity layout of that list, and the
     // per-item step counters and abort word of a call
     size_t off_pitems, off_pcav, off_done;
+    // two steps per launch (staged batches whose cavities have 8 x 8 nodes or
+    // more): the tiles and the packed constants
+    size_t off_titems, off_pair;
+    int n_titems;
+    bool all_tau1;
     std::vector<size_t> guards;        // offsets of the guard words after each region
     int n_sitems;
     std::vector<CUtensorMap> hmaps[2];
@@ -73,6 +78,7 @@ struct lbm_batch {
     const lbm::StagedItem* sitems() const { return (const lbm::StagedItem*)(ws + off_sitems); }
     const lbm::StagedItem* pitems() const { return (const lbm::StagedItem*)(ws + off_pitems); }
     const lbm::PersistCavity* pcav() const { return (const lbm::PersistCavity*)(ws + off_pcav); }
+    const lbm::TileItem* titems() const { return (const lbm::TileItem*)(ws + off_titems); }
     int* done() const { return (int*)(ws + off_done); }
     size_t es() const { return precision == LBM_F64 ? 8 : 4; }
 };
@@ -176,6 +182,17 @@ std::vector<lbm::StagedItem> make_persist_items(const std::vector<lbm_params>& p
     return v;
 }
 
+// Tiles of the two-step launch, cavity by cavity; none if a cavity is too small.
+std::vector<lbm::TileItem> make_tile_items(const std::vector<lbm_params>& prm) {
+    std::vector<lbm::TileItem> v;
+    for (int c = 0; c < (int)prm.size(); ++c) {
+        if (prm[c].nx < 8 || prm[c].ny < 8) return {};
+        const std::vector<lbm::TileItem> one = lbm::tile_items(c, prm[c].nx, prm[c].ny);
+        v.insert(v.end(), one.begin(), one.end());
+    }
+    return v;
+}
+
 // Block ranges of equal estimated cost: bounds[k] is the first item of block k.
 std::vector<int> make_bounds(const std::vector<double>& cum, int grid) {
     const int n = (int)cum.size() - 1;
@@ -233,7 +250,10 @@ lbm_status batch_layout(const lbm_params* p, int n, lbm_batch* b, std::string* w
     }
     b->off_bounds = take((size_t)(kMaxGrid + 1) * sizeof(int));
     b->n_sitems = 0;
-    b->off_maps = b->off_sitems = b->off_pitems = b->off_pcav = b->off_done = o;
+    b->off_maps = b->off_sitems = b->off_pitems = b->off_pcav = b->off_done = b->off_titems = b->off_pair = o;
+    b->n_titems = 0;
+    b->all_tau1 = true;
+    for (int c = 0; c < n; ++c) b->all_tau1 = b->all_tau1 && p[c].tau_f == 1.0 && p[c].tau_T == 1.0;
     if (stageable(b->prm)) {
         const size_t ns = make_staged_items(b->prm, lbm::tma_batch_rows()).size();
         if (ns >= (size_t)1 << 31) { *why = "batch too large"; return LBM_ERR_ARG; }
@@ -243,6 +263,11 @@ lbm_status batch_layout(const lbm_params* p, int n, lbm_batch* b, std::string* w
         b->off_pitems = take(ns * sizeof(lbm::StagedItem));
         b->off_pcav = take((size_t)n * sizeof(lbm::PersistCavity));
         b->off_done = take((ns + 1) * sizeof(int));
+        b->n_titems = (int)make_tile_items(b->prm).size();
+        if (b->n_titems > 0) {
+            b->off_titems = take((size_t)b->n_titems * sizeof(lbm::TileItem));
+            b->off_pair = take((size_t)n * lbm::pair_const_bytes());
+        }
     }
     b->off_fields = take(4 * b->max_cells * sizeof(double));
     b->off_nu = take((size_t)n * sizeof(double));
@@ -306,6 +331,17 @@ cudaError_t fused_step(lbm_batch* b, int tile_x, int grid) {
     });
 }
 
+// Steps that the next fused launch takes of the `left` ones.
+int steps_of_launch(const lbm_batch* b, int64_t left) { return b->staged && b->n_titems > 0 && left >= 2 ? 2 : 1; }
+
+// One fused launch of m = steps_of_launch() steps.
+cudaError_t fused_steps(lbm_batch* b, int m, int tile_x, int grid) {
+    if (m == 1) return fused_step(b, tile_x, grid);
+    return lbm::launch_two_steps_batch((const lbm::BatchCavity<float>*)(b->ws + b->off_cav), b->ws + b->off_pair,
+                                       b->titems(), b->n_titems, b->all_tau1, (const float*)b->buf(b->cur),
+                                       (float*)b->buf(1 - b->cur), b->stream);
+}
+
 cudaError_t per_case_step(lbm_batch* b) {
     const int src = b->cur, dst = 1 - b->cur;
     if (b->staged) {
@@ -345,10 +381,12 @@ lbm_status capture(lbm_batch* b, int start) {
     cudaGraph_t g = nullptr;
     LBM_BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < kGraphChunk && e == cudaSuccess; ++i) {
-        e = fused_step(b, b->tile_x, b->grid);
+    for (int i = 0; i < kGraphChunk && e == cudaSuccess;) {
+        const int m = steps_of_launch(b, kGraphChunk - i);
+        e = fused_steps(b, m, b->tile_x, b->grid);
         b->cur = 1 - b->cur;
-        ++b->steps;
+        b->steps += m;
+        i += m;
     }
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     b->cur = saved_cur;
@@ -454,6 +492,13 @@ lbm_status lbm_batch_create(const lbm_params* p, int32_t n, void* stream, void* 
             if (s == LBM_OK && (int)pit.size() != b->n_sitems) s = bfail(b, LBM_ERR_ARG, "persistent work list size");
             if (s == LBM_OK) s = upload(b->off_pitems, pit.data(), pit.size() * sizeof(lbm::StagedItem), "persistent work list");
             if (s == LBM_OK) s = upload(b->off_pcav, pc.data(), pc.size() * sizeof(lbm::PersistCavity), "persistent layout");
+            const std::vector<lbm::TileItem> ti = make_tile_items(b->prm);
+            std::vector<unsigned char> pairs;
+            if (s == LBM_OK && !ti.empty()) {
+                lbm::make_pair_consts(b->cav32.data(), n, &pairs);
+                s = upload(b->off_titems, ti.data(), ti.size() * sizeof(lbm::TileItem), "tiles");
+                if (s == LBM_OK) s = upload(b->off_pair, pairs.data(), pairs.size(), "packed constants");
+            }
             for (int i = 0; i < 2 && s == LBM_OK; ++i)
                 s = upload(b->off_maps + (size_t)i * n * sizeof(CUtensorMap), b->hmaps[i].data(),
                            (size_t)n * sizeof(CUtensorMap), "tensor maps");
@@ -561,17 +606,21 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n, int mode) {
                 b->graph_grid = b->grid;
             }
             LBM_BCUDA(b, cudaGraphLaunch(b->graph[b->cur], b->stream), "graph launch");
+            const int launches = kGraphChunk / steps_of_launch(b, kGraphChunk);  // 50 or 25
             b->steps += kGraphChunk;
-            b->launches += kGraphChunk;
-            done += kGraphChunk;  // kGraphChunk is even: the current buffer is unchanged
+            b->launches += launches;
+            done += kGraphChunk;
+            if (launches & 1) b->cur = 1 - b->cur;
         }
     }
-    for (; done < n; ++done) {
-        cudaError_t e = (mode == LBM_BATCH_PER_CASE) ? per_case_step(b) : fused_step(b, b->tile_x, b->grid);
+    while (done < n) {
+        const int m = mode == LBM_BATCH_PER_CASE ? 1 : steps_of_launch(b, n - done);
+        cudaError_t e = (mode == LBM_BATCH_PER_CASE) ? per_case_step(b) : fused_steps(b, m, b->tile_x, b->grid);
         if (e != cudaSuccess) return bcuda(b, e, "batched step");
         b->launches += (mode == LBM_BATCH_PER_CASE) ? b->n : 1;
         b->cur = 1 - b->cur;
-        ++b->steps;
+        b->steps += m;
+        done += m;
     }
     return LBM_OK;
 }

@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -138,6 +140,21 @@ cudaError_t launch_step_tma(const KConst<float>& k, const CUtensorMap& tm, const
 bool two_steps_supported(const KConst<float>& k);
 cudaError_t launch_two_steps(const KConst<float>& k, const float* src, float* mid, float* dst, uint32_t launch, int sms,
                              cudaStream_t st);
+// Tile of a batch's two-step launch: columns x0 .. x1 - 1, rows y0 .. y1 - 1 of a
+// cavity.
+struct TileItem {
+    int cavity, x0, x1, y0, y1;
+};
+// The tiles of one cavity (row of tiles by row of tiles).
+std::vector<TileItem> tile_items(int cavity, int nx, int ny);
+// The cavities' constants in the packed form's layout (lbm_core.cuh,
+// PairConst), pair_const_bytes() each.
+size_t pair_const_bytes();
+void make_pair_consts(const BatchCavity<float>* cav, int n, std::vector<unsigned char>* out);
+// Two steps of a batch of FP32 cavities walled on all four sides (8 x 8 nodes or
+// more each); tau1: every cavity has tau_f = tau_T = 1.
+cudaError_t launch_two_steps_batch(const BatchCavity<float>* cav, const void* pair, const TileItem* items, int n_items,
+                                   bool tau1, const float* src, float* dst, cudaStream_t st);
 // Work item of the staged batched step: the band of 128 columns from x0 and
 // the segment of rows from y0 of a cavity ny rows high.
 struct StagedItem {
