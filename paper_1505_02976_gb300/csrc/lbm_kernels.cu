@@ -104,9 +104,10 @@ cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step,
     // occupancy (12 blocks of one warp), which leaves SMs idle where the grid
     // is smaller: unused shared memory keeps each SM to its share of the
     // blocks.  FP64 130^2 13.2 -> 12.0, 201^2 21.6 -> 18.9 us a step; with
-    // fewer than four blocks an SM the launches overlap less and it costs 0.5 us.
+    // fewer than four blocks an SM the launches overlap less and it costs 0.5 us,
+    // and four would need more than the 48 KB a launch may ask for unasked.
     const long long per = (cfg.gridDim.x + device_sms() - 1) / device_sms();
-    cfg.dynamicSmemBytes = sizeof(R) == 8 && per >= 4 && per < 12 ? (size_t)(227 / per - 1) * 1024 : 0;
+    cfg.dynamicSmemBytes = sizeof(R) == 8 && per >= 5 && per < 12 ? (size_t)(227 / per - 1) * 1024 : 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
