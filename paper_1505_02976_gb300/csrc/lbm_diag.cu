@@ -15,22 +15,39 @@ namespace lbm {
 constexpr int kResBlock = 256;
 constexpr int kResGrid = 65536;
 
-// Block sum of one value per thread: warp sums in R, then the warps' sums
-// in FP64 in a fixed order (valid in thread 0).
+// Block sums of four values per thread into out[0..3]: warp sums in R, then the
+// warps' sums in FP64, both by halving in a fixed order (a chain of one thread
+// over 32 warps and four values took most of k_reduce4's 14 us at any size).  sh: 4 doubles per warp.
 template <class R>
-__device__ __forceinline__ double block_sum_r(R v, double* sh) {
+__device__ __forceinline__ void block_sum4(const R* v, double* sh, double* __restrict__ out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    R a[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
+    if (lane < 4) sh[4 * wid + lane] = double(lane == 0 ? a[0] : (lane == 1 ? a[1] : (lane == 2 ? a[2] : a[3])));
     __syncthreads();
-    if (lane == 0) sh[wid] = double(v);
-    __syncthreads();
+    if (wid > 0) return;
+    // lane 4 j + m adds value m of warps j, j + 8, ..., then the eight j are added
     double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += sh[i];
-    return s;
+    for (int w = lane >> 2; w < warps; w += 8) s += sh[4 * w + (lane & 3)];
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < 4) out[lane] = s;
 }
 
+// R to FP64.  The conversion instruction runs on the FP64 pipe (two lanes a cycle
+// and SM: four a node were 0.55 of the 0.69 ms of the 8192^2 readout); moving
+// the bits does not.  Arithmetic here flushes subnormal values to zero.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), e = b & 0x7f800000u, sign = b & 0x80000000u;
+    const unsigned hi = ((b & 0x7fffffffu) >> 3) + (e == 0x7f800000u ? 0x70000000u : 0x38000000u);
+    return e == 0u ? __hiloint2double((int)sign, 0) : __hiloint2double((int)(hi | sign), (int)(b << 29));
+}
+
+// Outputs may be null.
 template <class R, class S>
 __global__ void k_moments(const __grid_constant__ KConst<R> k, const S* __restrict__ src,
                           double* __restrict__ p, double* __restrict__ ux, double* __restrict__ uy,
@@ -40,10 +57,10 @@ __global__ void k_moments(const __grid_constant__ KConst<R> k, const S* __restri
     if (x >= k.nx) return;
     const State<R> s = node_state_at(k, src, x, y);
     const long long c = (long long)y * k.nx + x;
-    p[c] = double(s.p);
-    ux[c] = double(s.ux);
-    uy[c] = double(s.uy);
-    T[c] = double(k.T0) + double(s.th);
+    if (p) p[c] = widen(s.p);
+    if (ux) ux[c] = widen(s.ux);
+    if (uy) uy[c] = widen(s.uy);
+    if (T) T[c] = widen(k.T0) + widen(s.th);
 }
 
 template <class R, class S>
@@ -112,11 +129,13 @@ __global__ void k_nusselt_mean(const double* __restrict__ nu, int n, double* __r
 // Per-node terms in the lattice's arithmetic R (the snapshot holds values
 // of type R, so the differences are exact up to one rounding); per-thread
 // sums in R over the thread's nodes, block and grid sums in FP64.
-template <class R, class S>
+// SNAPSHOT: only the snapshot is taken (a new state, whose differences nobody
+// asked for): no read of the old one, no sums.
+template <class R, class S, bool SNAPSHOT>
 __global__ void __launch_bounds__(kResBlock)
 k_residual(const __grid_constant__ KConst<R> k, const S* __restrict__ src, double* __restrict__ snap,
            double* __restrict__ partial) {
-    __shared__ double sh[kResBlock / 32];
+    __shared__ double sh[4 * (kResBlock / 32)];
     const long long N = (long long)k.nx * k.ny;
     // the snapshot holds values of type R (FP64 conversions are slow here)
     R* sn = reinterpret_cast<R*>(snap);
@@ -124,24 +143,27 @@ k_residual(const __grid_constant__ KConst<R> k, const S* __restrict__ src, doubl
     for (long long c = (long long)blockIdx.x * kResBlock + threadIdx.x; c < N; c += (long long)gridDim.x * kResBlock) {
         const int y = (int)((unsigned long long)c / (unsigned)k.nx), x = (int)(c - (long long)y * k.nx);
         // snapshot loads first: they do not depend on the node's moments
-        const R s0 = sn[c], s1 = sn[N + c], s2 = sn[2 * N + c];
+        R s0 = R(0), s1 = R(0), s2 = R(0);
+        if constexpr (!SNAPSHOT) {
+            s0 = sn[c];
+            s1 = sn[N + c];
+            s2 = sn[2 * N + c];
+        }
         R ux, uy, th;
         node_u_th(k, src, x, y, &ux, &uy, &th);
         const R T = k.T0 + th;
-        const R dx = ux - s0, dy = uy - s1, dT = T - s2;
-        v[0] += sqrt(dx * dx + dy * dy);
-        v[1] += sqrt(ux * ux + uy * uy);
-        v[2] += fabs(dT);
-        v[3] += fabs(T);
+        if constexpr (!SNAPSHOT) {
+            const R dx = ux - s0, dy = uy - s1, dT = T - s2;
+            v[0] += sqrt(dx * dx + dy * dy);
+            v[1] += sqrt(ux * ux + uy * uy);
+            v[2] += fabs(dT);
+            v[3] += fabs(T);
+        }
         sn[c] = ux;
         sn[N + c] = uy;
         sn[2 * N + c] = T;
     }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const double s = block_sum_r(v[m], sh);
-        if (threadIdx.x == 0) partial[4 * blockIdx.x + m] = s;
-    }
+    if constexpr (!SNAPSHOT) block_sum4(v, sh, partial + 4 * blockIdx.x);
 }
 
 // Per-block sums of sum_{i=1..8} f_i and sum_i g_i over the stored state.
@@ -171,44 +193,42 @@ k_totals(const __grid_constant__ KConst<R> k, const S* __restrict__ src, double 
     }
 }
 
-constexpr int kReduce4Block = 1024;
+constexpr int kReduce4Block = 512;
 
 __global__ void __launch_bounds__(kReduce4Block) k_reduce4(const double* __restrict__ partial, long long nb,
                                                           double* __restrict__ out) {
-    __shared__ double sh[kReduce4Block / 32];
+    __shared__ double sh[4 * (kReduce4Block / 32)];
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     for (long long b = threadIdx.x; b < nb; b += kReduce4Block)
 #pragma unroll
         for (int m = 0; m < 4; ++m) a[m] += partial[4 * b + m];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const double s = block_sum(a[m], sh);
-        if (threadIdx.x == 0) out[m] = s;
-    }
+    block_sum4(a, sh, out);
 }
 
 // Stream function up each column x: psi(x, 0) = 0 and
 // psi(x, y) = psi(x, y - 1) + (u_x(x, y - 1) + u_x(x, y)) / 2, the trapezoid
-// rule for u_x = d psi / dy.  One thread per column; rows are coalesced.
-__global__ void k_stream_function(const double* __restrict__ ux, int nx, int ny, double* __restrict__ psi) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nx) return;
-    double s = 0.0;
-    psi[x] = 0.0;
-    for (int y = 1; y < ny; ++y) {
-        s = s + 0.5 * (ux[(long long)(y - 1) * nx + x] + ux[(long long)y * nx + x]);
-        psi[(long long)y * nx + x] = s;
-    }
+// rule for u_x = d psi / dy.  Columns are cut into chunks of kPsiRows rows: one
+// launch sums every chunk, the next starts each chunk from the sums below it, so
+// that all rows are read and written at once (one thread a column from the
+// bottom up and one block for the extremes took most of the 1.2 ms by which a
+// 1025^2 readout with psi is now shorter).
+constexpr int kPsiRows = 32, kPsiBlock = 128;
+
+__device__ __forceinline__ double psi_part(const double* __restrict__ u, int nx, int x, int y) {
+    return 0.5 * (u[(long long)(y - 1) * nx + x] + u[(long long)y * nx + x]);
 }
 
-// out[0] = min, out[1] = max of v[0 .. n-1] (one block; order-independent).
-__global__ void k_minmax(const double* __restrict__ v, long long n, double* __restrict__ out) {
-    __shared__ double lo_s[kReduceBlock / 32], hi_s[kReduceBlock / 32];
-    double lo = INFINITY, hi = -INFINITY;
-    for (long long i = threadIdx.x; i < n; i += kReduceBlock) {
-        lo = fmin(lo, v[i]);
-        hi = fmax(hi, v[i]);
-    }
+__global__ void __launch_bounds__(kPsiBlock) k_psi_sums(const double* __restrict__ ux, int nx, int ny, double* __restrict__ sums) {
+    const int x = blockIdx.x * kPsiBlock + threadIdx.x, y0 = blockIdx.y * kPsiRows;
+    if (x >= nx) return;
+    double s = 0.0;
+    for (int y = max(y0, 1); y < min(y0 + kPsiRows, ny); ++y) s += psi_part(ux, nx, x, y);
+    sums[(long long)blockIdx.y * nx + x] = s;
+}
+
+// Extremes of one value pair per thread over the block (order-independent).
+__device__ __forceinline__ void block_minmax(double lo, double hi, double* __restrict__ out) {
+    __shared__ double lo_s[32], hi_s[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -221,13 +241,42 @@ __global__ void k_minmax(const double* __restrict__ v, long long n, double* __re
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int i = 1; i < kReduceBlock / 32; ++i) {
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
             lo = fmin(lo, lo_s[i]);
             hi = fmax(hi, hi_s[i]);
         }
         out[0] = lo;
         out[1] = hi;
     }
+}
+
+// extremes: two values per block
+__global__ void __launch_bounds__(kPsiBlock) k_psi(const double* __restrict__ ux, int nx, int ny,
+                                                   const double* __restrict__ sums, double* __restrict__ psi,
+                                                   double* __restrict__ extremes) {
+    const int x = blockIdx.x * kPsiBlock + threadIdx.x, y0 = blockIdx.y * kPsiRows;
+    double lo = INFINITY, hi = -INFINITY;
+    if (x < nx) {
+        double s = 0.0;
+        for (int c = 0; c < (int)blockIdx.y; ++c) s += sums[(long long)c * nx + x];
+        for (int y = y0; y < min(y0 + kPsiRows, ny); ++y) {
+            if (y > 0) s += psi_part(ux, nx, x, y);
+            psi[(long long)y * nx + x] = s;
+            lo = fmin(lo, s);
+            hi = fmax(hi, s);
+        }
+    }
+    block_minmax(lo, hi, extremes + 2 * ((long long)blockIdx.y * gridDim.x + blockIdx.x));
+}
+
+// out[0] = min, out[1] = max of the n pairs v (one block).
+__global__ void __launch_bounds__(1024) k_minmax(const double* __restrict__ v, long long n, double* __restrict__ out) {
+    double lo = INFINITY, hi = -INFINITY;
+    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+        lo = fmin(lo, v[2 * i]);
+        hi = fmax(hi, v[2 * i + 1]);
+    }
+    block_minmax(lo, hi, out);
 }
 
 template <class R>
@@ -246,12 +295,18 @@ cudaError_t launch_convert(const double* in, R* out, long long n, cudaStream_t s
 template cudaError_t launch_convert<double>(const double*, double*, long long, cudaStream_t);
 template cudaError_t launch_convert<float>(const double*, float*, long long, cudaStream_t);
 
-cudaError_t launch_stream_function(const double* ux, int nx, int ny, double* psi, double* range,
+cudaError_t launch_stream_function(const double* ux, int nx, int ny, double* psi, double* scratch, double* range,
                                    cudaStream_t st) {
-    k_stream_function<<<(nx + 127) / 128, 128, 0, st>>>(ux, nx, ny, psi);
+    const dim3 grid((unsigned)((nx + kPsiBlock - 1) / kPsiBlock), (unsigned)((ny + kPsiRows - 1) / kPsiRows));
+    double* extremes = scratch + (long long)grid.y * nx;
+    k_psi_sums<<<grid, kPsiBlock, 0, st>>>(ux, nx, ny, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_minmax<<<1, kReduceBlock, 0, st>>>(psi, (long long)nx * ny, range);
+    k_psi<<<grid, kPsiBlock, 0, st>>>(ux, nx, ny, scratch, psi, extremes);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const long long n = (long long)grid.x * grid.y;
+    k_minmax<<<1, n > 256 ? 1024 : 256, 0, st>>>(extremes, n, range);
     return cudaGetLastError();
 }
 
@@ -295,10 +350,16 @@ cudaError_t launch_nusselt(const KConst<R>& k, const DiagConst& d, const S* src,
 template <class R, class S>
 cudaError_t launch_residual(const KConst<R>& k, const S* src, double* snap, double* partial,
                             double* out, cudaStream_t st) {
-    k_residual<R, S><<<(unsigned)residual_blocks(k.nx, k.ny), kResBlock, 0, st>>>(k, src, snap, partial);
+    k_residual<R, S, false><<<(unsigned)residual_blocks(k.nx, k.ny), kResBlock, 0, st>>>(k, src, snap, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_reduce4<<<1, kReduce4Block, 0, st>>>(partial, residual_blocks(k.nx, k.ny), out);
+    return cudaGetLastError();
+}
+
+template <class R, class S>
+cudaError_t launch_snapshot(const KConst<R>& k, const S* src, double* snap, cudaStream_t st) {
+    k_residual<R, S, true><<<(unsigned)residual_blocks(k.nx, k.ny), kResBlock, 0, st>>>(k, src, snap, nullptr);
     return cudaGetLastError();
 }
 
@@ -324,7 +385,8 @@ cudaError_t launch_totals(const KConst<R>& k, const S* src, double sT0, double* 
     template cudaError_t launch_nusselt<R, S>(const KConst<R>&, const DiagConst&, const S*, int,    \
                                               double*, double*, cudaStream_t);                      \
     template cudaError_t launch_residual<R, S>(const KConst<R>&, const S*, double*, double*,        \
-                                               double*, cudaStream_t);
+                                               double*, cudaStream_t);                              \
+    template cudaError_t launch_snapshot<R, S>(const KConst<R>&, const S*, double*, cudaStream_t);
 
 LBM_INSTANTIATE_DIAG(double, double)
 LBM_INSTANTIATE_DIAG(float, float)

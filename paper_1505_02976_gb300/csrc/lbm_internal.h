@@ -52,6 +52,10 @@ template <class R, class S>
 cudaError_t launch_residual(const KConst<R>& k, const S* src, double* snap, double* partial,
                             double* out, cudaStream_t st);
 
+// Only the snapshot (of a new state).
+template <class R, class S>
+cudaError_t launch_snapshot(const KConst<R>& k, const S* src, double* snap, cudaStream_t st);
+
 long long residual_blocks(int nx, int ny);
 
 // out[0] = sum over nodes of sum_{i=1..8} f_i, out[1] = sum over nodes of
@@ -61,8 +65,9 @@ cudaError_t launch_totals(const KConst<R>& k, const S* src, double sT0, double* 
                           cudaStream_t st);
 
 // Stream function psi [ny][nx] from u_x [ny][nx] (psi = 0 along y = 0,
-// trapezoid rule up each column); range[0..1] = min, max of psi.
-cudaError_t launch_stream_function(const double* ux, int nx, int ny, double* psi, double* range,
+// trapezoid rule up each column); range[0..1] = min, max of psi.  scratch: at
+// least 2 nx ny doubles (lattices of one node take two), apart from ux and psi.
+cudaError_t launch_stream_function(const double* ux, int nx, int ny, double* psi, double* scratch, double* range,
                                    cudaStream_t st);
 
 // out[i] = R(in[i]) for i < n.
