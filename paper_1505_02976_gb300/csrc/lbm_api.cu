@@ -490,11 +490,9 @@ lbm_status lbm_moments(lbm_handle* h, double* p, double* ux, double* uy, double*
         return lbm::launch_moments(k, (const S*)h->buf(h->cur), to[0], to[1], to[2], to[3], h->stream);
     });
     if (e != cudaSuccess) return cuda_fail(h, e, "moments kernel");
-    for (int q = 0; q < 4; ++q)
-        if (outs[q] && !direct)
-            LBM_CUDA(h, cudaMemcpyAsync(outs[q], F + q * N, N * sizeof(double),
-                                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
-                     "copy of a moment field");
+    if (!direct)
+        LBM_CUDA(h, copy_moments(outs, F, N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
+                 "copy of the moment fields");
     if (!on_device) LBM_CUDA(h, cudaStreamSynchronize(h->stream), "moments");
     return LBM_OK;
 }

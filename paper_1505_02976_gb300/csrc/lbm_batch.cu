@@ -745,10 +745,7 @@ lbm_status lbm_batch_moments(lbm_batch* b, int32_t cavity, double* p, double* ux
     });
     if (e != cudaSuccess) return bcuda(b, e, "moments kernel");
     double* outs[4] = {p, ux, uy, T};
-    for (int q = 0; q < 4; ++q)
-        if (outs[q])
-            LBM_BCUDA(b, cudaMemcpyAsync(outs[q], F + q * N, N * sizeof(double), cudaMemcpyDeviceToHost, b->stream),
-                      "moment copy");
+    LBM_BCUDA(b, copy_moments(outs, F, N, cudaMemcpyDeviceToHost, b->stream), "moment copy");
     LBM_BCUDA(b, cudaStreamSynchronize(b->stream), "moments");
     return LBM_OK;
 }

@@ -97,6 +97,23 @@ inline size_t elem_size(int precision) {
 
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
+// The four moment fields from the device area F (nx ny doubles each, one after
+// the other) to outs (null: not wanted), fields that lie one after the other at
+// the destination too in one copy: a pageable copy costs 10 us before its first
+// byte (256^2: 60 -> 35 us a call).
+inline cudaError_t copy_moments(double* const outs[4], const double* F, size_t N, cudaMemcpyKind kind, cudaStream_t st) {
+    for (int q = 0; q < 4;) {
+        int n = 1;
+        while (outs[q] && q + n < 4 && outs[q + n] == outs[q] + n * N) ++n;
+        if (outs[q]) {
+            const cudaError_t e = cudaMemcpyAsync(outs[q], F + q * N, n * N * sizeof(double), kind, st);
+            if (e != cudaSuccess) return e;
+        }
+        q += n;
+    }
+    return cudaSuccess;
+}
+
 // NVTX range over one entry point (visible to Nsight tools; a no-op
 // otherwise).
 struct NvtxRange {
