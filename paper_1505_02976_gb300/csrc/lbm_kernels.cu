@@ -29,7 +29,32 @@ namespace lbm {
 // warp's chain, and blocks of one warp put every warp on an SM of its own: 32^2
 // 8.7 us a step (10.0 in blocks of four; 17.3 with the wall nodes inside, 38
 // before).
-template <class R, class S, bool EPS_FIELD, bool TAU1>
+// One block's share: block b of the numbering above.  PART: lbm_step.cuh.
+template <class R, class S, bool EPS_FIELD, bool TAU1, int PART>
+__device__ __forceinline__ void step_block(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst, unsigned b,
+                                           int wall_blocks, int bx, uint32_t step) {
+    if ((int)b < wall_blocks) {
+        const int n = (int)(b * blockDim.x + threadIdx.x);
+        if (n >= perimeter_nodes(k)) return;
+        int x, y;
+        perimeter_node(k, n, x, y);
+        if constexpr (PART == 0) wall_update(k, src, dst, x, y, step);
+        else wall_update_tau1<R, S, PART>(k, src, dst, x, y, step);
+        return;
+    }
+    b -= wall_blocks;
+    const int y = (int)(b / (unsigned)bx);
+    const int x = (int)((b - (unsigned)y * bx) * blockDim.x + threadIdx.x);
+    if (x >= k.nx || is_wall(k, x, y)) return;
+    interior_update<R, S, EPS_FIELD, TAU1, PART>(k, src, dst, x, y, step);
+}
+
+// SPLIT (FP64, tau = 1): two blocks for each share, one for the flow and one for
+// the thermal planes.  They repeat what both need, but each has the shorter
+// chain, and a small lattice's step lasts as long as the longest chain: 32^2 8.6
+// -> 7.1 us a step, 80^2 (250 shares) 8.8 -> 8.2, but 100^2 (425) 9.1 -> 9.6, so up
+// to two shares an SM.
+template <class R, class S, bool EPS_FIELD, bool TAU1, bool SPLIT>
 __global__ void __launch_bounds__(kStepBlock, StepOccupancy<R>::blocks)
 k_step(const __grid_constant__ KConst<R> k, const S* __restrict__ src, S* __restrict__ dst, int wall_blocks, int bx,
        uint32_t step) {
@@ -41,19 +66,13 @@ k_step(const __grid_constant__ KConst<R> k, const S* __restrict__ src, S* __rest
     // a step against 19.4.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if ((int)blockIdx.x < wall_blocks) {
-        const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-        if (n >= perimeter_nodes(k)) return;
-        int x, y;
-        perimeter_node(k, n, x, y);
-        wall_update(k, src, dst, x, y, step);
-        return;
+    if constexpr (SPLIT) {
+        const unsigned b = blockIdx.x >> 1;
+        if (blockIdx.x & 1u) step_block<R, S, EPS_FIELD, TAU1, 1>(k, src, dst, b, wall_blocks, bx, step);
+        else step_block<R, S, EPS_FIELD, TAU1, 2>(k, src, dst, b, wall_blocks, bx, step);
+    } else {
+        step_block<R, S, EPS_FIELD, TAU1, 0>(k, src, dst, blockIdx.x, wall_blocks, bx, step);
     }
-    const unsigned b = blockIdx.x - wall_blocks;
-    const int y = (int)(b / (unsigned)bx);
-    const int x = (int)((b - (unsigned)y * bx) * blockDim.x + threadIdx.x);
-    if (x >= k.nx || is_wall(k, x, y)) return;
-    interior_update<R, S, EPS_FIELD, TAU1>(k, src, dst, x, y, step);
 }
 
 template <class R, class S>
@@ -98,7 +117,10 @@ cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step,
     const long long full = (long long)((k.nx + kStepBlock - 1) / kStepBlock) * k.ny;
     const int block = sizeof(R) == 8 || full < 2LL * device_sms() ? 32 : kStepBlock;
     const int bx = (k.nx + block - 1) / block, wall_blocks = (perimeter_nodes(k) + block - 1) / block;
-    cfg.gridDim = dim3((unsigned)(wall_blocks + (long long)bx * k.ny));
+    const bool tau1 = k.omf == R(0) && k.omT == R(0);
+    const long long shares = wall_blocks + (long long)bx * k.ny;
+    const bool split = sizeof(R) == 8 && tau1 && shares <= 2LL * device_sms();
+    cfg.gridDim = dim3((unsigned)(split ? 2 * shares : shares));
     cfg.blockDim = dim3((unsigned)block);
     // The blocks of a dependent launch fill SM after SM up to the kernel's
     // occupancy (12 blocks of one warp), which leaves SMs idle where the grid
@@ -114,12 +136,11 @@ cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool tau1 = k.omf == R(0) && k.omT == R(0);
-    if (k.eps_field)
-        return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, true, true>, k, src, dst, wall_blocks, bx, step)
-                    : cudaLaunchKernelEx(&cfg, k_step<R, S, true, false>, k, src, dst, wall_blocks, bx, step);
-    return tau1 ? cudaLaunchKernelEx(&cfg, k_step<R, S, false, true>, k, src, dst, wall_blocks, bx, step)
-                : cudaLaunchKernelEx(&cfg, k_step<R, S, false, false>, k, src, dst, wall_blocks, bx, step);
+    auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, k, src, dst, wall_blocks, bx, step); };
+    if constexpr (sizeof(R) == 8)
+        if (split) return k.eps_field ? go(k_step<R, S, true, true, true>) : go(k_step<R, S, false, true, true>);
+    if (k.eps_field) return tau1 ? go(k_step<R, S, true, true, false>) : go(k_step<R, S, true, false, false>);
+    return tau1 ? go(k_step<R, S, false, true, false>) : go(k_step<R, S, false, false, false>);
 }
 
 template <class R, class S>

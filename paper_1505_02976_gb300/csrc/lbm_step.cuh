@@ -23,11 +23,24 @@ __device__ __forceinline__ void store_node(const KConst<R>& k, S* __restrict__ d
     store_planes<S, R>(dst + at, k.plane, fo, ho, k.inv_scale, dither);
 }
 
+// PART 1: the flow planes alone, 2: the thermal planes alone (what only the
+// others need is then not computed).
+template <int PART, class R>
+__device__ __forceinline__ void store_part(R* __restrict__ d, long long pl, const R* fo, const R* ho) {
+    if constexpr (PART == 1) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i) d[(i - 1) * pl] = fo[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) d[(8 + i) * pl] = ho[i];
+    }
+}
+
 // Interior node of one step: the nine pull sources are 32-bit offsets from
 // the node (periodic wrap by per-thread deltas), plane strides are uniform
 // across the launch.  TAU1: tau_f = tau_T = 1 (FP16 storage then takes its
 // scale in the collision weights).
-template <class R, class S, bool EPS_FIELD, bool TAU1>
+template <class R, class S, bool EPS_FIELD, bool TAU1, int PART = 0>
 __device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __restrict__ src,
                                                 S* __restrict__ dst, int x, int y, uint32_t step) {
     const int dxm = x == 0 ? k.nx - 1 : -1;
@@ -50,9 +63,13 @@ __device__ __forceinline__ void interior_update(const KConst<R>& k, const S* __r
     R fo[9], ho[9];
     constexpr bool prescale = TAU1 && std::is_same<S, __half>::value;
     core_interior<TAU1>(k, cell, eps_ay(k, k, cell, y), f, h, fo, ho, prescale ? R(k.inv_scale) : R(1));
-    if (!lfinite(ho[0])) atomicOr(k.flag, 1);
-    Dither dither((uint32_t)at, step);
-    store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
+    if (PART != 1 && !lfinite(ho[0])) atomicOr(k.flag, 1);
+    if constexpr (PART != 0) {
+        store_part<PART>(dst + at, pl, fo, ho);
+    } else {
+        Dither dither((uint32_t)at, step);
+        store_planes<S, R>(dst + at, pl, fo, ho, prescale ? 1.0f : k.inv_scale, &dither);
+    }
 }
 
 // Wall node idx of a lattice in perimeter order: S row, N row, W column, E
@@ -150,13 +167,17 @@ __device__ __forceinline__ void wall_node_generic(const KConst<R>& k, const Sour
 }
 
 // Both out of line: only the 4(N - 1) wall threads take them.
-template <class R, class S>
+template <class R, class S, int PART>
 __device__ __noinline__ void wall_update_tau1(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst,
                                               int x, int y, uint32_t step) {
     R fo[9], ho[9];
     wall_node_tau1(k, GlobalSource<R, S>{src}, x, y, fo, ho);
-    Dither dither((uint32_t)(y * k.pitch + x), step);
-    store_node(k, dst, (long long)y * k.pitch + x, fo, ho, &dither);
+    if constexpr (PART != 0) {
+        store_part<PART>(dst + (long long)y * k.pitch + x, k.plane, fo, ho);
+    } else {
+        Dither dither((uint32_t)(y * k.pitch + x), step);
+        store_node(k, dst, (long long)y * k.pitch + x, fo, ho, &dither);
+    }
 }
 template <class R, class S>
 __device__ __noinline__ void wall_update_generic(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst,
@@ -170,7 +191,7 @@ __device__ __noinline__ void wall_update_generic(const KConst<R>& k, const S* __
 template <class R, class S>
 __device__ __forceinline__ void wall_update(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst, int x,
                                             int y, uint32_t step) {
-    if (k.omf == R(0) && k.omT == R(0)) wall_update_tau1(k, src, dst, x, y, step);
+    if (k.omf == R(0) && k.omT == R(0)) wall_update_tau1<R, S, 0>(k, src, dst, x, y, step);
     else wall_update_generic(k, src, dst, x, y, step);
 }
 
