@@ -12,7 +12,7 @@
 //     (Pi, u u, u F), so its coefficients fold into those of Q;
 //   * likewise the thermal odd part is c . V, its even part B0 + Kc (c.u)^2;
 //   * 1/a and b/(a - b |u|^2) of the gradient solve share one reciprocal.
-// FP32: 163 operations a node plus two square roots and two reciprocals; the
+// FP32: 162 operations a node plus two square roots and two reciprocals; the
 // direction-by-direction form took 215 (FP64 instructions of the whole step,
 // square roots and reciprocals included: see k_step in lbm_kernels.cu).
 //
@@ -116,28 +116,25 @@ __device__ __forceinline__ bool lfinite(float2 a) { return isfinite(a.x) && isfi
 // 104 with the moves, 70 without; 59.9 -> 58.3 us a step at 2048^2, the FP16
 // step unchanged within 1 %).
 struct PairConst {
-    float2 inv_rho0, hq_sigma, half_Q, eay, half_ax, nnuK_q2, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie, a_ep, a_const, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF, gain, h_sig, h_kQ, h_pT, h_u3, h_uQ, h_g, h_W, h_Wr, inv_sigma, T0, invD, rho0, gbeta, ax, omf, omT;
+    float2 inv_rho0, hq_sigma, half_Q, eay, half_ax, nnuK_q2, nnuK_0, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie, a_ep, a_const, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF, h_sig, h_kQ, h_pT, h_u3, h_uQ, h_g, h_W, h_Wr, inv_sigma, T0, invD, rho0, gbeta, ax, omf, omT;
     float2 half, nhalf, nthird, nquarter, one, two;  // literals
-    float2 w1, w5f, w5h, w0, pT, n1, n5f;            // weights (core_weights)
+    float2 w1, w5, w0, pT, n1, n5;                   // weights (core_weights)
     Cell<float2> cell;
 };
 
-// Weights of the outputs: axis, diagonal (flow, thermal), rest, and the rest
+// Weights of the outputs: axis, diagonal, rest, and the rest
 // direction's T p term; all times the storage scale.
 template <class L>
 struct CoreWeights {
-    L w1, w5f, w5h, w0, pT, n1, n5f;  // n1, n5f: -w1, -w5f
+    L w1, w5, w0, pT, n1, n5;  // n1, n5: -w1, -w5
 };
 template <class R>
 __host__ __device__ __forceinline__ CoreWeights<R> core_weights(const KConst<R>& k, R scale) {
-    // the flow's own diagonal weight, rounded to nearest: 2 w_1 + 4 w_5 is
-    // then within 7.5e-9 of 1/3, which scales the momentum in each step
-    // (w_diag, fitted to the sum of all nine, is 1.5e-8 off)
-    return {scale * (R(1) / R(9)), scale * (R(1) / R(36)), scale * w_diag<R>(), scale * (R(4) / R(9)), scale * k.h0_pT,
-            -(scale * (R(1) / R(9))), -(scale * (R(1) / R(36)))};
+    return {scale * (R(1) / R(9)), scale * w_diag<R>(), scale * (R(4) / R(9)), scale * k.h0_pT, -(scale * (R(1) / R(9))),
+            -(scale * w_diag<R>())};
 }
 __device__ __forceinline__ CoreWeights<float2> core_weights(const PairConst& q, float) {
-    return {q.w1, q.w5f, q.w5h, q.w0, q.pT, q.n1, q.n5f};
+    return {q.w1, q.w5, q.w0, q.pT, q.n1, q.n5};
 }
 
 // The pairs of a run's constants; scale: the storage scale of the outputs.
@@ -150,6 +147,7 @@ inline PairConst make_pair_const(const KConst<float>& k, float scale) {
     q.eay = two(k.eay);
     q.half_ax = two(k.half_ax);
     q.nnuK_q2 = two(k.nnuK_q2);
+    q.nnuK_0 = two(k.nnuK_0);
     q.nFK_q = two(k.nFK_q);
     q.e1 = two(k.e1);
     q.e1_lo = two(k.e1_lo);
@@ -171,7 +169,6 @@ inline PairConst make_pair_const(const KConst<float>& k, float scale) {
     q.fA_ep = two(k.fA_ep);
     q.f_cu = two(k.f_cu);
     q.f_cF = two(k.f_cF);
-    q.gain = two(k.gain);
     q.h_sig = two(k.h_sig);
     q.h_kQ = two(k.h_kQ);
     q.h_pT = two(k.h_pT);
@@ -196,23 +193,20 @@ inline PairConst make_pair_const(const KConst<float>& k, float scale) {
     q.two = two(2.0f);
     const CoreWeights<float> w = core_weights(k, scale);
     q.w1 = two(w.w1);
-    q.w5f = two(w.w5f);
-    q.w5h = two(w.w5h);
+    q.w5 = two(w.w5);
     q.w0 = two(w.w0);
     q.pT = two(w.pT);
     q.n1 = two(w.n1);
-    q.n5f = two(w.n5f);
+    q.n5 = two(w.n5);
     q.cell.eps = two(k.cell.eps);
     q.cell.ie = two(k.cell.ie);
+    q.cell.elo = two(k.cell.elo);
     q.cell.eg = two(k.cell.eg);
     q.cell.eax = two(k.cell.eax);
     q.cell.heax = two(k.cell.heax);
     q.cell.c0 = two(k.cell.c0);
     q.cell.c0sq = two(k.cell.c0sq);
     q.cell.c1 = two(k.cell.c1);
-    q.cell.ih = two(k.cell.ih);
-    q.cell.il = two(k.cell.il);
-    q.cell.ci = two(k.cell.ci);
     q.cell.nnuK = two(k.cell.nnuK);
     q.cell.nFK = two(k.cell.nFK);
     q.cell.e2 = two(k.cell.e2);
@@ -253,19 +247,15 @@ __device__ __forceinline__ Cell<L> field_cell(const Q& q, L e) {
     const L r = lmul(lsub(q_one(q), e), ie);
     c.eps = e;
     c.ie = ie;
+    c.elo = lmul(e, lfma(lneg(e), ie, q_one(q)));
     c.eg = lmul(e, q.gbeta);
     c.eax = lmul(e, q.ax);
     c.heax = lmul(e, q.half_ax);
-    c.nnuK = lmul(lmul(r, r), q.nnuK_q2);
+    c.nnuK = lfma(lmul(r, r), q.nnuK_q2, q.nnuK_0);
     c.nFK = lmul(lmul(r, ie), q.nFK_q);
     c.c0 = lfma(q_nquarter(q), c.nnuK, q_half(q));
     c.c0sq = lmul(c.c0, c.c0);
     c.c1 = lmul(q_nhalf(q), c.nFK);
-    const L d = lfma(q_nhalf(q), c.nnuK, q_one(q));  // 2 c0
-    c.ih = lrcp(d);
-    c.il = lmul(c.ih, lfma(lneg(d), c.ih, q_one(q)));
-    if constexpr (sizeof(R) == 4) c.il = lfma(c.ih, q.gain, c.il);
-    c.ci = lneg(lmul(c.c1, c.ih));
     c.e2 = lmul(ie, q.e2_ie);
     c.e3 = lmul(ie, q.e3_ie);
     c.re = lmul(ie, q.rho0);
@@ -347,19 +337,8 @@ __device__ __forceinline__ CoreState<L> core_moments(const Q& q, const Cell<L>& 
     const L vmag = lsqrt(lfma(vx, vx, lmul(vy, vy)));
     const L iden = lrcp(ladd(c.c0, lsqrt(lfma(c.c1, vmag, c.c0sq))));
     const L um = lmul(vmag, iden);  // |u| = |v| / (c0 + sqrt(c0^2 + c1 |v|)): no further square root
-    if constexpr (sizeof(R) == 4) {
-        // The same quotient as v/(2 c0) less a small part: with
-        // sqrt(c0^2 + c1 |v|) - c0 = c1 |u|, 1/den = ih - ih c1 |u|/den,
-        // ih + il = 1/(2 c0).  v iden would carry the rounding of den, the same
-        // at every step where c1 |v| is small: a gain or loss of momentum of up
-        // to 1e-7 a step that builds up.
-        const L rest = lfma(lmul(c.ci, um), iden, c.il);
-        s.ux = lfma(vx, c.ih, lmul(vx, rest));
-        s.uy = lfma(vy, c.ih, lmul(vy, rest));
-    } else {
-        s.ux = lmul(vx, iden);
-        s.uy = lmul(vy, iden);
-    }
+    s.ux = lmul(vx, iden);
+    s.uy = lmul(vy, iden);
     const L uu = lfma(s.ux, s.ux, lmul(s.uy, s.uy));
     const L nd = lfma(c.nFK, um, c.nnuK);
     s.Fx = lfma(nd, s.ux, c.eax);
@@ -460,17 +439,17 @@ __device__ __forceinline__ void core_emit(const Q& q, const Cell<L>& c, const Co
             Dx = SOURCES ? lfma(fu, s.ux, lmul(fF, s.Fx)) : lmul(fu, s.ux);
             Dy = SOURCES ? lfma(fu, s.uy, lmul(fF, s.Fy)) : lmul(fu, s.uy);
         }
-        const L w5 = w_.w5f;
+        const L w5 = w_.w5;
         put_f(1, 3, w1, w_.n1, ladd(E, Qxx), Dx);
         put_f(2, 4, w1, w_.n1, ladd(E, Qyy), Dy);
-        put_f(5, 7, w5, w_.n5f, ladd(Ed, Q2), SOURCES ? ladd(Dx, Dy) : lfma(fu, s.uy, Dx));
-        put_f(6, 8, w5, w_.n5f, lsub(Ed, Q2), SOURCES ? lsub(Dy, Dx) : lfma(lneg(q.f_cu), s.ux, Dy));
+        put_f(5, 7, w5, w_.n5, ladd(Ed, Q2), SOURCES ? ladd(Dx, Dy) : lfma(fu, s.uy, Dx));
+        put_f(6, 8, w5, w_.n5, lsub(Ed, Q2), SOURCES ? lsub(Dy, Dx) : lfma(lneg(q.f_cu), s.ux, Dy));
     }
     {
         // even part: sigma theta plus small terms, summed among themselves first
         const L T = s.T, Tep = lmul(T, s.ep);
         const L th = lmul(q.h_sig, s.th);
-        L kx, ky, tr;
+        L kx = L(), ky = L(), tr = L();
         if constexpr (!REST) {
             const L kc = lmul(c.kc, T);
             kx = lmul(kc, s.ux);
@@ -504,7 +483,7 @@ __device__ __forceinline__ void core_emit(const Q& q, const Cell<L>& c, const Co
             Vx = lfma(K, s.ux, lmul(hg, s.gx));
             Vy = lfma(K, s.uy, lmul(hg, s.gy));
         }
-        const L w5 = w_.w5h;
+        const L w5 = w_.w5;
         auto relax = [&](const L& w, const L& small, const L& in) {
             return ladd(in, lfma(itT, lfma(w, tr0, lneg(in)), lmul(w, small)));
         };

@@ -67,10 +67,9 @@ enum : int { SW = 0, SE = 1, SS = 2, SN = 3 };
 // porosity, itf, itT = 1/tau, a = 1.5 itf rho0 A invD the share of S in Q.
 template <class V>
 struct Cell {
-    V eps, ie;         // e, 1/e
+    V eps, ie, elo;    // e, 1/e, and 1/ie - e (what rounding left of e (1/e) = 1)
     V eg, eax, heax;   // e g beta, e a_x, e a_x / 2
     V c0, c0sq, c1;    // quadratic solve (Sec. 3.1)
-    V ih, il, ci;      // 1/(2 c0) and its rounding error, -c1/(2 c0)
     V nnuK, nFK;       // - e nu/K, - e F_e/sqrt(K)
     V e2, e3;          // e p = e1 sum f + e2 u.F + e3 |u|^2
     V re;              // rho0 / e
@@ -116,8 +115,8 @@ struct KConst {
     // porosity, and the factors that give a porosity field's
     Cell<R> cell;
     R inv_rho0, hq_sigma, half_Q, eay, half_ax;      // 1/rho0, Q/(2 sigma), Q/2, eps a_y, a_x/2
-    R nnuK_q2, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie;
-    R a_ep, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF, gain;
+    R nnuK_q2, nnuK_0, nFK_q, e1, e1_lo, e2_ie, e3_ie, qu_ie, qF_ie, cu2_ie, cuF_ie, b_0, ug_b, kc_ie;
+    R a_ep, aS, aS2, f_ScS, f_ScS2, fA_ep, f_cu, f_cF;
     R h_sig, h_kQ, h_pT, h0_pT, h_u3, h_uQ, h_g, h_W, h_Wr;
     R u_abs[4];            // |u_bc| per side
     // nodes at the end of a staged step's sweep whose stores ask L2 to keep
