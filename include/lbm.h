@@ -126,7 +126,8 @@ typedef struct {
  * post-collision populations the moments define). */
 
 /* Row segments per column band of the moment-state step (segments >= 1;
- * 0 restores the default, which fills the GPU's resident blocks once).
+ * 0 restores the default: segments that fill the GPU's resident blocks twice,
+ * and for smaller FP32 lattices a kernel over tiles instead of bands).
  * Every choice computes the same values.  LBM_ERR_ARG on a population
  * handle. */
 lbm_status lbm_set_moment_segments(lbm_handle* h, int32_t segments);

@@ -253,10 +253,7 @@ lbm_status lbm_create(const lbm_params* p, void* stream, void* workspace, size_t
         cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         (void)cudaGetLastError();
     h->two_steps = p->precision == LBM_F32 && !p->moment_state && lbm::two_steps_supported(h->k32);
-    h->msegments = 1;
-    if (p->moment_state)
-        h->msegments = p->precision == LBM_F64 ? lbm::moment_segments_default(h->k64)
-                                               : lbm::moment_segments_default(h->k32);
+    h->msegments = 0;
     h->diag.T0 = d.T0;
     h->diag.inv_sigma = 1.0 / p->sigma;
     h->diag.Q = d.Q;
@@ -376,6 +373,9 @@ lbm_status lbm_step(lbm_handle* h, int64_t n) {
             cudaError_t e = h->prm.precision == LBM_F64
                                 ? lbm::launch_step_m(h->k64, (const double*)h->mom(src), (double*)h->mom(dst),
                                                      h->msources, h->msegments, h->stream)
+                            : h->msegments == 0 && lbm::moment_tiles_preferred(h->k32, h->sms)
+                                ? lbm::launch_step_m_tiles(h->k32, (const float*)h->mom(src), (float*)h->mom(dst),
+                                                           h->msources, h->sms, h->stream)
                                 : lbm::launch_step_m(h->k32, (const float*)h->mom(src), (float*)h->mom(dst),
                                                      h->msources, h->msegments, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "moment step kernel");
@@ -438,9 +438,6 @@ int32_t lbm_step_staged(const lbm_handle* h) { return h && h->tma ? 1 : 0; }
 lbm_status lbm_set_moment_segments(lbm_handle* h, int32_t segments) {
     if (!h) return LBM_ERR_ARG;
     if (!h->moments_kind() || segments < 0) return fail(h, LBM_ERR_ARG, "not a moment-state handle, or segments < 0");
-    if (segments == 0)
-        segments = h->prm.precision == LBM_F64 ? lbm::moment_segments_default(h->k64)
-                                               : lbm::moment_segments_default(h->k32);
     h->msegments = segments;
     return LBM_OK;
 }

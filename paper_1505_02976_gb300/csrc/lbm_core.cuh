@@ -527,6 +527,43 @@ __device__ __forceinline__ void core_interior(const Q& q, const Cell<L>& c, L ea
     core_emit<TAU1, true>(q, c, s, Qxx, Qyy, Q2, f, h, fo, ho, wscale);
 }
 
+// Moment state (tau_f = tau_T = 1): the nine stored moments of a state ...
+template <class L, class Q>
+__device__ __forceinline__ void stored_moments(const Q& q, const Cell<L>& c, const CoreState<L>& s, L* m) {
+    const Shear<L> S = core_shear(q, c, s);
+    m[MP] = lmul(s.ep, c.ie);
+    m[MUX] = s.ux;
+    m[MUY] = s.uy;
+    m[MSXX] = S.xx;
+    m[MSYY] = S.yy;
+    m[MSXY] = S.xy;
+    m[MTH] = s.th;
+    m[MGX] = s.gx;
+    m[MGY] = s.gy;
+}
+// ... and the populations of a node from them; F is recomputed from (u, T) as in
+// core_moments (and, for a wall node, as in core_boundary).
+template <bool SOURCES, class L, class Q>
+__device__ __forceinline__ void expand_moments(const Q& q, const Cell<L>& c, L eay, const L* m, L* fo, L* ho) {
+    CoreState<L> s;
+    s.ux = m[MUX];
+    s.uy = m[MUY];
+    s.th = m[MTH];
+    s.gx = m[MGX];
+    s.gy = m[MGY];
+    s.T = ladd(q.T0, s.th);
+    const L uu = lfma(s.ux, s.ux, lmul(s.uy, s.uy));
+    const L nd = lfma(c.nFK, lsqrt(uu), c.nnuK);
+    s.Fx = lfma(nd, s.ux, c.eax);
+    s.Fy = lfma(nd, s.uy, lfma(c.eg, s.th, eay));
+    s.ep = lfma(c.eps, m[MP], lmul(c.elo, m[MP]));  // the inverse of p = ep ie as stored (e ie != 1)
+    const Shear<L> S = {m[MSXX], m[MSYY], m[MSXY]};
+    L Qxx, Qyy, Q2;
+    shear_form<SOURCES>(q, c, s.ux, s.uy, s.Fx, s.Fy, S, Qxx, Qyy, Q2);
+    core_emit<true, SOURCES>(q, c, s, Qxx, Qyy, Q2, (const L*)nullptr, (const L*)nullptr, fo, ho,
+                             typename LaneReal<L>::type(1));
+}
+
 // Wall node at tau_f = tau_T = 1 (Sec. 3.4): there the extrapolated
 // non-equilibrium part carries the factor 1 - 1/tau = 0, so the node is the
 // collision of its boundary state b alone.  s, S: state and shear rate of

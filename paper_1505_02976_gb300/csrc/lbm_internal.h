@@ -109,9 +109,15 @@ cudaError_t launch_nusselt_batch(const BatchCavity<R>* cav, int n, const S* src,
 // One step of the moment state (9 planes: p, u, S, T - T0, grad T) from src
 // to dst; sources = false when src is the state written by launch_init_m
 // (equilibria without force and source terms).  segments: row segments per
-// band (clamped so that each keeps >= 3 rows).
+// band (clamped so that each keeps >= 3 rows; 0: moment_segments_default).
 template <class R>
 cudaError_t launch_step_m(const KConst<R>& k, const R* src, R* dst, bool sources, int segments, cudaStream_t st);
+
+// The same for an FP32 lattice of at least 8 x 8 nodes over the tiles of the
+// two-step kernel (lbm_tile.cu).
+cudaError_t launch_step_m_tiles(const KConst<float>& k, const float* src, float* dst, bool sources, int sms, cudaStream_t st);
+// Whether that is the faster of the two for this lattice.
+bool moment_tiles_preferred(const KConst<float>& k, int sms);
 
 // Post-collision populations (17 planes, as the population kernels store
 // them) of the moment state src.

@@ -49,28 +49,6 @@ constexpr int kMStrip = 30;      // output columns of a strip, at most (32 lanes
 template <class R> struct MomentOccupancy { static constexpr int blocks = LBM_MOMENT_BLOCKS; };
 template <> struct MomentOccupancy<double> { static constexpr int blocks = 2; };
 
-// Populations of a node from its stored moments; F is recomputed from (u, T)
-// as in core_moments (and, for a wall node, as in core_boundary).
-template <class R, bool SOURCES>
-__device__ __forceinline__ void expand_moments(const KConst<R>& k, const Cell<R>& c, R eay, const R* m, R* fo, R* ho) {
-    CoreState<R> s;
-    s.ux = m[MUX];
-    s.uy = m[MUY];
-    s.th = m[MTH];
-    s.gx = m[MGX];
-    s.gy = m[MGY];
-    s.T = ladd(k.T0, s.th);
-    const R uu = lfma(s.ux, s.ux, lmul(s.uy, s.uy));
-    const R nd = lfma(c.nFK, lsqrt(uu), c.nnuK);
-    s.Fx = lfma(nd, s.ux, c.eax);
-    s.Fy = lfma(nd, s.uy, lfma(c.eg, s.th, eay));
-    s.ep = lmul(c.eps, m[MP]);
-    const Shear<R> S = {m[MSXX], m[MSYY], m[MSXY]};
-    R Qxx, Qyy, Q2;
-    shear_form<SOURCES>(k, c, s.ux, s.uy, s.Fx, s.Fy, S, Qxx, Qyy, Q2);
-    core_emit<true, SOURCES>(k, c, s, Qxx, Qyy, Q2, (const R*)nullptr, (const R*)nullptr, fo, ho, R(1));
-}
-
 // Constants of node (x, y), the porosity field known at compile time.
 template <class R, bool EPS_FIELD>
 __device__ __forceinline__ Cell<R> moment_cell(const KConst<R>& k, int x, int y) {
@@ -146,7 +124,7 @@ __device__ __forceinline__ Expanded<R> expand_node(const KConst<R>& k, const R* 
     if (!ok) return e;
     R fo[9], ho[9];
     const Cell<R> c = moment_cell<R, EPS_FIELD>(k, xe, r);
-    expand_moments<R, SOURCES>(k, c, eps_ay(k, k, c, r), m, fo, ho);
+    expand_moments<SOURCES>(k, c, eps_ay(k, k, c, r), m, fo, ho);
     e.up[0] = fo[2]; e.up[1] = fo[5]; e.up[2] = fo[6];
     e.up[3] = ho[2]; e.up[4] = ho[5]; e.up[5] = ho[6];
     e.hz[0] = fo[1]; e.hz[1] = fo[3]; e.hz[2] = ho[0]; e.hz[3] = ho[1]; e.hz[4] = ho[3];
@@ -237,18 +215,8 @@ k_step_m(const __grid_constant__ KConst<R> k, const R* __restrict__ src, R* dst,
             R mo[kMPlanes] = {};
             if (out_col && !wall_col) {
                 const Cell<R> c = moment_cell<R, EPS_FIELD>(k, x, y);
-                const CoreState<R> s = core_moments(k, c, eps_ay(k, k, c, y), f, h);
-                const Shear<R> S = core_shear(k, c, s);
-                if (!isfinite(s.th + s.ux + s.uy)) atomicOr(k.flag, 1);
-                mo[MP] = lmul(s.ep, c.ie);
-                mo[MUX] = s.ux;
-                mo[MUY] = s.uy;
-                mo[MSXX] = S.xx;
-                mo[MSYY] = S.yy;
-                mo[MSXY] = S.xy;
-                mo[MTH] = s.th;
-                mo[MGX] = s.gx;
-                mo[MGY] = s.gy;
+                stored_moments(k, c, core_moments(k, c, eps_ay(k, k, c, y), f, h), mo);
+                if (!isfinite(mo[MTH] + mo[MUX] + mo[MUY])) atomicOr(k.flag, 1);
                 store_moments(k, dst, (long long)y * k.pitch + x, mo);
             }
             if (wallWE) {
@@ -290,7 +258,7 @@ __global__ void k_expand_m(const __grid_constant__ KConst<R> k, const R* __restr
     for (int q = 0; q < kMPlanes; ++q) m[q] = src[q * k.plane + at];
     const Cell<R> c = node_cell(k, x, y);
     R fo[9], ho[9];
-    expand_moments<R, SOURCES>(k, c, eps_ay(k, k, c, y), m, fo, ho);
+    expand_moments<SOURCES>(k, c, eps_ay(k, k, c, y), m, fo, ho);
 #pragma unroll
     for (int i = 1; i < 9; ++i) dst[(i - 1) * k.plane + at] = fo[i];
 #pragma unroll
@@ -364,6 +332,7 @@ int moment_segments_default(const KConst<R>& k) {
 
 template <class R>
 cudaError_t launch_step_m(const KConst<R>& k, const R* src, R* dst, bool sources, int segments, cudaStream_t st) {
+    if (segments == 0) segments = moment_segments_default(k);
     int nstrips = 0, nseg = 0;
     moment_shape(k, segments, &nstrips, &nseg);
     if (k.eps_field)

@@ -339,7 +339,139 @@ k_tile(const __grid_constant__ KConst<float> k, const __grid_constant__ PairCons
     tile_two_steps<EPS_FIELD, TAU1>(k, pc, src, mid, dst, slots, X0, X1, Y0, Y1, warps, hot);
 }
 
-// The same for a batch of FP32 cavities walled on all four sides: block i takes
+// ------------------------------------------------------------- moment state
+// One step of the FP32 moment state (lbm_moment.cu) over the same tiles: the
+// moments of the tile and its ring are expanded into populations in the shared
+// rows (two x-neighbours a lane, packed), and the tile's new moments computed
+// from their pulls.  Wall nodes expand like any other; their new state is the
+// boundary state of x_f's new moments, one wall node a thread.
+// Against warps that march up strips of columns (k_step_m), which expand fewer
+// nodes twice but keep only one row a warp in flight: 64^2 3.7 against 6.1 us a
+// step, 201^2 4.0 / 7.6, 512^2 7.2 / 11.3, 1024 x 777 15.1 / 18.9, but 2048^2 73.9 /
+// 72.4 and 3000 x 2900 145 / 139: the line lies between, at 16 tiles an SM.
+__device__ __noinline__ void tile_wall_m(const KConst<float>& k, TileSource src, float* __restrict__ dst, int x, int y) {
+    const WallInfo w = classify(k, x, y);
+    Pops<float> P;
+    src(k, w.xs, w.ys, P);
+    const Cell<float> c = node_cell(k, w.xs, w.ys);
+    float m[kMPlanes];
+    stored_moments(k, c, core_moments(k, c, eps_ay(k, k, c, w.ys), P.f, P.h), m);
+    m[MUX] = k.u_bc[w.uside][0];
+    m[MUY] = k.u_bc[w.uside][1];
+    if (w.tside >= 0) {
+        m[MTH] = lsub(k.T_bc[w.tside], k.T0);
+    } else {
+        Pops<float> Q;
+        src(k, w.xff, w.yff, Q);
+        m[MTH] = lmul(lfma(4.f, m[MTH], -core_theta(k, core_hsum(Q.h))), 1.f / 3.f);
+        if (w.fixgx) m[MGX] = 0.f;
+        if (w.fixgy) m[MGY] = 0.f;
+    }
+    if (!isfinite(m[MTH] + m[MP])) atomicOr(k.flag, 1);
+    float* d = dst + ((long long)y * k.pitch + x);
+#pragma unroll
+    for (int q = 0; q < kMPlanes; ++q) d[q * k.plane] = m[q];
+}
+
+template <bool EPS_FIELD, bool SOURCES>
+__global__ void __launch_bounds__(kTileMaxThreads, 2)
+k_tile_m(const __grid_constant__ KConst<float> k, const __grid_constant__ PairConst pc, const float* __restrict__ src,
+         float* __restrict__ dst, TileSplit sx, TileSplit sy, int warps, bool early) {
+    extern __shared__ __align__(16) float slots[];
+    if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int X0 = sx.begin(blockIdx.x), X1 = sx.begin(blockIdx.x + 1), Y0 = sy.begin(blockIdx.y), Y1 = sy.begin(blockIdx.y + 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool wx = k.bc[SW] != BC_PERIODIC, wy = k.bc[SS] != BC_PERIODIC;
+    const int nx = k.nx, ny = k.ny, pl = k.plane32, pitch = k.pitch;
+    const int ya = wy ? max(Y0 - 1, 0) : Y0 - 1, yb = wy ? min(Y1 + 1, ny) : Y1 + 1;
+    const int xa = wx ? max(X0 - 1, 0) : X0 - 1, xb = wx ? min(X1 + 1, nx) : X1 + 1;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    auto cell_of = [&](int y, unsigned c0, unsigned c1) {
+        if constexpr (EPS_FIELD) {
+            const float* e = k.eps_field + (long long)y * nx;
+            return field_cell(pc, make_float2(e[c0], e[c1]));
+        } else {
+            return pc.cell;
+        }
+    };
+    {
+        const int x = X0 - 1 + 2 * lane;
+        const bool va = x >= xa && x < xb, vb = x + 1 >= xa && x + 1 < xb;
+        auto col = [&](int c) { return wx ? min(max(c, 0), nx - 1) : (c < 0 ? c + nx : (c >= nx ? c - nx : c)); };
+        const int xe = min(x, X1);  // (a lane beyond the ring repeats its end)
+        const unsigned c0 = col(xe), c1 = col(min(x + 1, X1));
+        for (int yy = warp < warps ? ya + warp : yb; yy < yb; yy += warps) {
+            const int y = wy ? yy : (yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy));
+            const unsigned r = y * pitch;
+            float2 m[kMPlanes], fo[9], ho[9];
+#pragma unroll
+            for (int q = 0; q < kMPlanes; ++q) {
+                const float* s = src + q * pl;
+                m[q] = make_float2(s[r + c0], s[r + c1]);
+            }
+            const Cell<float2> c = cell_of(y, c0, c1);
+            expand_moments<SOURCES>(pc, c, eps_ay(k, pc, c, y), m, fo, ho);
+            float* d = slots + (yy - Y0 + 1) * kTileRowElems + 2 * lane;
+            if (va && vb) {
+#pragma unroll
+                for (int i = 1; i < 9; ++i) *reinterpret_cast<float2*>(d + (i - 1) * kTileCols) = fo[i];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(d + (8 + i) * kTileCols) = ho[i];
+            } else if (va || vb) {
+                d += va ? 0 : 1;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) d[(i - 1) * kTileCols] = va ? fo[i].x : fo[i].y;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) d[(8 + i) * kTileCols] = va ? ho[i].x : ho[i].y;
+            }
+        }
+    }
+    __syncthreads();
+    {
+        const int x = X0 + 2 * lane;
+        const bool in = lane < kTilePairs && x < X1;
+        const bool va = in && !(wx && (x == 0 || x == nx - 1)), vb = in && x + 1 < X1 && !(wx && x + 1 == nx - 1);
+        const int l = min(lane, kTilePairs - 1);
+        for (int y = warp < warps ? Y0 + warp : Y1; y < Y1; y += warps) {
+            if (wy && (y == 0 || y == ny - 1)) continue;
+            const float* s0 = slots + (y - Y0 + 1) * kTileRowElems + 2 * l;
+            float2 f[9], h[9], m[kMPlanes];
+            auto load = [&](int i, int plane) {
+                const float* s = s0 + (plane * kTileCols - cy_of(i) * kTileRowElems);
+                return cx_of(i) > 0 ? ld2(s) : (cx_of(i) < 0 ? ld2(s + 2) : make_float2(s[1], s[2]));
+            };
+#pragma unroll
+            for (int i = 1; i < 9; ++i) f[i] = load(i, i - 1);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) h[i] = load(i, 8 + i);
+            const Cell<float2> c = cell_of(y, min(x, nx - 1), min(x + 1, nx - 1));
+            stored_moments(pc, c, core_moments(pc, c, eps_ay(k, pc, c, y), f, h), m);
+            const float2 check = ladd(ladd(m[MTH], m[MUX]), m[MUY]);
+            if ((va && !lfinite(check.x)) || (vb && !lfinite(check.y))) atomicOr(k.flag, 1);
+            float* d = dst + (y * pitch + x);
+            if (va && vb) {
+#pragma unroll
+                for (int q = 0; q < kMPlanes; ++q) *reinterpret_cast<float2*>(d + q * pl) = m[q];
+            } else if (va || vb) {
+                d += va ? 0 : 1;
+#pragma unroll
+                for (int q = 0; q < kMPlanes; ++q) d[q * pl] = va ? m[q].x : m[q].y;
+            }
+        }
+        const int wall_threads = (int)blockDim.x > 32 * warps ? (int)blockDim.x - 32 * warps : (int)blockDim.x;
+        const int wall_thread = (int)(blockDim.x - 1 - threadIdx.x);
+        const TileWalls W(k, X0, X1, Y0, Y1);
+        const int nw = W.count();
+        for (int n = wall_thread < wall_threads ? wall_thread : nw; n < nw; n += wall_threads) {
+            int X, Y;
+            W.at(n, X, Y);
+            tile_wall_m(k, TileSource{slots, X0 - 1, Y0 - 1}, dst, X, Y);
+        }
+    }
+}
+
+// Two steps of a batch of FP32 cavities walled on all four sides: block i takes
 // tile i of the list (cavity by cavity, tiles of the large shape) and reads the
 // cavity's constants from shared memory (128 cavities of 64^2 to 512^2: 54.5
 // GLUPS against 44 of the staged one-step kernel).  TAU1: every cavity has tau_f = tau_T =
@@ -432,6 +564,41 @@ cudaError_t launch_two_steps_batch(const BatchCavity<float>* cav, const void* pa
     cfg.numAttrs = 1;
     return tau1 ? cudaLaunchKernelEx(&cfg, k_tile_batch<true>, cav, (const PairConst*)pair, items, src, dst)
                 : cudaLaunchKernelEx(&cfg, k_tile_batch<false>, cav, (const PairConst*)pair, items, src, dst);
+}
+
+template <bool E, bool S>
+static cudaError_t launch_tile_m(cudaLaunchConfig_t& cfg, const KConst<float>& k, const float* src, float* dst,
+                                 const TileSplit& sx, const TileSplit& sy, int warps, bool early) {
+    const PairConst pc = make_pair_const(k, 1.0f);
+    return cudaLaunchKernelEx(&cfg, k_tile_m<E, S>, k, pc, src, dst, sx, sy, warps, early);
+}
+
+bool moment_tiles_preferred(const KConst<float>& k, int sms) {
+    return two_steps_supported(k) &&
+           (long long)tile_split(k.nx, 2, kTilePairs).n * tile_split(k.ny, 1, kTileLarge.rows).n <= 16LL * sms;
+}
+
+cudaError_t launch_step_m_tiles(const KConst<float>& k, const float* src, float* dst, bool sources, int sms, cudaStream_t st) {
+    if (!two_steps_supported(k)) return cudaErrorInvalidValue;
+    const TileSplit sx = tile_split(k.nx, 2, kTilePairs);
+    const bool small = (long long)sx.n * tile_split(k.ny, 1, kTileSmall.rows).n <= (long long)kTileSmallWaves * sms;
+    const TileShape shape = small ? kTileSmall : kTileLarge;
+    const TileSplit sy = tile_split(k.ny, 1, shape.rows);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)sx.n, (unsigned)sy.n);
+    cfg.blockDim = dim3((unsigned)(32 * (shape.warps + shape.wall_warps)));
+    cfg.dynamicSmemBytes = tile_smem(shape.rows);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (k.eps_field)
+        return sources ? launch_tile_m<true, true>(cfg, k, src, dst, sx, sy, shape.warps, !small)
+                       : launch_tile_m<true, false>(cfg, k, src, dst, sx, sy, shape.warps, !small);
+    return sources ? launch_tile_m<false, true>(cfg, k, src, dst, sx, sy, shape.warps, !small)
+                   : launch_tile_m<false, false>(cfg, k, src, dst, sx, sy, shape.warps, !small);
 }
 
 bool two_steps_supported(const KConst<float>& k) { return k.nx >= 8 && k.ny >= 8; }
