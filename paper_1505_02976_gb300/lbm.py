@@ -203,12 +203,14 @@ def _ptr(a):
 
 
 def _moment_arrays(ny: int, nx: int) -> dict:
-    """p, ux, uy, T as the four parts of one allocation: the library then
-    fetches them in one copy, and the fresh pages of one large array cost less
-    than those of four (numpy asks for huge pages from 4 MB on).  128 cavities of
-    100 to 250 columns: 75 -> 6 ms, 80 -> 36 ms where all fields are kept.  (A
-    part that is kept keeps all four: copy it to keep one alone.)"""
-    fields = np.empty((4, ny, nx))
+    """p, ux, uy, T.  Up to 16 MB they are the four parts of one allocation: the
+    library then fetches them in one copy, and the fresh pages of one large
+    array cost less than those of four (numpy asks for huge pages from 4 MB on;
+    128 cavities of 64^2 to 512^2: 75 -> 6 ms, 80 -> 36 ms where all fields are
+    kept; a part that is kept keeps all four).  Above, where the C library maps
+    each allocation of more than 32 MB anew and only smaller ones come back from
+    its heap, each field is its own (1025^2 with its fields: 3.9 ms, 5.4 as one)."""
+    fields = [np.empty((ny, nx)) for _ in range(4)] if 32 * nx * ny > 2**24 else np.empty((4, ny, nx))
     return dict(zip(("p", "ux", "uy", "T"), fields))
 
 
