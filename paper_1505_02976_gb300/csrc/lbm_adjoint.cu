@@ -366,7 +366,7 @@ struct Interior {
 // latency of its chain (loads, ~600 dependent operations, stores).  Before, 9
 // to 11 forward-mode passes a node in a thread each, then a combining and a
 // gathering launch: whole calls with 256 steps at 256^2 FP32 took 38.0 ms
-// against 7.0 ms, with 100 steps at 65 x 49 FP64 45.7 against 6.6 ms (forward and
+// against 7.0 ms, with 100 steps at 65 x 49 FP64 45.7 against 6.3 ms (forward and
 // recomputed steps included; 7.5 and 8.4 ms with the wall nodes' chains in the
 // threads of the nodes they hang on).
 constexpr int kAdjNodes = 64, kAdjRing = 32;
@@ -639,10 +639,10 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
     const size_t sb = h->L.buf_bytes;  // one state
     // few and small states are all kept as the forward pass computes them, and
     // nothing is recomputed (65 x 49 FP64, 100 steps: 4.7 ms a call
-    // against 5.7 with checkpoints)
-    const bool keep = seg_len == 0 && (double)sb * (double)n <= (double)kKeepBytes;
-    const int64_t K = keep ? n : (seg_len > 0 ? seg_len : (int64_t)ceil(sqrt((double)n)));
-    const int64_t nseg = (n + K - 1) / K;
+    // against 5.7 with checkpoints); where the memory for that is not to be had,
+    // checkpoints are
+    bool keep = seg_len == 0 && (double)sb * (double)n <= (double)kKeepBytes;
+    const int64_t seg = seg_len > 0 ? seg_len : (int64_t)ceil(sqrt((double)n));
     const size_t lam_bytes = 17 * (size_t)k.plane * sizeof(R);    // one adjoint state
     std::vector<void*> allocs;
     auto fail_free = [&](lbm_status s, const std::string& m) {
@@ -656,13 +656,19 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
         allocs.push_back(a);
         return a;
     };
-    char* ckpt = (char*)alloc(keep ? 256 : sb * (size_t)nseg);
-    char* segs = (char*)alloc(sb * (size_t)K);
     R* lam0 = (R*)alloc(lam_bytes);
     R* lam1 = (R*)alloc(lam_bytes);
     const size_t ff_bytes = (size_t)k.plane * sizeof(R);
     R* ff0 = (R*)alloc(2 * ff_bytes);  // T(x_ff) adjoints left at the wall nodes, two buffers
     double* g = (double*)alloc(3 * N * sizeof(double));  // g_eps, g_tb, dL/dT
+    char* segs = keep ? (char*)alloc(sb * (size_t)n) : nullptr;
+    if (keep && !segs) {
+        (void)cudaGetLastError();
+        keep = false;
+    }
+    const int64_t K = keep ? n : seg, nseg = (n + K - 1) / K;
+    char* ckpt = keep ? segs : (char*)alloc(sb * (size_t)nseg);
+    if (!keep) segs = (char*)alloc(sb * (size_t)K);
     if (!ckpt || !segs || !lam0 || !lam1 || !ff0 || !g)
         return fail_free(LBM_ERR_OOM, "adjoint buffers (checkpoints grow as sqrt(n))");
     R* ff1 = ff0 + k.plane;
@@ -677,7 +683,7 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
     auto kept = [&](int64_t t) { return (S*)(segs + sb * (size_t)t); };  // state t of the segment in hand
     for (int64_t t = 0; t < n;) {
         if (t % K == 0)
-            if (cudaMemcpyAsync(keep ? segs : ckpt + sb * (size_t)(t / K), h->buf(h->cur), sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+            if (cudaMemcpyAsync(ckpt + sb * (size_t)(t / K), h->buf(h->cur), sb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
                 return fail_free(LBM_ERR_CUDA, "checkpoint copy");
         // as many steps as one launch takes, up to the next checkpoint
         const int64_t m = steps_of_launch<S>(h, std::min(K - t % K, n - t));
