@@ -263,56 +263,6 @@ __device__ __forceinline__ Acc pull_hsum(const KConst<R>& k, const S* __restrict
     return s;
 }
 
-// ------------------------------------------------------------ dual numbers
-// Forward-mode derivatives: a value and one tangent.  The generic per-node
-// functions below are templates over the value type V (R, or Dual<R> for
-// the adjoint), so the adjoint differentiates exactly the code that runs.
-template <class R>
-struct Dual {
-    R v, d;
-    __host__ __device__ Dual() : v(R(0)), d(R(0)) {}
-    __host__ __device__ Dual(R v_) : v(v_), d(R(0)) {}
-    __host__ __device__ Dual(R v_, R d_) : v(v_), d(d_) {}
-};
-template <class R> __device__ __forceinline__ Dual<R> operator+(Dual<R> a, Dual<R> b) { return {a.v + b.v, a.d + b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a, Dual<R> b) { return {a.v - b.v, a.d - b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(Dual<R> a, Dual<R> b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator/(Dual<R> a, Dual<R> b) {
-    const R q = a.v / b.v;
-    return {q, (a.d - q * b.d) / b.v};
-}
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a) { return {-a.v, -a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator+(Dual<R> a, R b) { return {a.v + b, a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator+(R a, Dual<R> b) { return {a + b.v, b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a, R b) { return {a.v - b, a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(R a, Dual<R> b) { return {a - b.v, -b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(Dual<R> a, R b) { return {a.v * b, a.d * b}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(R a, Dual<R> b) { return {a * b.v, a * b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator/(Dual<R> a, R b) { return {a.v / b, a.d / b}; }
-template <class R> __device__ __forceinline__ Dual<R> operator/(R a, Dual<R> b) {
-    const R q = a / b.v;
-    return {q, -q * b.d / b.v};
-}
-
-template <class R> __device__ __forceinline__ R val(R x) { return x; }
-template <class R> __device__ __forceinline__ R val(Dual<R> x) { return x.v; }
-
-// Square root of an argument that is never zero.
-template <class R> __device__ __forceinline__ R vsqrt(R x) { return sqrt(x); }
-template <class R> __device__ __forceinline__ Dual<R> vsqrt(Dual<R> x) {
-    const R r = sqrt(x.v);
-    return {r, x.d / (R(2) * r)};
-}
-// Euclidean norm from its square.  Where the vector is zero the norm is not
-// differentiable, but it only enters multiplied by the vector itself
-// (abs(v) v in the quadratic solve, abs(u) u in the Forchheimer drag), whose
-// derivative there is zero: the tangent is set to 0.
-template <class R> __device__ __forceinline__ R vnorm(R sq) { return sqrt(sq); }
-template <class R> __device__ __forceinline__ Dual<R> vnorm(Dual<R> sq) {
-    const R r = sqrt(sq.v);
-    return {r, r > R(0) ? sq.d / (R(2) * r) : R(0)};
-}
-
 // Porosity-dependent constants of one node, and the y-component of the
 // external acceleration a at its row.
 template <class V>
@@ -361,8 +311,8 @@ __device__ __forceinline__ CellC<V> cell_consts(const KConst<R>& k, V eps) {
         const V ratio = eps * eps * eps / (om * om) * k.kc_inv_ref;  // K / K_ref
         c.e_nuK = eps * k.nu_over_Kref / ratio;
         if (k.forch) {
-            const V Feps = R(1.75) / vsqrt(R(150) * eps * eps * eps);
-            c.e_FK = eps * Feps * k.inv_sqrt_Kref / vsqrt(ratio);
+            const V Feps = R(1.75) / sqrt(R(150) * eps * eps * eps);
+            c.e_FK = eps * Feps * k.inv_sqrt_Kref / sqrt(ratio);
         } else {
             c.e_FK = V(R(0));
         }
@@ -407,12 +357,12 @@ __device__ __forceinline__ State<V> node_moments(const KConst<R>& k, const CellC
     const V Gy = k.gbeta * s.th + c.ay;
     const V vx = mx * k.inv_rho0 + R(0.5) * c.eps * Gx;
     const V vy = my * k.inv_rho0 + R(0.5) * c.eps * Gy;
-    const V vmag = vnorm(vx * vx + vy * vy);
-    const V den = c.c0 + vsqrt(c.c0sq + c.c1 * vmag);
+    const V vmag = sqrt(vx * vx + vy * vy);
+    const V den = c.c0 + sqrt(c.c0sq + c.c1 * vmag);
     s.ux = vx / den;
     s.uy = vy / den;
     const V uu = s.ux * s.ux + s.uy * s.uy;
-    const V umag = vnorm(uu);
+    const V umag = sqrt(uu);
     const V drag = c.e_nuK + c.e_FK * umag;
     s.Fx = c.eps * Gx - drag * s.ux;
     s.Fy = c.eps * Gy - drag * s.uy;
@@ -508,7 +458,7 @@ __device__ __forceinline__ State<V> wall_state(const KConst<R>& k, const CellC<V
         if (w.fixgy) b.gy = V(R(0));
         b.th = (R(4) * sf.th - thff) * (R(1) / R(3));
     }
-    const V umag = vnorm(b.ux * b.ux + b.uy * b.uy);
+    const V umag = sqrt(b.ux * b.ux + b.uy * b.uy);
     const V drag = cb.e_nuK + cb.e_FK * umag;
     b.Fx = cb.eps * k.ax - drag * b.ux;
     b.Fy = cb.eps * (k.gbeta * b.th + cb.ay) - drag * b.uy;
