@@ -257,13 +257,13 @@ inline lbm::KConst<R> make_kconst(const lbm_params* p, const Derived& d, const L
     k.qF_ie = R(rho0 * (9.0 * kf + aS));
     k.f_cu = R(3.0 * rho0 * itf);
     // In FP32 each step scales the momentum by 1 - 1/tau + (f_cu/rho0) (2 w_1 + 4
-    // w_5) = 1 - 1.5e-8/tau.  The drag coefficient gives a twenty-fifth of that
-    // back: not to cancel it, but so that the drag is nowhere exactly zero and
-    // the tied roundings of f_cu u_x + f_cF F_x in a clear fluid do not all go to
-    // even (residual of a clear 201^2 cavity after 100 steps against 64 bits:
-    // 2.0e-6 off without, 5e-7 with; other flows move by less than 1e-6).
-    const double drift = 1.0 - 3.0 * (2.0 * double(R(1) / R(9)) + 4.0 * double(lbm::w_diag<R>()));
-    k.nnuK_0 = sizeof(R) == 4 ? R(0.04 * itf * drift / kf) : R(0);
+    // w_5) = 1 - 1.5e-8/tau.  In a clear fluid (Darcy drag smaller than that)
+    // nothing else damps it, and tied roundings of f_cu u_x add to it: there the
+    // drag coefficient gives it back (u of clear 90^2 to 400 x 301 cavities after
+    // 100 steps against 64 bits: 2e-6 too small without, 3e-7 off with).  Where
+    // there is drag it stays.
+    const double back = itf / kf * (1.0 - 3.0 * (2.0 * double(R(1) / R(9)) + 4.0 * double(lbm::w_diag<R>())));
+    k.nnuK_0 = sizeof(R) == 4 && eps * nuK < back ? R(back) : R(0);
     // The sum of the collided f_1..f_8 is fA wsum (eps p) + tsum tr Q, and the
     // u u and u F parts of the two cancel (e2 = -(4/5) rho0 kf tau/eps, e3 =
     // -(2/5) rho0/eps): fitted to the factors as R holds them, since the rest
