@@ -13,7 +13,7 @@
  * the local shear-rate and temperature-gradient schemes of Sec. 3.3
  * (Eqs. ShearEqCom, TeEqCom) and the non-equilibrium extrapolation walls of
  * Sec. 3.4 (Eqs. NEESVel, TNEESAp, TNEESApGra), all fused into one kernel
- * launch per step.  Lattice units throughout: dx = dt = 1, c_s^2 = 1/3.
+ * launch per step (one per two steps of an FP32 lattice).  Lattice units throughout: dx = dt = 1, c_s^2 = 1/3.
  *
  * Conventions shared by every entry point
  * ----------------------------------------

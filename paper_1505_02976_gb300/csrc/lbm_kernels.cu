@@ -13,8 +13,6 @@
 
 namespace lbm {
 
-
-
 // The fused step: one thread per node.  The first `wall_blocks` blocks take the
 // wall nodes in perimeter order (the NEES path), the others the interior nodes
 // row by row, bx blocks a row: a warp then runs one of the two paths, where a
@@ -27,8 +25,8 @@ namespace lbm {
 // direction-by-direction arithmetic too); blocks of one warp end most evenly
 // (130 us in blocks of four).  A lattice that leaves SMs empty is bound by one
 // warp's chain, and blocks of one warp put every warp on an SM of its own: 32^2
-// 8.7 us a step (10.0 in blocks of four; 17.3 with the wall nodes inside, 38
-// before).
+// 8.6 us a step (10.0 in blocks of four; 17.3 with the wall nodes inside, 38
+// before), 7.1 with SPLIT (below).
 // One block's share: block b of the numbering above.  PART: lbm_step.cuh.
 template <class R, class S, bool EPS_FIELD, bool TAU1, int PART>
 __device__ __forceinline__ void step_block(const KConst<R>& k, const S* __restrict__ src, S* __restrict__ dst, unsigned b,

@@ -20,8 +20,8 @@
 //
 // Bound: neither pipe alone.  2048^2: 285 + 236 MB of DRAM traffic and 67 M
 // warp instructions a launch, issue 48 % active with 18 warps an SM, DRAM at
-// 4.5 TB/s; 57.4 us a step in the timed loop (73 GLUPS) against 86 us (48.7) of
-// the one-step staged kernel, which is at 0.98 of measured HBM; 4096^2 222 us
+// 4.5 TB/s; 58.4 us a step in the timed loop (72 GLUPS) against 86 us (48.7) of
+// the one-step staged kernel, which is at 0.98 of measured HBM; 4096^2 219 us
 // (76); 1024 x 513 periodic 9.0 us against 12.7 of the global-load kernel;
 // 1000 x 777 with a porosity field off tau = 1 14.6 us against 24.
 // Copying the pulls into the shared rows asynchronously (cp.async, every row of
