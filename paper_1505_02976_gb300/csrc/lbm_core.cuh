@@ -84,9 +84,9 @@ __device__ __forceinline__ float lrcp(float a) {
 // third order, Newton's iteration for 1/a and 1/sqrt(a) with the next term of
 // its series: with e = 1 - a r, 1/a = r/(1 - e) = r (1 + e + e^2 + ...); with
 // y ~ 1/sqrt(a), g = a y and 2 d = 1 - g y, sqrt(a) = g/sqrt(1 - 2 d) =
-// g (1 + d + 3/2 d^2 + ...).  Arguments here are positive and normal, or zero
-// under the root; over 2^24 random arguments in 2^-60 .. 2^60 at most 0.51 and
-// 0.76 units in the last place off.  FP64 instructions of the step at 700 x 517:
+// g (1 + d + 3/2 d^2 + ...).  Reciprocals here are of positive normal values; over
+// 2^24 random arguments in 2^-60 .. 2^60 at most 0.51 and 0.76 units in the
+// last place off.  FP64 instructions of the step at 700 x 517:
 // 2.21 -> 2.06 M a launch against the language's division and square root,
 // 139.6 -> 130.6 us.
 __device__ __forceinline__ double lrcp(double a) {
@@ -98,7 +98,10 @@ __device__ __forceinline__ double lrcp(double a) {
 __device__ __forceinline__ double lsqrt(double a) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    if (__double2hiint(a) == 0) y = 0.0;  // a = 0 (below 1e-308): 0
+    // The approximation takes subnormal arguments for 0 and gives infinity: the
+    // root of these is 0 here.  They are |v|^2 of |v| < 1.5e-154, which the step
+    // adds (times c1, or F_e/sqrt(K)) to numbers it is far below the last place of.
+    if (__double2hiint(a) < 0x00100000) y = 0.0;
     const double g = __dmul_rn(a, y), d = __fma_rn(-g, __dmul_rn(0.5, y), 0.5);
     return __fma_rn(g, __dmul_rn(d, __fma_rn(1.5, d, 1.0)), g);
 }
