@@ -80,20 +80,21 @@ __device__ __forceinline__ float lrcp(float a) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-// FP64: from the hardware's approximations (about 2^-20 off) by one step of
-// third order, Newton's iteration for 1/a and 1/sqrt(a) with the next term of
-// its series: with e = 1 - a r, 1/a = r/(1 - e) = r (1 + e + e^2 + ...); with
-// y ~ 1/sqrt(a), g = a y and 2 d = 1 - g y, sqrt(a) = g/sqrt(1 - 2 d) =
-// g (1 + d + 3/2 d^2 + ...).  Reciprocals here are of positive normal values; over
-// 2^24 random arguments in 2^-60 .. 2^60 at most 0.51 and 0.76 units in the
-// last place off.  FP64 instructions of the step at 700 x 517:
-// 2.21 -> 2.06 M a launch against the language's division and square root,
-// 139.6 -> 130.6 us.
+// FP64: from the hardware's approximations (about 2^-20 off) by Newton's
+// iteration, once for the value and once more for its last place, so that the
+// rounding of the last operation is all that is left: r' = r + r (1 - a r) twice
+// for 1/a; with y ~ 1/sqrt(a), g = a y and h = y/2, d = 1/2 - g h once for both
+// (g + g d ~ sqrt(a), h + h d ~ 1/(2 sqrt(a))), then g + h (a - g^2).
+// Reciprocals here are of positive normal values.  Both are within 0.501 units in
+// the last place, as the language's are, over 2^-900 .. 2^900.  700 x 517 with 50
+// steps: 6.81 ms, about 7.2 with the language's; one iteration of third order instead
+// of the two takes four FP64 instructions a node less (6.69 ms) and leaves 0.76
+// and 0.51 units.
 __device__ __forceinline__ double lrcp(double a) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = __fma_rn(-a, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
+    r = __fma_rn(r, __fma_rn(-a, r, 1.0), r);
+    return __fma_rn(r, __fma_rn(-a, r, 1.0), r);
 }
 __device__ __forceinline__ double lsqrt(double a) {
     double y;
@@ -102,8 +103,11 @@ __device__ __forceinline__ double lsqrt(double a) {
     // root of these is 0 here.  They are |v|^2 of |v| < 1.5e-154, which the step
     // adds (times c1, or F_e/sqrt(K)) to numbers it is far below the last place of.
     if (__double2hiint(a) < 0x00100000) y = 0.0;
-    const double g = __dmul_rn(a, y), d = __fma_rn(-g, __dmul_rn(0.5, y), 0.5);
-    return __fma_rn(g, __dmul_rn(d, __fma_rn(1.5, d, 1.0)), g);
+    double g = __dmul_rn(a, y), h = __dmul_rn(0.5, y);
+    const double d = __fma_rn(-g, h, 0.5);
+    g = __fma_rn(g, d, g);
+    h = __fma_rn(h, d, h);
+    return __fma_rn(__fma_rn(-g, g, a), h, g);
 }
 __device__ __forceinline__ float2 lsqrt(float2 a) { return make_float2(lsqrt(a.x), lsqrt(a.y)); }
 __device__ __forceinline__ float2 lrcp(float2 a) { return make_float2(lrcp(a.x), lrcp(a.y)); }

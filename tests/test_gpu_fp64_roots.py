@@ -64,3 +64,13 @@ def test_root_and_reciprocal_of_normal_values(roots):
     root, inverse = roots(x)
     assert np.all(np.abs(root - np.sqrt(x)) <= np.spacing(np.sqrt(x)))
     assert np.all(np.abs(inverse - 1.0 / x) <= np.spacing(1.0 / x))
+
+
+def test_root_and_reciprocal_are_rounded_once(roots):
+    """At most half a unit in the last place off (and 1e-3 of one), as the language's own."""
+    x = np.r_[_samples(-900, 900, 1 << 18, 3), _samples(-4, 5, 1 << 19, 4), np.nextafter(1.0, [0.0, 2.0]), 0.25, 1.0, 2.0, 4.0]
+    root, inverse = roots(x)
+    wide = x.astype(np.longdouble)
+    for got, want in ((root, np.sqrt(wide)), (inverse, 1 / wide)):
+        ulp = np.spacing(np.abs(want).astype(np.float64))
+        assert np.max(np.abs(got.astype(np.longdouble) - want) / ulp) <= 0.501
