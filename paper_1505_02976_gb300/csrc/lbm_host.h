@@ -97,14 +97,25 @@ inline size_t elem_size(int precision) {
 
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
+// Host memory that CUDA knows nothing of (not page-locked, not managed).
+inline bool pageable(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeUnregistered;
+    (void)cudaGetLastError();
+    return false;
+}
+
 // The four moment fields from the device area F (nx ny doubles each, one after
-// the other) to outs (null: not wanted), fields that lie one after the other at
-// the destination too in one copy: a pageable copy costs 10 us before its first
-// byte (256^2: 60 -> 35 us a call).
+// the other) to outs (null: not wanted).  Pageable host fields that lie one
+// after the other go in one copy: each costs 10 us before its first byte (256^2:
+// 60 -> 35 us a call).  Other memory is copied field by field: fields that touch
+// may belong to two allocations or registrations, which one copy must not span.
 inline cudaError_t copy_moments(double* const outs[4], const double* F, size_t N, cudaMemcpyKind kind, cudaStream_t st) {
+    bool joins[4];
+    for (int q = 0; q < 4; ++q) joins[q] = outs[q] && kind == cudaMemcpyDeviceToHost && pageable(outs[q]);
     for (int q = 0; q < 4;) {
         int n = 1;
-        while (outs[q] && q + n < 4 && outs[q + n] == outs[q] + n * N) ++n;
+        while (joins[q] && q + n < 4 && joins[q + n] && outs[q + n] == outs[q] + n * N) ++n;
         if (outs[q]) {
             const cudaError_t e = cudaMemcpyAsync(outs[q], F + q * N, n * N * sizeof(double), kind, st);
             if (e != cudaSuccess) return e;
