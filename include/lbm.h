@@ -141,8 +141,10 @@ lbm_status lbm_set_moment_segments(lbm_handle* h, int32_t segments);
  * shared memory with tensor copies and waits on them with bounded waits.
  * staged = 0 selects the kernel in which every thread loads its own 17
  * values from global memory, one step per launch; staged = 1 restores the default
- * (LBM_ERR_ARG where it is unavailable: FP64, a periodic side, the moment
- * state, a lattice under 4 x 4, or a CUDA driver without tensor-map encoding).
+ * (LBM_ERR_ARG where no rows can be staged: FP64, a periodic side, the moment
+ * state, a lattice under 4 x 4, or a CUDA driver without tensor-map encoding;
+ * an FP32 lattice that takes its steps in pairs returns to that from an
+ * earlier staged = 0 all the same).
  * Both kernels run the same per-node arithmetic (results agree to rounding;
  * bit for bit in FP32 at tau_f = tau_T = 1).  In FP16 at tau_f = tau_T = 1
  * the staged kernel computes pairs of interior nodes with packed FP32

@@ -252,7 +252,8 @@ lbm_status lbm_create(const lbm_params* p, void* stream, void* workspace, size_t
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         (void)cudaGetLastError();
-    h->two_steps = p->precision == LBM_F32 && !p->moment_state && lbm::two_steps_supported(h->k32);
+    h->two_steps_ready = p->precision == LBM_F32 && !p->moment_state && lbm::two_steps_supported(h->k32);
+    h->two_steps = h->two_steps_ready;
     h->msegments = 0;
     h->diag.T0 = d.T0;
     h->diag.inv_sigma = 1.0 / p->sigma;
@@ -426,10 +427,12 @@ lbm_status lbm_step(lbm_handle* h, int64_t n) {
 
 lbm_status lbm_set_step_staging(lbm_handle* h, int32_t staged) {
     if (!h) return LBM_ERR_ARG;
-    if (staged && !h->tma_ready)
+    // without staged rows, 1 only undoes an earlier 0
+    const bool undoes = h->two_steps_ready && !h->two_steps;
+    if (staged && !h->tma_ready && !undoes)
         return fail(h, LBM_ERR_ARG, "staged rows need FP32 or FP16 populations on a lattice walled on all sides");
-    h->tma = staged != 0;
-    h->two_steps = staged != 0 && h->prm.precision == LBM_F32 && lbm::two_steps_supported(h->k32);
+    h->tma = staged != 0 && h->tma_ready;
+    h->two_steps = staged != 0 && h->two_steps_ready;
     return LBM_OK;
 }
 

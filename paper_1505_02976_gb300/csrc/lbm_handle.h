@@ -30,7 +30,7 @@ struct lbm_handle {
     CUtensorMap tmap[2];
     int tma_rows;
     int sms;
-    bool two_steps;  // FP32 populations: pairs of steps go through launch_two_steps
+    bool two_steps, two_steps_ready;  // FP32 populations: pairs of steps go through launch_two_steps, and whether they can
     bool nonfinite, timeout;
     lbm::KConst<double> k64;
     lbm::KConst<float> k32;
