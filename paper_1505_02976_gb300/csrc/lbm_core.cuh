@@ -571,11 +571,11 @@ __device__ __forceinline__ void expand_moments(const Q& q, const Cell<L>& c, L e
                              typename LaneReal<L>::type(1));
 }
 
-// Wall node at tau_f = tau_T = 1 (Sec. 3.4): there the extrapolated
-// non-equilibrium part carries the factor 1 - 1/tau = 0, so the node is the
-// collision of its boundary state b alone.  s, S: state and shear rate of
-// x_f (on entry s; b on return), cs / cb: constants of x_f and of the node,
-// thff: T(x_ff) - T0, thb: the Dirichlet T_b - T0 where `given`.
+// Boundary state b of a wall node (Sec. 3.4); S(x_f) stands beside it.  At tau_f =
+// tau_T = 1 the extrapolated non-equilibrium part carries the factor 1 - 1/tau =
+// 0, and the node is the collision of b alone.  s: state of x_f on entry, b on
+// return; cs / cb: constants of x_f and of the node, thff: T(x_ff) - T0, thb: the
+// Dirichlet T_b - T0 where `given`.
 template <class R>
 __device__ __forceinline__ void core_boundary(const KConst<R>& k, const Cell<R>& cs, const Cell<R>& cb, R eay_b,
                                               R ubx, R uby, R ubm, bool given, bool fixgx, bool fixgy, R thb, R thff,
@@ -596,6 +596,62 @@ __device__ __forceinline__ void core_boundary(const KConst<R>& k, const Cell<R>&
     const R nd = lfma(cb.nFK, ubm, cb.nnuK);
     s.Fx = lfma(nd, s.ux, cb.eax);
     s.Fy = lfma(nd, s.uy, lfma(cb.eg, s.th, eay_b));
+}
+
+// Wall node at any relaxation times: f* = (1 - 1/tau) [f(x_f) - f^eq(s)] +
+// f^eq(b) + F_i(b) and g* likewise (Eqs. NEESVel, TNEESAp), the two equilibria and the
+// sources gathered into one scalar, form and vector per distribution as in
+// core_emit.  s, S: state and shear rate of x_f, b: the boundary state
+// (core_boundary), cs / cb their constants, f, h: the values pulled at x_f.
+template <class R>
+__device__ __forceinline__ void wall_emit(const KConst<R>& k, const Cell<R>& cs, const Cell<R>& cb, const CoreState<R>& s,
+                                          const Shear<R>& S, const CoreState<R>& b, const R* f, const R* h, R* fo, R* ho) {
+    const CoreWeights<R> w_ = core_weights(k, R(1));
+    const R third = R(1) / R(3);
+    {
+        const R m = -k.omf, c2 = lmul(R(4.5), cs.re), cb2 = lmul(R(4.5), cb.re), cF = lmul(lmul(R(9), k.kf), cb.re);
+        const R sx = lmul(c2, s.ux), sy = lmul(c2, s.uy);
+        const R tx = lfma(cb2, b.ux, lmul(cF, b.Fx)), ty = lfma(cb2, b.uy, lmul(cF, b.Fy));
+        const R fS = lmul(lmul(lmul(R(1.5), k.rho0), k.A), ladd(R(1), m));  // S is that of x_f in both
+        const R Qxx = lfma(m, lmul(s.ux, sx), lfma(b.ux, tx, lmul(fS, S.xx)));
+        const R Qyy = lfma(m, lmul(s.uy, sy), lfma(b.uy, ty, lmul(fS, S.yy)));
+        const R Q2 = lfma(m, lfma(s.ux, sy, lmul(s.uy, sx)), lfma(b.ux, ty, lfma(b.uy, tx, lmul(lmul(R(2), fS), S.xy))));
+        const R tr = ladd(Qxx, Qyy), E = lfma(-third, tr, lmul(R(3), lfma(m, s.ep, b.ep))), Ed = ladd(E, tr);
+        const R c1 = lmul(R(3), k.rho0), cf = lmul(c1, k.kf);
+        const R Dx = lfma(c1, lfma(m, s.ux, b.ux), lmul(cf, b.Fx)), Dy = lfma(c1, lfma(m, s.uy, b.uy), lmul(cf, b.Fy));
+        auto put = [&](int i, int j, R w, R n, R e, R d) {
+            const R we = lmul(w, e);
+            fo[i] = lfma(w, d, lfma(k.omf, f[i], we));
+            fo[j] = lfma(n, d, lfma(k.omf, f[j], we));
+        };
+        put(1, 3, w_.w1, w_.n1, ladd(E, Qxx), Dx);
+        put(2, 4, w_.w1, w_.n1, ladd(E, Qyy), Dy);
+        put(5, 7, w_.w5, w_.n5, ladd(Ed, Q2), ladd(Dx, Dy));
+        put(6, 8, w_.w5, w_.n5, lsub(Ed, Q2), lsub(Dy, Dx));
+    }
+    {
+        const R m = -k.omT, ks = lmul(lmul(R(4.5), cs.ie), s.T), kb = lmul(lmul(R(4.5), cb.ie), b.T);
+        const R sx = lmul(ks, s.ux), sy = lmul(ks, s.uy), tx = lmul(kb, b.ux), ty = lmul(kb, b.uy);
+        const R Kxx = lfma(m, lmul(sx, s.ux), lmul(tx, b.ux)), Kyy = lfma(m, lmul(sy, s.uy), lmul(ty, b.uy));
+        const R K2 = lmul(R(2), lfma(m, lmul(sx, s.uy), lmul(tx, b.uy)));
+        const R tr = ladd(Kxx, Kyy), th = lmul(k.sigma, lfma(m, s.th, b.th)), m0 = lfma(-third, tr, k.h_kQ);
+        const R pT = lmul(lmul(R(3), k.inv_rho0), lfma(m, lmul(s.T, s.ep), lmul(b.T, b.ep)));
+        const R e = ladd(m0, pT), ed = ladd(e, tr);
+        const R sB = lmul(k.sigma, k.B), hg = lfma(k.h_Wr, b.ep, sB), hT = lmul(k.h_W, b.T), T3 = lmul(R(3), s.T);
+        const R K = lfma(R(3), b.T, lfma(cb.ug, lfma(b.ux, b.gx, lmul(b.uy, b.gy)), k.h_uQ));
+        const R Vx = lfma(m, lfma(T3, s.ux, lmul(sB, s.gx)), lfma(K, b.ux, lfma(hg, b.gx, lmul(hT, b.Fx))));
+        const R Vy = lfma(m, lfma(T3, s.uy, lmul(sB, s.gy)), lfma(K, b.uy, lfma(hg, b.gy, lmul(hT, b.Fy))));
+        auto put = [&](int i, int j, R w, R small, R d) {
+            const R even = ladd(th, small), wd = lmul(w, d);
+            ho[i] = lfma(w, even, lfma(k.omT, h[i], wd));
+            ho[j] = lfma(w, even, lfma(k.omT, h[j], lneg(wd)));
+        };
+        put(1, 3, w_.w1, ladd(e, Kxx), Vx);
+        put(2, 4, w_.w1, ladd(e, Kyy), Vy);
+        put(5, 7, w_.w5, ladd(ed, K2), ladd(Vx, Vy));
+        put(6, 8, w_.w5, lsub(ed, K2), lsub(Vy, Vx));
+        ho[0] = lfma(w_.w0, ladd(th, m0), lfma(k.omT, h[0], lmul(-(R(5) / R(9)), pT)));
+    }
 }
 
 }  // namespace lbm

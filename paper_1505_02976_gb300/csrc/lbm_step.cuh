@@ -137,33 +137,29 @@ __device__ __forceinline__ void wall_node_tau1(const KConst<R>& k, const Source&
     if (!lfinite(ho[0])) atomicOr(k.flag, 1);
 }
 
-// The same at other relaxation times: the generic update of its x_f
-// neighbour's pulled populations (NEES rebuild and boundary collision, see
-// node_update_generic).
+// The same at other relaxation times, where the non-equilibrium part stays
+// (wall_emit).  Every operation is spelled out here too: kernels that take one
+// and two steps, from global and from shared memory, give the same bits.
 template <class R, class Source>
 __device__ __forceinline__ void wall_node_generic(const KConst<R>& k, const Source& source, int x, int y, R* fo, R* ho) {
     const WallInfo w = classify(k, x, y);
     Pops<R> P;
     source(k, w.xs, w.ys, P);
-    R in[17], out[17];
-#pragma unroll
-    for (int i = 1; i < 9; ++i) in[i - 1] = P.f[i];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) in[8 + i] = P.h[i];
     R thff = R(0);
     if (w.tside < 0) {
         Pops<R> Q;
-        source(k, w.xff, w.yff, Q);
-        thff = (Q.h[0] + Q.h[1] + Q.h[2] + Q.h[3] + Q.h[4] + Q.h[5] + Q.h[6] + Q.h[7] + Q.h[8] + R(0.5) * k.Q) * k.inv_sigma;
+        source(k, w.xff, w.yff, Q);  // only h is used
+        thff = core_theta(k, core_hsum(Q.h));
     }
+    const Cell<R> cs = node_cell(k, w.xs, w.ys), cb = node_cell(k, x, y);
+    const CoreState<R> s = core_moments(k, cs, eps_ay(k, k, cs, w.ys), P.f, P.h);
+    const Shear<R> S_ = core_shear(k, cs, s);
     const R thb = w.tside >= 0 ? k.T_bc[w.tside] - k.T0 : R(0);
-    node_update_generic(k, w, in, node_eps(k, w.xs, w.ys), node_eps(k, x, y), thff, thb, row_ay(k, w.ys),
-                        row_ay(k, y), out);
-    if (!isfinite(out[0] + out[8])) atomicOr(k.flag, 1);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) fo[i] = out[i - 1];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) ho[i] = out[8 + i];
+    CoreState<R> b = s;
+    core_boundary(k, cs, cb, eps_ay(k, k, cb, y), k.u_bc[w.uside][0], k.u_bc[w.uside][1], k.u_abs[w.uside], w.tside >= 0,
+                  w.fixgx != 0, w.fixgy != 0, thb, thff, b);
+    wall_emit(k, cs, cb, s, S_, b, P.f, P.h, fo, ho);
+    if (!lfinite(fo[1]) || !lfinite(ho[0])) atomicOr(k.flag, 1);
 }
 
 // Both out of line: only the 4(N - 1) wall threads take them.
