@@ -218,6 +218,7 @@ inline PairConst make_pair_const(const KConst<float>& k, float scale) {
     q.cell.nFK = two(k.cell.nFK);
     q.cell.e2 = two(k.cell.e2);
     q.cell.e3 = two(k.cell.e3);
+    q.cell.e3_lo = two(k.cell.e3_lo);
     q.cell.re = two(k.cell.re);
     q.cell.qu = two(k.cell.qu);
     q.cell.qF = two(k.cell.qF);
@@ -265,6 +266,7 @@ __device__ __forceinline__ Cell<L> field_cell(const Q& q, L e) {
     c.c1 = lmul(q_nhalf(q), c.nFK);
     c.e2 = lmul(ie, q.e2_ie);
     c.e3 = lmul(ie, q.e3_ie);
+    c.e3_lo = lfma(ie, q.e3_ie, lneg(c.e3));
     c.re = lmul(ie, q.rho0);
     c.qu = lmul(ie, q.qu_ie);
     c.qF = lmul(ie, q.qF_ie);
@@ -352,7 +354,7 @@ __device__ __forceinline__ CoreState<L> core_moments(const Q& q, const Cell<L>& 
     s.Fy = lfma(nd, s.uy, eGy);
     const L uF = lfma(s.ux, s.Fx, lmul(s.uy, s.Fy));
     L ep = lfma(c.e2, uF, lmul(c.e3, uu));
-    if constexpr (sizeof(R) == 4) ep = lfma(q.e1_lo, sf, ep);
+    if constexpr (sizeof(R) == 4) ep = lfma(q.e1_lo, sf, lfma(c.e3_lo, uu, ep));
     s.ep = lfma(q.e1, sf, ep);
     s.Px = lsub(Pxx, s.ep);
     s.Py = lsub(Pyy, s.ep);

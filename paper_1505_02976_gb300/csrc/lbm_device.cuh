@@ -71,7 +71,7 @@ struct Cell {
     V eg, eax, heax;   // e g beta, e a_x, e a_x / 2
     V c0, c0sq, c1;    // quadratic solve (Sec. 3.1)
     V nnuK, nFK;       // - e nu/K, - e F_e/sqrt(K)
-    V e2, e3;          // e p = e1 sum f + e2 u.F + e3 |u|^2
+    V e2, e3, e3_lo;   // e p = e1 sum f + e2 u.F + e3 |u|^2; e3_lo: what rounding e3 left
     V re;              // rho0 / e
     V qu, qF;          // of u u and u F in Q, S folded in: cu2 - a re, cuF + a re
     V cu2, cuF;        // the same with S apart: 4.5 itf rho0/e, 9 rho0 (1 - 1/2tau_f)/e
