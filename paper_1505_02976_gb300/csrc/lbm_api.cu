@@ -255,6 +255,9 @@ lbm_status lbm_create(const lbm_params* p, void* stream, void* workspace, size_t
     h->two_steps_ready = p->precision == LBM_F32 && !p->moment_state && lbm::two_steps_supported(h->k32);
     h->two_steps = h->two_steps_ready;
     h->msegments = 0;
+    h->mdefault = 1;
+    if (p->moment_state)
+        h->mdefault = p->precision == LBM_F64 ? lbm::moment_segments_default(h->k64) : lbm::moment_segments_default(h->k32);
     h->diag.T0 = d.T0;
     h->diag.inv_sigma = 1.0 / p->sigma;
     h->diag.Q = d.Q;
@@ -369,16 +372,18 @@ lbm_status lbm_step(lbm_handle* h, int64_t n) {
     if (h->timeout) return fail(h, LBM_ERR_TIMEOUT, "a bounded wait of the TMA step gave up");
     if (h->nonfinite) return fail(h, LBM_ERR_NONFINITE, "non-finite velocity or temperature");
     if (h->moments_kind()) {
+        const bool tiles = h->prm.precision == LBM_F32 && h->msegments == 0 && lbm::moment_tiles_preferred(h->k32, h->sms);
+        const int segments = h->msegments > 0 ? h->msegments : h->mdefault;
         for (int64_t i = 0; i < n; ++i) {
             const int src = h->mcur, dst = 1 - h->mcur;
             cudaError_t e = h->prm.precision == LBM_F64
                                 ? lbm::launch_step_m(h->k64, (const double*)h->mom(src), (double*)h->mom(dst),
-                                                     h->msources, h->msegments, h->stream)
-                            : h->msegments == 0 && lbm::moment_tiles_preferred(h->k32, h->sms)
+                                                     h->msources, segments, h->stream)
+                            : tiles
                                 ? lbm::launch_step_m_tiles(h->k32, (const float*)h->mom(src), (float*)h->mom(dst),
                                                            h->msources, h->sms, h->stream)
                                 : lbm::launch_step_m(h->k32, (const float*)h->mom(src), (float*)h->mom(dst),
-                                                     h->msources, h->msegments, h->stream);
+                                                     h->msources, segments, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "moment step kernel");
             h->mcur = dst;
             h->msources = true;

@@ -22,7 +22,7 @@ struct lbm_handle {
     // after set_fields), and whether the expansion in buf(0) is up to date
     int mcur;
     bool msources, pops_valid;
-    int msegments;  // row segments per band of the moment step (0: default)
+    int msegments, mdefault;  // row segments per band of the moment step (0: default), and the default of the bands' kernel
     // FP32 / FP16 walled lattices: the step with TMA-staged rows (tensor maps
     // of the two population buffers, whether they could be made, whether
     // the step uses them) and its rows per block segment

@@ -109,7 +109,7 @@ cudaError_t launch_nusselt_batch(const BatchCavity<R>* cav, int n, const S* src,
 // One step of the moment state (9 planes: p, u, S, T - T0, grad T) from src
 // to dst; sources = false when src is the state written by launch_init_m
 // (equilibria without force and source terms).  segments: row segments per
-// band (clamped so that each keeps >= 3 rows; 0: moment_segments_default).
+// band (clamped so that each keeps >= 3 rows).
 template <class R>
 cudaError_t launch_step_m(const KConst<R>& k, const R* src, R* dst, bool sources, int segments, cudaStream_t st);
 

@@ -332,7 +332,6 @@ int moment_segments_default(const KConst<R>& k) {
 
 template <class R>
 cudaError_t launch_step_m(const KConst<R>& k, const R* src, R* dst, bool sources, int segments, cudaStream_t st) {
-    if (segments == 0) segments = moment_segments_default(k);
     int nstrips = 0, nseg = 0;
     moment_shape(k, segments, &nstrips, &nseg);
     if (k.eps_field)
