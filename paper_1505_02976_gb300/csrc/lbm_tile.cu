@@ -65,11 +65,15 @@ constexpr int kTileSmallWaves = 3;             // in SMs: at most 3 x 152 tiles
 // x_f and x_ff of a tile's wall rows and their ring: three rows at least, which
 // an even split of eight or more rows into tiles of at most four has
 static_assert(kTileLarge.rows >= 4 && kTileSmall.rows >= 4, "tiles are at least three rows tall");
-constexpr int kTileMaxRows = kTileLarge.rows;
 constexpr int kTileMaxThreads = 32 * (kTileSmall.warps + kTileSmall.wall_warps);
 constexpr int kTileRowElems = NPLANES * kTileCols;
 
 __host__ __device__ constexpr size_t tile_smem(int rows) { return (size_t)(rows + 2) * kTileRowElems * sizeof(float); }
+// what a launch may ask for without the function's opt-in, beside the batch
+// kernel's constants (43 520 bytes and about 1.5 KB)
+static_assert(tile_smem(kTileLarge.rows) + sizeof(KConst<float>) + sizeof(PairConst) <= 48 * 1024 &&
+                  kTileSmall.rows <= kTileLarge.rows,
+              "a tile's shared rows fit 48 KB");
 
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 
@@ -508,26 +512,9 @@ static TileSplit tile_split(int size, int unit, int most) {
     return {n, u / n, u % n, unit, size};
 }
 
-// Dynamic shared memory beyond 48 KB needs the function's opt-in, once per
-// device.
-template <bool E, bool T>
-static cudaError_t allow_tile_smem() {
-    constexpr int kMaxDev = 64;
-    static bool done[kMaxDev] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < kMaxDev && done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(k_tile<E, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem(kTileMaxRows));
-    if (e == cudaSuccess && dev < kMaxDev) done[dev] = true;
-    return e;
-}
-
 template <bool E, bool T>
 static cudaError_t launch_tile(cudaLaunchConfig_t& cfg, const KConst<float>& k, const float* src, float* mid,
                                float* dst, const TileSplit& sx, const TileSplit& sy, int warps, bool early, uint32_t launch) {
-    cudaError_t e = allow_tile_smem<E, T>();
-    if (e != cudaSuccess) return e;
     const PairConst pc = make_pair_const(k, 1.0f);
     return cudaLaunchKernelEx(&cfg, k_tile<E, T>, k, pc, src, mid, dst, sx, sy, warps, early, launch);
 }
