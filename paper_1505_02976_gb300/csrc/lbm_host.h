@@ -179,7 +179,8 @@ inline Layout layout(const lbm_params* p) {
         L.mom_bytes = 0;
         L.off_mom[0] = L.off_mom[1] = 0;
     }
-    L.off_fields = take(4 * N * sizeof(double));
+    // four fields; a lattice of one node needs a fifth value for the stream function
+    L.off_fields = take((N == 1 ? 5 : 4 * N) * sizeof(double));
     L.off_snap = take(3 * N * sizeof(double));
     L.off_nu = take((size_t)(p->nx > p->ny ? p->nx : p->ny) * sizeof(double));
     L.off_partial = take((size_t)lbm::residual_blocks(p->nx, p->ny) * 4 * sizeof(double));

@@ -65,8 +65,8 @@ cudaError_t launch_totals(const KConst<R>& k, const S* src, double sT0, double* 
                           cudaStream_t st);
 
 // Stream function psi [ny][nx] from u_x [ny][nx] (psi = 0 along y = 0,
-// trapezoid rule up each column); range[0..1] = min, max of psi.  scratch: at
-// least 2 nx ny doubles (lattices of one node take two), apart from ux and psi.
+// trapezoid rule up each column); range[0..1] = min, max of psi.  scratch: 2 nx ny
+// doubles, but 3 for a lattice of one node, apart from ux and psi.
 cudaError_t launch_stream_function(const double* ux, int nx, int ny, double* psi, double* scratch, double* range,
                                    cudaStream_t st);
 
