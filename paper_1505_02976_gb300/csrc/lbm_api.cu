@@ -67,12 +67,13 @@ lbm_status copy_in(lbm_handle* h, double* dst, const double* src, int on_device)
     return LBM_OK;
 }
 
-// Device memory of the stream's own GPU that a kernel may access as doubles.
+// Memory of the workspace's own GPU that a kernel may access as doubles.  (The
+// GPU is known from the handle: asking the stream for it would end the stream's
+// capture into a graph.)
 bool own_device_memory(const lbm_handle* h, const void* p) {
     cudaPointerAttributes a;
-    int dev = -1;
     const bool ok = ((uintptr_t)p & 7) == 0 && cudaPointerGetAttributes(&a, p) == cudaSuccess &&
-                    a.type == cudaMemoryTypeDevice && cudaStreamGetDevice(h->stream, &dev) == cudaSuccess && a.device == dev;
+                    a.type == cudaMemoryTypeDevice && a.device == h->device;
     if (!ok) (void)cudaGetLastError();
     return ok;
 }
@@ -247,6 +248,10 @@ lbm_status lbm_create(const lbm_params* p, void* stream, void* workspace, size_t
         h->tma = h->tma_ready;
         h->tma_rows = lbm::tma_rows_default(h->k32);
     }
+    h->device = -1;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, h->ws) == cudaSuccess && at.type == cudaMemoryTypeDevice) h->device = at.device;
+    else (void)cudaGetLastError();
     h->sms = 1;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||

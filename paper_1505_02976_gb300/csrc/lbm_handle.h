@@ -29,6 +29,7 @@ struct lbm_handle {
     bool tma, tma_ready;
     CUtensorMap tmap[2];
     int tma_rows;
+    int device;  // that the workspace is on (-1: not plain device memory)
     int sms;
     bool two_steps, two_steps_ready;  // FP32 populations: pairs of steps go through launch_two_steps, and whether they can
     bool nonfinite, timeout;
