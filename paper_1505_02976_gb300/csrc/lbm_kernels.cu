@@ -9,6 +9,8 @@
 // (lbm_step_tma.cu) unless the global-load kernel is selected.
 #include <math.h>
 
+#include <atomic>
+
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -99,12 +101,12 @@ __global__ void k_init(const __grid_constant__ KConst<R> k, S* __restrict__ dst,
 // Multiprocessors of the current device (asked once per device).
 static int device_sms() {
     constexpr int kMaxDev = 64;
-    static int known[kMaxDev] = {};
+    static std::atomic<int> known[kMaxDev];  // 0: not asked yet (any thread may ask)
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (dev < kMaxDev && known[dev] > 0) return known[dev];
+    if (dev < kMaxDev && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
-    if (dev < kMaxDev) known[dev] = sms;
+    if (dev < kMaxDev) known[dev].store(sms, std::memory_order_relaxed);
     return sms;
 }
 
