@@ -134,23 +134,20 @@ lbm_status lbm_set_moment_segments(lbm_handle* h, int32_t segments);
 
 /* Step kernel of a population handle (no counterpart in the paper; a
  * launch choice).  FP32 lattices of at least 8 x 8 nodes (any sides) take
- * their steps in pairs by default, two per launch, each node computed as in
- * the one-step kernels; the last of an odd number of steps, and smaller
- * lattices, take a one-step kernel.  FP32 and FP16 lattices walled on all four sides default
- * to staged rows: each block loads the 17 planes its rows pull from into
- * shared memory with tensor copies and waits on them with bounded waits.
+ * their steps in pairs by default, two per launch; the last of an odd number
+ * of steps, and smaller lattices, take a one-step kernel.  There FP32 lattices
+ * walled on all four sides, and FP16 ones at every step, default to staged
+ * rows: each block loads the 17 planes its rows pull from into shared memory
+ * with tensor copies and waits on them with bounded waits.
  * staged = 0 selects the kernel in which every thread loads its own 17
  * values from global memory, one step per launch; staged = 1 restores the default
  * (LBM_ERR_ARG where no rows can be staged: FP64, a periodic side, the moment
  * state, a lattice under 4 x 4, or a CUDA driver without tensor-map encoding;
  * an FP32 lattice that takes its steps in pairs returns to that from an
  * earlier staged = 0 all the same).
- * Both kernels run the same per-node arithmetic (results agree to rounding;
- * bit for bit in FP32 at tau_f = tau_T = 1).  In FP16 at tau_f = tau_T = 1
- * the staged kernel computes pairs of interior nodes with packed FP32
- * instructions, whose fused multiply-adds can round differently: its stored
- * values then agree with the other kernel's to within one FP16 rounding
- * step plus FP32 rounding.  lbm_step_staged returns 1 when the next step
+ * All of them run the same operations on every node, wall nodes included, so
+ * that the state after n steps does not depend on the choice, nor on how the
+ * n steps are cut into calls.  lbm_step_staged returns 1 when a single step
  * uses staged rows, else 0. */
 lbm_status lbm_set_step_staging(lbm_handle* h, int32_t staged);
 int32_t lbm_step_staged(const lbm_handle* h);
@@ -219,10 +216,10 @@ lbm_status lbm_stream_function(lbm_handle* h, double* psi, int on_device, double
 lbm_status lbm_set_force_profile(lbm_handle* h, const double* ay);
 
 /* Advance n >= 0 time steps (stream, rebuild walls, collide; one kernel
- * launch per step, or per two steps of an FP32 lattice).  Asynchronous on the handle's stream.  Returns
- * LBM_ERR_NONFINITE or LBM_ERR_TIMEOUT if an earlier synchronising call saw
- * the corresponding flag.  FP32 lattices walled on all four sides stage the
- * pulled rows in shared memory with tensor copies and bounded waits. */
+ * launch per step, or per two steps of an FP32 lattice).  Asynchronous on the
+ * handle's stream.  Returns LBM_ERR_NONFINITE or LBM_ERR_TIMEOUT if an earlier
+ * synchronising call saw the corresponding flag.  Which kernel takes a step:
+ * lbm_set_step_staging. */
 lbm_status lbm_step(lbm_handle* h, int64_t n);
 
 /* Wait for the handle's stream; returns LBM_ERR_TIMEOUT if a bounded
@@ -406,15 +403,15 @@ lbm_status lbm_batch_set_launch(lbm_batch* b, int32_t tile_x, int32_t grid);
 
 /* Step kernel of a batch (no counterpart in the paper; a launch choice).
  * A batch of FP32 cavities that are all walled on all four sides (each at
- * least 4 x 4) defaults to staged rows: one block per band of 128 columns x
- * 4 rows of one cavity loads the planes its rows pull from with tensor
- * copies (the maps of every cavity live in the workspace) and waits on them
- * with bounded waits, in every mode (per-case mode launches the single-
- * lattice staged kernel per cavity).  staged = 0 selects the global-load
+ * least 4 x 4) defaults to staged rows: in the fused and graph modes two steps
+ * per launch over tiles of all cavities (each at least 8 x 8), and otherwise
+ * one block per band of 128 columns x 4 rows of one cavity loads the planes
+ * its rows pull from with tensor copies (the maps of every cavity live in the
+ * workspace) and waits on them with bounded waits (per-case mode launches the
+ * single-lattice staged kernel per cavity).  staged = 0 selects the global-load
  * kernel and its launch shape; staged = 1 restores staging (LBM_ERR_ARG
- * where it is unavailable).  Both run the same per-node arithmetic (bit for
- * bit at tau_f = tau_T = 1).  lbm_batch_staged returns 1 when the next
- * step uses staged rows, else 0. */
+ * where it is unavailable).  All run the same operations on every node (the
+ * same bits).  lbm_batch_staged returns 1 when steps use staged rows, else 0. */
 lbm_status lbm_batch_set_staging(lbm_batch* b, int32_t staged);
 int32_t lbm_batch_staged(const lbm_batch* b);
 

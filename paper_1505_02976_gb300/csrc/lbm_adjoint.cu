@@ -15,7 +15,8 @@
 // is then a store of each adjoint at the place it was pulled from: every
 // place is pulled by at most one interior node, so no two threads write the
 // same word and the result does not depend on their order.
-// States are recomputed from checkpoints kept every ceil(sqrt(n)) steps.
+// A run whose states fit 256 MB keeps them all; a longer one keeps checkpoints
+// every ceil(sqrt(n)) steps and recomputes the states between them.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -366,8 +367,8 @@ struct Interior {
 // latency of its chain (loads, ~600 dependent operations, stores).  Before, 9
 // to 11 forward-mode passes a node in a thread each, then a combining and a
 // gathering launch: whole calls with 256 steps at 256^2 FP32 took 38.0 ms
-// against 7.0 ms, with 100 steps at 65 x 49 FP64 45.7 against 6.3 ms (forward and
-// recomputed steps included; 7.5 and 8.4 ms with the wall nodes' chains in the
+// against 7.0 ms, with 100 steps at 65 x 49 FP64 45.7 against 6.3 ms (lattice,
+// uploads, forward and recomputed steps included; 7.5 and 8.4 ms with the wall nodes' chains in the
 // threads of the nodes they hang on).
 constexpr int kAdjNodes = 64, kAdjRing = 32;
 template <class R> struct AdjLaunch { static constexpr int blocks = 8; };
@@ -638,8 +639,8 @@ lbm_status run_adjoint(lbm_handle* h, const lbm::KConst<R>& k, int64_t n, int64_
     const size_t N = (size_t)p.nx * p.ny;
     const size_t sb = h->L.buf_bytes;  // one state
     // few and small states are all kept as the forward pass computes them, and
-    // nothing is recomputed (65 x 49 FP64, 100 steps: 4.7 ms a call
-    // against 5.7 with checkpoints); where the memory for that is not to be had,
+    // nothing is recomputed (65 x 49 FP64, 100 steps: 4.8 ms in this call
+    // against 5.7 with checkpoints; the same in FP32 1.4 and 1.7); where the memory for that is not to be had,
     // checkpoints are
     bool keep = seg_len == 0 && (double)sb * (double)n <= (double)kKeepBytes;
     const int64_t seg = seg_len > 0 ? seg_len : (int64_t)ceil(sqrt((double)n));

@@ -12,7 +12,7 @@
 //     (Pi, u u, u F), so its coefficients fold into those of Q;
 //   * likewise the thermal odd part is c . V, its even part B0 + Kc (c.u)^2;
 //   * 1/a and b/(a - b |u|^2) of the gradient solve share one reciprocal.
-// FP32: 162 operations a node plus two square roots and two reciprocals; the
+// FP32: 163 operations a node plus two square roots and two reciprocals; the
 // direction-by-direction form took 215 (FP64 instructions of the whole step,
 // square roots and reciprocals included: see k_step in lbm_kernels.cu).
 //
@@ -87,7 +87,7 @@ __device__ __forceinline__ float lrcp(float a) {
 // (g + g d ~ sqrt(a), h + h d ~ 1/(2 sqrt(a))), then g + h (a - g^2).
 // Reciprocals here are of positive normal values.  Both are within 0.501 units in
 // the last place, as the language's are, over 2^-900 .. 2^900.  700 x 517 with 50
-// steps: 6.81 ms, about 7.2 with the language's; one iteration of third order instead
+// steps: 6.81 ms, about 7.1 with the language's; one iteration of third order instead
 // of the two takes four FP64 instructions a node less (6.69 ms) and leaves 0.76
 // and 0.51 units.
 __device__ __forceinline__ double lrcp(double a) {

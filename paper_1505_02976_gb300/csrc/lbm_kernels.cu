@@ -4,9 +4,10 @@
 // per-node arithmetic of the step in registers, and one write of the 17
 // post-collision planes to the pong buffer.  Wall nodes take the NEES rebuild
 // inside the same launch (an out-of-line path that pulls the populations of
-// the wall node's fluid neighbour x_f instead of its own).  FP32 and FP16
-// lattices walled on all four sides run the kernel with TMA-staged rows
-// (lbm_step_tma.cu) unless the global-load kernel is selected.
+// the wall node's fluid neighbour x_f instead of its own).  It steps FP64
+// lattices, FP16 lattices with a periodic side, and what FP32 lattices do not
+// take in pairs (lbm_tile.cu) where rows cannot be staged (lbm_step_tma.cu); and
+// FP32 and FP16 lattices on which it is selected (lbm_set_step_staging).
 #include <math.h>
 
 #include <atomic>
@@ -21,11 +22,12 @@ namespace lbm {
 // warp with both would run them one after the other, and the wall nodes'
 // longer chain starts first.  TAU1: tau_f = tau_T = 1 (the paper's default,
 // Sec. 4), where the (1 - 1/tau) terms vanish.
-// FP64 is bound by its pipe (two lanes a cycle and SM): 700 x 517 takes 126 us a
-// step, 0.95 of the measured FP64 rate for its 182 FP64 instructions a warp and
-// node (165 us with the wall nodes inside the rows' warps, 267 with the
-// direction-by-direction arithmetic too); blocks of one warp end most evenly
-// (130 us in blocks of four).  A lattice that leaves SMs empty is bound by one
+// FP64 is bound by its pipe (two lanes a cycle and SM): 700 x 517 takes 128 us a
+// step, 0.98 of the measured FP64 rate for its 183 FP64 instructions a node.
+// Before the root and the reciprocal took their second iteration (2 % of every
+// FP64 figure here): 126 us, 165 with the wall nodes inside the rows' warps, 267
+// with the direction-by-direction arithmetic too; blocks of one warp end most
+// evenly (130 us in blocks of four).  A lattice that leaves SMs empty is bound by one
 // warp's chain, and blocks of one warp put every warp on an SM of its own: 32^2
 // 8.6 us a step (10.0 in blocks of four; 17.3 with the wall nodes inside, 38
 // before), 7.1 with SPLIT (below).

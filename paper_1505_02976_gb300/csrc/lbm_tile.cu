@@ -18,12 +18,13 @@
 // global memory are aligned 64-bit ones.  Step 1 writes only to shared memory
 // and step 2 only reads there, so one block barrier separates them.
 //
-// Bound: neither pipe alone.  2048^2: 285 + 236 MB of DRAM traffic and 67 M
-// warp instructions a launch, issue 48 % active with 18 warps an SM, DRAM at
-// 4.5 TB/s; 58.4 us a step in the timed loop (72 GLUPS) against 86 us (48.7) of
-// the one-step staged kernel, which is at 0.98 of measured HBM; 4096^2 219 us
-// (76); 1024 x 513 periodic 9.0 us against 12.7 of the global-load kernel;
-// 1000 x 777 with a porosity field off tau = 1 14.6 us against 24.
+// Bound: neither pipe alone.  2048^2: 285 + 236 MB of DRAM traffic and 69 M
+// warp instructions a launch, issue 49 % active with 18 warps an SM, DRAM at
+// 4.4 TB/s; 58.8 us a step in the timed loop (71 GLUPS) against 85 us (49) of
+// the one-step kernels, which are at 0.98 of measured HBM; 4096^2 222 us (76)
+// against 342; 1024 x 513 periodic 9.0 us against 9.3 of the global-load kernel;
+// 1000 x 777 with a porosity field off tau = 1 16.6 us against 17.2 (12.7 and
+// 24 before the node update was rearranged).
 // Copying the pulls into the shared rows asynchronously (cp.async, every row of
 // a warp in flight at once) took as long at 2048^2 and 3 to 8 % longer below
 // 1024^2 (more instructions for the same bytes).
@@ -57,7 +58,7 @@ struct TileShape {
 constexpr TileShape kTileLarge = {8, 5, 0};
 // Lattices that do not fill the GPU: the step lasts as long as one block, so
 // every warp has one row, and the wall nodes' long chain runs beside the rows
-// (201^2: 2.9 us a step against 5.1 with the large shape, 3.6 without the wall
+// (201^2: 2.8 us a step against 5.1 with the large shape, 3.6 without the wall
 // warps; 32^2: 2.5 against 3.9).  The line lies at one and a half waves of its
 // blocks: 384^2 (448 tiles) 5.0 against 5.7 us, 512^2 (774 tiles) 7.2 against 5.8.
 constexpr TileShape kTileSmall = {6, 8, 2};

@@ -3,7 +3,7 @@ steps are cut into calls: pairs of steps, single steps and the kernels that take
 them (two steps from shared memory, staged rows, global loads) run the same
 operations, at the walls too.  Sizes at the edges of a tile (62 columns, 6 or
 8 rows) and of both launch shapes; a run resumed from a checkpoint after an odd
-number of steps; batches."""
+number of steps; batches in every mode; and FP16 storage with either kernel."""
 import numpy as np
 import pytest
 
@@ -69,8 +69,10 @@ def test_a_resumed_run(tmp_path, sides):
 def test_batches():
     probs = [_problem(nx, ny, s, False) for nx, ny, s in ((20, 31, "cavity"), (130, 50, "mixed"), (64, 64, "cavity"))]
     runs = []
-    for mode, calls in (("fused", [9]), ("fused", [1] * 9), ("per_case", [9])):
+    for mode, calls, staged in (("fused", [9], True), ("fused", [1] * 9, True), ("per_case", [9], True),
+                                ("persistent", [4, 5], True), ("fused", [9], False)):
         b = lbm.Batch([p for p, _, _ in probs], "f32")
+        b.staged = staged
         for c, (_, fields, _) in enumerate(probs):
             b.set_fields(c, *fields)
         for n in calls:
@@ -80,3 +82,22 @@ def test_batches():
     for other in runs[1:]:
         for a, m in zip(runs[0], other):
             assert all(np.array_equal(a[k], m[k]) for k in ("p", "ux", "uy", "T"))
+
+
+@pytest.mark.parametrize("tau", [dict(), TAU])
+@pytest.mark.parametrize("nx,ny,field", [(300, 50, False), (129, 131, True), (517, 9, False), (4, 4, False)])
+def test_fp16_kernels(nx, ny, field, tau):
+    """FP16 storage: node pairs from staged rows and single nodes from global memory."""
+    p = W.cavity(nx, 1e5, 1e-3, 0.5, ny=ny, **tau, **SIDES["mixed"])
+    eps = np.random.Generator(np.random.PCG64(nx)).uniform(0.3, 0.9, (ny, nx)) if field else None
+    fields = W.random_fields(p, seed=nx + ny, amp_u=2e-3, amp_T=0.3)
+    states = []
+    for staged in (True, False):
+        g = lbm.Lattice(p, "f16")
+        g.set_fields(*fields, eps_field=eps)
+        g.staged = staged
+        g.step(30)
+        g.sync()
+        f, h = g.get_state()
+        states.append(np.concatenate([f[1:], h]))
+    assert np.array_equal(states[0], states[1])
