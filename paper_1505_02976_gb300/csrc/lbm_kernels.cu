@@ -125,13 +125,21 @@ cudaError_t launch_step(const KConst<R>& k, const S* src, S* dst, uint32_t step,
     cfg.gridDim = dim3((unsigned)(split ? 2 * shares : shares));
     cfg.blockDim = dim3((unsigned)block);
     // The blocks of a dependent launch fill SM after SM up to the kernel's
-    // occupancy (12 blocks of one warp), which leaves SMs idle where the grid
-    // is smaller: unused shared memory keeps each SM to its share of the
-    // blocks.  FP64 130^2 13.2 -> 12.0, 201^2 21.6 -> 18.9 us a step; with
-    // fewer than four blocks an SM the launches overlap less and it costs 0.5 us,
-    // and four would need more than the 48 KB a launch may ask for unasked.
-    const long long per = (cfg.gridDim.x + device_sms() - 1) / device_sms();
-    cfg.dynamicSmemBytes = sizeof(R) == 8 && per >= 5 && per < 12 ? (size_t)(227 / per - 1) * 1024 : 0;
+    // occupancy (12 or more blocks of one warp), which leaves SMs idle where the
+    // grid is smaller, and in the last round where that is less than half full:
+    // unused shared memory keeps each SM to its share of the blocks, in rounds of
+    // one size.  FP64 130^2 13.2 -> 12.0, 201^2 21.6 -> 18.9 us a step in one round
+    // (with fewer than four blocks an SM the launches overlap less and it costs
+    // 0.5 us, and four would need more than the 48 KB a launch may ask for
+    // unasked); 243 x 240 29.0 -> 25.9, 261 x 258 32.5 -> 29.4, 279 x 276 34.9 -> 31.0 in
+    // two, 351 x 348 48.4 -> 46.4 in three.  Where the last round is fuller, or
+    // holds an eighth of the SMs' number or less, it costs up to 7 % (333 x 330
+    // periodic: 41.9 -> 44.7); beyond three rounds it changes nothing.
+    const long long sms = device_sms(), per = (cfg.gridDim.x + sms - 1) / sms;
+    const long long rounds = (per + 11) / 12, last = per - 12 * (rounds - 1), over = cfg.gridDim.x - 12 * (rounds - 1) * sms;
+    const bool spread = sizeof(R) == 8 && per >= 5 && (rounds == 1 ? last < 12 : rounds <= 3 && last <= 6 && over > sms / 8);
+    const long long resident = (per + rounds - 1) / rounds;
+    cfg.dynamicSmemBytes = spread ? (size_t)(227 / resident - 1) * 1024 : 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
